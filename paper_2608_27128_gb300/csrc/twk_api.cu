@@ -232,12 +232,12 @@ twinkv_status run_audit(const DeviceInfo& dev, const twinkv_shape& s, const uint
     const int64_t U = static_cast<int64_t>(s.L) * s.H;
     twinkv_status r = make_map(&tmA, keys16, U * s.N, s.d, kBM);
     if (r != TWINKV_OK) return r;
-    r = make_map(&tmB, bkeys, b_rows, s.d, kBN);
+    r = make_map(&tmB, bkeys, b_rows, s.d, kBN / 2);
     if (r != TWINKV_OK) return r;
-    const int64_t items = U * a.RB;
-    const int grid = static_cast<int>(items < dev.sms ? items : dev.sms);
+    const int64_t items = U * a.RB;   // one CTA pair each, on one SM per CTA
+    const int pairs = static_cast<int>(std::min<int64_t>(items, dev.sms / 2));
     ProfScope p(TWINKV_KERNEL_AUDIT, st);
-    return cuda_status(launch_audit(s.d, mode, tmA, tmB, a, grid, st));
+    return cuda_status(launch_audit(s.d, mode, tmA, tmB, a, 2 * pairs, st));
 }
 
 twinkv_status params_ok(const twinkv_params& p, float threshold)
@@ -600,7 +600,7 @@ twinkv_status redundancy_impl(const void* keys, twinkv_shape s, int32_t window, 
     a.U = U;
     a.N = s.N;
     a.NP = static_cast<int>(NP);
-    a.RB = (s.N + kBM - 1) / kBM;
+    a.RB = (s.N + kPM - 1) / kPM;
     a.window = window < s.N ? window : s.N;
     a.repair_mode = 0;
     a.need_all = 0;
@@ -679,7 +679,7 @@ twinkv_status twinkv_policy(const void* keys, twinkv_shape s, const int32_t* bud
     a.U = U;
     a.N = s.N;
     a.NP = static_cast<int>(NP);
-    a.RB = (s.N + kBM - 1) / kBM;
+    a.RB = (s.N + kPM - 1) / kPM;
     a.window = p.window < s.N ? p.window : s.N;
     a.repair_mode = 0;
     a.need_all = 0;
@@ -759,7 +759,7 @@ twinkv_status main_stages(const DeviceInfo* dev, const uint16_t* k16, const twin
     a.U = U;
     a.N = s.N;
     a.NP = static_cast<int>(NP);
-    a.RB = (s.N + kBM - 1) / kBM;
+    a.RB = (s.N + kPM - 1) / kPM;
     a.window = p.window < s.N ? p.window : s.N;
     a.repair_mode = 1;
     a.need_all = need_all ? 1 : 0;

@@ -6,14 +6,26 @@
 //   Sec. 3.4 Eq. 4   b_i(S0) = max over retained j, -1 if none; and its argmax
 //   (b_i(all))       the same over every j
 //
-// Design (one persistent CTA per SM, 64 + 32 * kEpiWarps threads, warp-specialised):
-//   warp 0      TMA producer: the 128-row A block of keys i (once per work item), then
-//               per 256-column tile the B tile of keys j (in 64-wide K chunks) and the
-//               tile's column metadata (1/||k_j|| and original positions).
-//   warp 1      owns TMEM (512 columns = two 128x256 fp32 accumulators) and issues
-//               tcgen05.mma (M=128, N=256, K=16, bf16 -> fp32) from one thread.
+// Design (persistent pairs of CTAs, one CTA per SM, 64 + 32 * kEpiWarps threads each,
+// warp-specialised).  A pair shares each 256-row work item: CTA r holds rows
+// [128 r, 128 r + 128) of A and of each B tile, and the accumulators of its own rows.
+//   warp 0      TMA producer: its CTA's 128 rows of the keys i (once per work item), then
+//               per 256-column tile its half of the keys j (in 64-wide K chunks) and the
+//               whole tile's column metadata (1/||k_j|| and original positions).  Key
+//               copies of both CTAs complete on the even CTA's barriers.
+//   warp 1      owns TMEM (512 columns = two 128x256 fp32 accumulators); in the even CTA
+//               one thread issues tcgen05.mma.cta_group::2 (M=256, N=256, K=16,
+//               bf16 -> fp32) for both and commits to both CTAs' barriers.
 //   warps 2..   epilogue: four warps per column group g (kGW columns of each tile); a
 //               thread owns one row (TMEM lane) and keeps its running maximum.
+// Why pairs: with one CTA per 128 rows, each tile moves 64 KB of B into shared memory
+// and 96 KB of operands out of it (d = 128), beside the epilogue's broadcast loads; a
+// pair moves 32 KB in and 64 KB out per SM.  Whole calls, one CTA -> pair: Qwen3-4B
+// repair 36x8x16384x128 17.29 -> 16.71 ms, Llama-3.2-1B repair 16x8x8192x64
+// 1032 -> 1010 us, policy 36x8x8192x128 3965 -> 3838 us; the same outputs bit for bit.
+// The release of an accumulator to the even CTA is a remote arrival without a
+// cluster-scope release (only TMEM reads precede it): with one, each cost the epilogue
+// warp several hundred ns per tile (24.3 ms for the first of these calls).
 // Keys enter the tensor cores un-normalised (bf16 products are exact in fp32);
 // 1/||k_j|| (times a power of two per unit) is applied per element in fp32.
 // 1/||k_i|| > 0 does not change the argmax over j, so it is never applied: this kernel
@@ -65,8 +77,8 @@ struct AuditCfg {
     static constexpr int KC = D / 64;                 // 128-byte K chunks per key row
     static constexpr int A_CHUNK = kBM * 128;         // 16 KB
     static constexpr int A_BYTES = KC * A_CHUNK;
-    static constexpr int B_STAGE = kBN * 128;         // 32 KB: one K chunk of a tile
-    static constexpr int STAGES = (D == 128) ? 4 : 5;
+    static constexpr int B_STAGE = kBN / 2 * 128;     // 16 KB: this CTA's half of a K chunk
+    static constexpr int STAGES = 8;
     static constexpr int MSLOTS = 8;
     static constexpr int META = kBN * 8;              // rinv[256] + pos[256]
     static constexpr int OFF_A = 0;
@@ -361,7 +373,7 @@ template <bool kSym>
 __device__ __forceinline__ Tiles unit_tiles(const AuditArgs& a, int u, int rb)
 {
     if (kSym) {
-        const int t0 = rb >> 1;
+        const int t0 = rb;
         return {(a.N + kBN - 1) / kBN - t0, 0, t0};
     }
     if (!a.repair_mode) return {(a.N + kBN - 1) / kBN, 0, 0};
@@ -406,10 +418,10 @@ __device__ __forceinline__ int last_parity(long long total, int n, int s)
     return static_cast<int>((k / n) & 1);
 }
 
-// Registers are per sub-partition (16384 each): with W warps a sub-partition holds
+// kCount: Eq. 2 counts; kSym: upper-triangle tiles only.  Registers are per sub-partition (16384 each): with W warps a sub-partition holds
 // ceil(W / 4) of them, which bounds the registers per thread.
 template <int D, bool kCount, bool kSym>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     audit_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ AuditArgs a)
 {
@@ -445,7 +457,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_init(&a_full[i], 1);
             mbar_init(&a_empty[i], 1);
             mbar_init(&t_full[i], 1);
-            mbar_init(&t_empty[i], kEpiWarps);
+            mbar_init(&t_empty[i], 2 * kEpiWarps);   // both CTAs' epilogues
             mbar_init(&x_full[i], (kGroups - 1) * kBM);
             mbar_init(&x_empty[i], kBM);
         }
@@ -467,9 +479,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         prefetch_tensormap(&tmA);
         prefetch_tensormap(&tmB);
     }
-    if (warp == 1) tmem_alloc(tmem_slot, kTmemCols);
+    if (warp == 1) tmem_alloc<2>(tmem_slot, kTmemCols);
     tc_fence_before();
-    __syncthreads();
+    cluster_barrier();   // barriers of both CTAs initialised, tensor memory allocated
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
@@ -479,12 +491,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     wc.err = a.err;
     wc.where = 0;
     const int n_items = a.U * a.RB;
+    const int pair = static_cast<int>(blockIdx.x >> 1);
+    const int n_pairs = static_cast<int>(gridDim.x >> 1);
+    const uint32_t rank = cluster_rank();
+    const bool leader = rank == 0;
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
         long long n_a = 0, n_b = 0, n_m = 0;
         bool ok = true;
-        for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+        for (int item = pair; item < n_items && ok; item += n_pairs) {
             const int u = item / a.RB;
             const int rb = item - u * a.RB;
             const Tiles ut = unit_tiles<kSym>(a, u, rb);
@@ -492,12 +508,13 @@ __global__ void __launch_bounds__(kThreads, 1)
             ok = lane0_wait(&a_empty[ab], static_cast<uint32_t>(((n_a >> 1) & 1) ^ 1), wc, 1);
             if (!ok) break;
             if (lane == 0) {
-                mbar_arrive_expect_tx(&a_full[ab], C::A_BYTES);
-                const int y = u * a.N + rb * kBM;
+                if (leader) mbar_arrive_expect_tx(&a_full[ab], 2 * C::A_BYTES);
+                const uint32_t full = cluster_addr(&a_full[ab], 0);
+                const int y = u * a.N + rb * kPM + static_cast<int>(rank) * kBM;
 #pragma unroll
                 for (int kc = 0; kc < C::KC; ++kc)
-                    tma_load_2d(sA + ab * C::A_BYTES + kc * C::A_CHUNK, &tmA, &a_full[ab],
-                                kc * 64, y);
+                    tma_load_2d_pair(sA + ab * C::A_BYTES + kc * C::A_CHUNK, &tmA, full, kc * 64,
+                                     y);
             }
             __syncwarp();
             ++n_a;
@@ -517,28 +534,42 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
                 __syncwarp();
                 ++n_m;
-                const int yb = static_cast<int>(u * a.b_rows_per_unit + col0);
+                const int yb = static_cast<int>(u * a.b_rows_per_unit + col0) +
+                               static_cast<int>(rank) * (kBN / 2);
                 for (int kc = 0; kc < C::KC; ++kc) {
                     const int s = static_cast<int>(n_b % C::STAGES);
                     ok = lane0_wait(&b_empty[s],
                                     static_cast<uint32_t>(((n_b / C::STAGES) & 1) ^ 1), wc, 3);
                     if (!ok) break;
                     if (lane == 0) {
-                        mbar_arrive_expect_tx(&b_full[s], C::B_STAGE);
-                        tma_load_2d(sB + s * C::B_STAGE, &tmB, &b_full[s], kc * 64, yb);
+                        if (leader) mbar_arrive_expect_tx(&b_full[s], 2 * C::B_STAGE);
+                        tma_load_2d_pair(sB + s * C::B_STAGE, &tmB, cluster_addr(&b_full[s], 0),
+                                         kc * 64, yb);
                     }
                     __syncwarp();
                     ++n_b;
                 }
             }
         }
+        // The even CTA's commits release the rings in both CTAs: each CTA stays until the
+        // last release of every slot has reached it.
+        for (int s = 0; ok && s < 2; ++s) {
+            const int p = last_parity(n_a, 2, s);
+            if (p >= 0) ok = lane0_wait(&a_empty[s], static_cast<uint32_t>(p), wc, 12);
+        }
+        for (int s = 0; ok && s < C::STAGES; ++s) {
+            const int p = last_parity(n_b, C::STAGES, s);
+            if (p >= 0) ok = lane0_wait(&b_empty[s], static_cast<uint32_t>(p), wc, 13);
+        }
         if (!ok && lane == 0) {
-            // Let every copy this warp started land before the block exits.
-            for (int s = 0; s < 2; ++s) {
+            // Let every copy this warp started land before the block exits.  A and B copies
+            // of both CTAs complete on the even CTA's barriers; the odd CTA leaves its own
+            // to that wait (the cluster barrier at the end follows it).
+            for (int s = 0; leader && s < 2; ++s) {
                 const int p = last_parity(n_a, 2, s);
                 if (p >= 0) drain_wait(&a_full[s], p, a.timeout_ns);
             }
-            for (int s = 0; s < C::STAGES; ++s) {
+            for (int s = 0; leader && s < C::STAGES; ++s) {
                 const int p = last_parity(n_b, C::STAGES, s);
                 if (p >= 0) drain_wait(&b_full[s], p, a.timeout_ns);
             }
@@ -548,12 +579,14 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
         }
         __syncwarp();
+    } else if (warp == 1 && !leader) {
+        // the even CTA's MMA warp issues for both
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        constexpr uint32_t idesc = umma_idesc_bf16_f32(kBM, kBN);
+        constexpr uint32_t idesc = umma_idesc_bf16_f32(kPM, kBN);
         long long n_a = 0, n_b = 0, n_t = 0;
         bool ok = true;
-        for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+        for (int item = pair; item < n_items && ok; item += n_pairs) {
             const int u = item / a.RB;
             const Tiles ut = unit_tiles<kSym>(a, u, item - u * a.RB);
             const int ab = static_cast<int>(n_a & 1);
@@ -580,26 +613,26 @@ __global__ void __launch_bounds__(kThreads, 1)
                         const uint64_t bd = umma_desc_sw128(smem_u32(sB + s * C::B_STAGE));
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
-                            umma_bf16(d_tmem, ad + 2u * k, bd + 2u * k, idesc,
-                                      (kc | k) != 0 ? 1u : 0u);
-                        umma_commit(&b_empty[s]);
+                            umma_bf16_pair(d_tmem, ad + 2u * k, bd + 2u * k, idesc,
+                                           (kc | k) != 0 ? 1u : 0u);
+                        umma_commit_pair(&b_empty[s]);
                     }
                     __syncwarp();
                     ++n_b;
                 }
                 if (!ok) break;
-                if (lane == 0) umma_commit(&t_full[acc]);
+                if (lane == 0) umma_commit_pair(&t_full[acc]);
                 __syncwarp();
                 ++n_t;
             }
             if (!ok) break;
-            if (lane == 0) umma_commit(&a_empty[ab]);
+            if (lane == 0) umma_commit_pair(&a_empty[ab]);
             __syncwarp();
             ++n_a;
         }
         // Every MMA this thread issued completes before TMEM is released.
         if (lane == 0) {
-            umma_commit(drain);
+            umma_commit_own(drain);
             drain_wait(drain, 0, a.timeout_ns);
         }
         __syncwarp();
@@ -618,12 +651,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         uint32_t n_x = 0;
         uint32_t n_c = 0;   // symmetric mode: tiles whose column maxima were merged
         bool ok = true;
-        for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+        for (int item = pair; item < n_items && ok; item += n_pairs) {
             const int u = item / a.RB;
             const int rb = item - u * a.RB;
             const Tiles ut = unit_tiles<kSym>(a, u, rb);
             const int nt = ut.tr + ut.te;
-            const int r0 = rb * kBM;
+            const int r0 = rb * kPM + static_cast<int>(rank) * kBM;
             const int row = r0 + row_local;
             // symmetric mode: the row's own column scale (the value of row j's candidate
             // i is x_ij s_i), and whether this row block runs past the end of the unit
@@ -678,7 +711,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 // so it can compute the next-but-one tile while this one is reduced.
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&t_empty[acc]);
+                if (lane == 0) mbar_arrive_cluster(cluster_addr(&t_empty[acc], 0));
                 if (kSym) {
                     // row maxima (the eager fold: the column pass already costs more than
                     // the vote saves) and each chunk's column maxima over this warp's 32
@@ -831,10 +864,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     }
 
+    // Neither CTA frees its tensor memory or exits while the pair's MMAs, commits or
+    // arrivals can still reach it.
     tc_fence_before();
-    __syncthreads();
+    cluster_barrier();
     tc_fence_after();
-    if (warp == 1) tmem_dealloc(tmem, kTmemCols);
+    if (warp == 1) tmem_dealloc<2>(tmem, kTmemCols);
 }
 
 }  // namespace
@@ -904,7 +939,7 @@ __global__ void wait_probe_kernel(int* err, unsigned long long timeout_ns)
         abort_flag = 0;
         fence_mbarrier_init();
     }
-    if (threadIdx.x < 32) tmem_alloc(&slot, 32);
+    if (threadIdx.x < 32) tmem_alloc<1>(&slot, 32);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -918,7 +953,7 @@ __global__ void wait_probe_kernel(int* err, unsigned long long timeout_ns)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (threadIdx.x < 32) tmem_dealloc(slot, 32);
+    if (threadIdx.x < 32) tmem_dealloc<1>(slot, 32);
 }
 }  // namespace
 

@@ -8,7 +8,8 @@
 
 namespace twk {
 
-constexpr int kBM = 128;       // rows (keys i) per work item: the UMMA M
+constexpr int kBM = 128;       // rows (keys i) per CTA of a pair
+constexpr int kPM = 2 * kBM;   // rows per work item, a CTA pair's: the UMMA M
 constexpr int kBN = 256;       // columns (keys j) per tile: the UMMA N
 
 // Bounded waits.  A wait on work that another role of the block has to do gives up
@@ -25,7 +26,7 @@ constexpr unsigned long long kDrainFloorNs = 200000000ull;     // 200 ms
 inline int64_t column_stride(int N) { return ((int64_t)(N + kBN - 1) / kBN) * kBN + kBN; }
 
 struct AuditArgs {
-    int U, N, NP, RB;           // units, keys per unit, column stride, row blocks per unit
+    int U, N, NP, RB;           // units, keys per unit, column stride, kPM-row blocks per unit
     int window;                 // w, clamped to [0, N]
     int repair_mode;            // 0: one segment over the keys as given; 1: retained-first
     int need_all;               // repair mode: also scan the evicted segment
