@@ -409,17 +409,30 @@ __device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity, uint6
         if (globaltimer_ns() - t0 > limit) return;
 }
 
-// Parity of the last arming of slot s after `total` armings of a ring of `n` slots,
-// or -1 if slot s was never armed.
-__device__ __forceinline__ int last_parity(long long total, int n, int s)
-{
-    if (total <= s) return -1;
-    const long long k = s + (long long)n * ((total - 1 - s) / n);
-    return static_cast<int>((k / n) & 1);
-}
+// Position in a ring of kN slots: the slot in use and the parity of its current phase.
+template <int kN>
+struct Ring {
+    uint32_t slot = 0, phase = 0;
 
-// kCount: Eq. 2 counts; kSym: upper-triangle tiles only.  Registers are per sub-partition (16384 each): with W warps a sub-partition holds
-// ceil(W / 4) of them, which bounds the registers per thread.
+    __device__ __forceinline__ void next()
+    {
+        if (++slot == kN) {
+            slot = 0;
+            phase ^= 1u;
+            wrapped = true;
+        }
+    }
+    // Parity of the last use of slot s, or -1 if it was never used.
+    __device__ __forceinline__ int last_parity(uint32_t s) const
+    {
+        if (s < slot) return static_cast<int>(phase);
+        return wrapped ? static_cast<int>(phase ^ 1u) : -1;
+    }
+
+private:
+    bool wrapped = false;
+};
+
 template <int D, bool kCount, bool kSym>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     audit_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -498,140 +511,122 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
-        long long n_a = 0, n_b = 0, n_m = 0;
-        bool ok = true;
-        for (int item = pair; item < n_items && ok; item += n_pairs) {
-            const int u = item / a.RB;
-            const int rb = item - u * a.RB;
-            const Tiles ut = unit_tiles<kSym>(a, u, rb);
-            const int ab = static_cast<int>(n_a & 1);
-            ok = lane0_wait(&a_empty[ab], static_cast<uint32_t>(((n_a >> 1) & 1) ^ 1), wc, 1);
-            if (!ok) break;
-            if (lane == 0) {
-                if (leader) mbar_arrive_expect_tx(&a_full[ab], 2 * C::A_BYTES);
-                const uint32_t full = cluster_addr(&a_full[ab], 0);
+        // One thread runs the whole role: its waits are the shortest path from a released
+        // stage to the copy that fills it.
+        if (lane == 0) {
+            Ring<2> ra;
+            Ring<C::STAGES> rb_;
+            Ring<C::MSLOTS> rm;
+            bool ok = true;
+            for (int item = pair; item < n_items && ok; item += n_pairs) {
+                const int u = item / a.RB;
+                const int rb = item - u * a.RB;
+                const Tiles ut = unit_tiles<kSym>(a, u, rb);
+                ok = mbar_wait(&a_empty[ra.slot], ra.phase ^ 1u, wc, 1);
+                if (!ok) break;
+                if (leader) mbar_arrive_expect_tx(&a_full[ra.slot], 2 * C::A_BYTES);
+                const uint32_t full = cluster_addr(&a_full[ra.slot], 0);
                 const int y = u * a.N + rb * kPM + static_cast<int>(rank) * kBM;
 #pragma unroll
                 for (int kc = 0; kc < C::KC; ++kc)
-                    tma_load_2d_pair(sA + ab * C::A_BYTES + kc * C::A_CHUNK, &tmA, full, kc * 64,
-                                     y);
-            }
-            __syncwarp();
-            ++n_a;
-            const int nt = ut.tr + ut.te;
-            for (int t = 0; t < nt && ok; ++t) {
-                const int col0 = (ut.t0 + t) * kBN;
-                const int ms = static_cast<int>(n_m % C::MSLOTS);
-                ok = lane0_wait(&m_empty[ms],
-                                static_cast<uint32_t>(((n_m / C::MSLOTS) & 1) ^ 1), wc, 2);
-                if (!ok) break;
-                if (lane == 0) {
-                    mbar_arrive_expect_tx(&m_full[ms], C::META);
-                    const int64_t off = static_cast<int64_t>(u) * a.NP + col0;
-                    bulk_load(sMeta + ms * C::META, a.colrinv + off, kBN * 4, &m_full[ms]);
-                    bulk_load(sMeta + ms * C::META + kBN * 4, a.colpos + off, kBN * 4,
-                              &m_full[ms]);
-                }
-                __syncwarp();
-                ++n_m;
-                const int yb = static_cast<int>(u * a.b_rows_per_unit + col0) +
-                               static_cast<int>(rank) * (kBN / 2);
-                for (int kc = 0; kc < C::KC; ++kc) {
-                    const int s = static_cast<int>(n_b % C::STAGES);
-                    ok = lane0_wait(&b_empty[s],
-                                    static_cast<uint32_t>(((n_b / C::STAGES) & 1) ^ 1), wc, 3);
+                    tma_load_2d_pair(sA + ra.slot * C::A_BYTES + kc * C::A_CHUNK, &tmA, full,
+                                     kc * 64, y);
+                ra.next();
+                const int nt = ut.tr + ut.te;
+                int64_t off = static_cast<int64_t>(u) * a.NP + ut.t0 * kBN;
+                int yb = static_cast<int>(u * a.b_rows_per_unit + ut.t0 * kBN) +
+                         static_cast<int>(rank) * (kBN / 2);
+                for (int t = 0; t < nt; ++t, off += kBN, yb += kBN) {
+                    ok = mbar_wait(&m_empty[rm.slot], rm.phase ^ 1u, wc, 2);
                     if (!ok) break;
-                    if (lane == 0) {
-                        if (leader) mbar_arrive_expect_tx(&b_full[s], 2 * C::B_STAGE);
-                        tma_load_2d_pair(sB + s * C::B_STAGE, &tmB, cluster_addr(&b_full[s], 0),
-                                         kc * 64, yb);
+                    uint8_t* meta = sMeta + rm.slot * C::META;
+                    mbar_arrive_expect_tx(&m_full[rm.slot], C::META);
+                    bulk_load(meta, a.colrinv + off, kBN * 4, &m_full[rm.slot]);
+                    bulk_load(meta + kBN * 4, a.colpos + off, kBN * 4, &m_full[rm.slot]);
+                    rm.next();
+#pragma unroll
+                    for (int kc = 0; kc < C::KC; ++kc) {
+                        ok = mbar_wait(&b_empty[rb_.slot], rb_.phase ^ 1u, wc, 3);
+                        if (!ok) break;
+                        if (leader) mbar_arrive_expect_tx(&b_full[rb_.slot], 2 * C::B_STAGE);
+                        tma_load_2d_pair(sB + rb_.slot * C::B_STAGE, &tmB,
+                                         cluster_addr(&b_full[rb_.slot], 0), kc * 64, yb);
+                        rb_.next();
                     }
-                    __syncwarp();
-                    ++n_b;
+                    if (!ok) break;
                 }
             }
-        }
-        // The even CTA's commits release the rings in both CTAs: each CTA stays until the
-        // last release of every slot has reached it.
-        for (int s = 0; ok && s < 2; ++s) {
-            const int p = last_parity(n_a, 2, s);
-            if (p >= 0) ok = lane0_wait(&a_empty[s], static_cast<uint32_t>(p), wc, 12);
-        }
-        for (int s = 0; ok && s < C::STAGES; ++s) {
-            const int p = last_parity(n_b, C::STAGES, s);
-            if (p >= 0) ok = lane0_wait(&b_empty[s], static_cast<uint32_t>(p), wc, 13);
-        }
-        if (!ok && lane == 0) {
-            // Let every copy this warp started land before the block exits.  A and B copies
-            // of both CTAs complete on the even CTA's barriers; the odd CTA leaves its own
-            // to that wait (the cluster barrier at the end follows it).
-            for (int s = 0; leader && s < 2; ++s) {
-                const int p = last_parity(n_a, 2, s);
-                if (p >= 0) drain_wait(&a_full[s], p, a.timeout_ns);
+            // The even CTA's commits release the rings in both CTAs: each CTA stays until
+            // the last release of every slot has reached it.
+            for (int s = 0; ok && s < 2; ++s) {
+                const int p = ra.last_parity(s);
+                if (p >= 0) ok = mbar_wait(&a_empty[s], static_cast<uint32_t>(p), wc, 12);
             }
-            for (int s = 0; leader && s < C::STAGES; ++s) {
-                const int p = last_parity(n_b, C::STAGES, s);
-                if (p >= 0) drain_wait(&b_full[s], p, a.timeout_ns);
+            for (int s = 0; ok && s < C::STAGES; ++s) {
+                const int p = rb_.last_parity(s);
+                if (p >= 0) ok = mbar_wait(&b_empty[s], static_cast<uint32_t>(p), wc, 13);
             }
-            for (int s = 0; s < C::MSLOTS; ++s) {
-                const int p = last_parity(n_m, C::MSLOTS, s);
-                if (p >= 0) drain_wait(&m_full[s], p, a.timeout_ns);
+            if (!ok) {
+                // Let every copy this warp started land before the block exits.  A and B
+                // copies of both CTAs complete on the even CTA's barriers; the odd CTA
+                // leaves its own to that wait (the cluster barrier at the end follows it).
+                for (int s = 0; leader && s < 2; ++s) {
+                    const int p = ra.last_parity(s);
+                    if (p >= 0) drain_wait(&a_full[s], p, a.timeout_ns);
+                }
+                for (int s = 0; leader && s < C::STAGES; ++s) {
+                    const int p = rb_.last_parity(s);
+                    if (p >= 0) drain_wait(&b_full[s], p, a.timeout_ns);
+                }
+                for (int s = 0; s < C::MSLOTS; ++s) {
+                    const int p = rm.last_parity(s);
+                    if (p >= 0) drain_wait(&m_full[s], p, a.timeout_ns);
+                }
             }
         }
         __syncwarp();
-    } else if (warp == 1 && !leader) {
-        // the even CTA's MMA warp issues for both
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        constexpr uint32_t idesc = umma_idesc_bf16_f32(kPM, kBN);
-        long long n_a = 0, n_b = 0, n_t = 0;
-        bool ok = true;
-        for (int item = pair; item < n_items && ok; item += n_pairs) {
-            const int u = item / a.RB;
-            const Tiles ut = unit_tiles<kSym>(a, u, item - u * a.RB);
-            const int ab = static_cast<int>(n_a & 1);
-            ok = lane0_wait(&a_full[ab], static_cast<uint32_t>((n_a >> 1) & 1), wc, 4);
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t a_base = smem_u32(sA + ab * C::A_BYTES);
-            const int nt = ut.tr + ut.te;
-            for (int t = 0; t < nt && ok; ++t) {
-                const int acc = static_cast<int>(n_t & 1);
-                ok = lane0_wait(&t_empty[acc], static_cast<uint32_t>(((n_t >> 1) & 1) ^ 1), wc,
-                                5);
+        // One thread of the even CTA issues for both.
+        if (leader && lane == 0) {
+            constexpr uint32_t idesc = umma_idesc_bf16_f32(kPM, kBN);
+            Ring<2> ra, rt;
+            Ring<C::STAGES> rb_;
+            bool ok = true;
+            for (int item = pair; item < n_items && ok; item += n_pairs) {
+                const int u = item / a.RB;
+                const Tiles ut = unit_tiles<kSym>(a, u, item - u * a.RB);
+                ok = mbar_wait(&a_full[ra.slot], ra.phase, wc, 4);
                 if (!ok) break;
-                tc_fence_after();
-                const uint32_t d_tmem = tmem + static_cast<uint32_t>(acc * kBN);
-                for (int kc = 0; kc < C::KC; ++kc) {
-                    const int s = static_cast<int>(n_b % C::STAGES);
-                    ok = lane0_wait(&b_full[s], static_cast<uint32_t>((n_b / C::STAGES) & 1), wc,
-                                    6);
+                const uint64_t ad = umma_desc_sw128(smem_u32(sA + ra.slot * C::A_BYTES));
+                const int nt = ut.tr + ut.te;
+                for (int t = 0; t < nt; ++t) {
+                    ok = mbar_wait(&t_empty[rt.slot], rt.phase ^ 1u, wc, 5);
                     if (!ok) break;
-                    tc_fence_after();
-                    if (lane == 0) {
-                        const uint64_t ad = umma_desc_sw128(a_base + kc * C::A_CHUNK);
-                        const uint64_t bd = umma_desc_sw128(smem_u32(sB + s * C::B_STAGE));
+                    const uint32_t d_tmem = tmem + rt.slot * kBN;
+#pragma unroll
+                    for (int kc = 0; kc < C::KC; ++kc) {
+                        ok = mbar_wait(&b_full[rb_.slot], rb_.phase, wc, 6);
+                        if (!ok) break;
+                        tc_fence_after();
+                        const uint64_t bd =
+                            umma_desc_sw128(smem_u32(sB + rb_.slot * C::B_STAGE));
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
-                            umma_bf16_pair(d_tmem, ad + 2u * k, bd + 2u * k, idesc,
-                                           (kc | k) != 0 ? 1u : 0u);
-                        umma_commit_pair(&b_empty[s]);
+                            umma_bf16_pair(d_tmem, ad + (kc * C::A_CHUNK >> 4) + 2u * k,
+                                           bd + 2u * k, idesc, (kc | k) != 0 ? 1u : 0u);
+                        umma_commit_pair(&b_empty[rb_.slot]);
+                        rb_.next();
                     }
-                    __syncwarp();
-                    ++n_b;
+                    if (!ok) break;
+                    umma_commit_pair(&t_full[rt.slot]);
+                    rt.next();
                 }
                 if (!ok) break;
-                if (lane == 0) umma_commit_pair(&t_full[acc]);
-                __syncwarp();
-                ++n_t;
+                umma_commit_pair(&a_empty[ra.slot]);
+                ra.next();
             }
-            if (!ok) break;
-            if (lane == 0) umma_commit_pair(&a_empty[ab]);
-            __syncwarp();
-            ++n_a;
-        }
-        // Every MMA this thread issued completes before TMEM is released.
-        if (lane == 0) {
+            // Every MMA this thread issued completes before TMEM is released.
             umma_commit_own(drain);
             drain_wait(drain, 0, a.timeout_ns);
         }
