@@ -6,9 +6,9 @@
 //   Sec. 3.4 Eq. 4   b_i(S0) = max over retained j, -1 if none; and its argmax
 //   (b_i(all))       the same over every j
 //
-// Design (persistent pairs of CTAs, one CTA per SM, 64 + 32 * kEpiWarps threads each,
-// warp-specialised).  A pair shares each 256-row work item: CTA r holds rows
-// [128 r, 128 r + 128) of A and of each B tile, and the accumulators of its own rows.
+// Design (persistent pairs of CTAs, one CTA per SM, 384 threads each, warp-specialised).  A
+// pair shares each 256-row work item: CTA r holds rows [128 r, 128 r + 128) of A and of
+// each B tile, and the accumulators of its own rows.
 //   warp 0      TMA producer: its CTA's 128 rows of the keys i (once per work item), then
 //               per 256-column tile its half of the keys j (in 64-wide K chunks) and the
 //               whole tile's column metadata (1/||k_j|| and original positions).  Key
@@ -16,8 +16,9 @@
 //   warp 1      owns TMEM (512 columns = two 128x256 fp32 accumulators); in the even CTA
 //               one thread issues tcgen05.mma.cta_group::2 (M=256, N=256, K=16,
 //               bf16 -> fp32) for both and commits to both CTAs' barriers.
-//   warps 2..   epilogue: four warps per column group g (kGW columns of each tile); a
-//               thread owns one row (TMEM lane) and keeps its running maximum.
+//   warps 2, 3  merge the column groups of every finished row and write the results.
+//   warps 4..   epilogue: four warps per column group (128 columns of each tile); a thread
+//               owns one row (TMEM lane) and keeps its running maximum.
 // Why pairs: with one CTA per 128 rows, each tile moves 64 KB of B into shared memory
 // and 96 KB of operands out of it (d = 128), beside the epilogue's broadcast loads; a
 // pair moves 32 KB in and 64 KB out per SM.  Whole calls, one CTA -> pair: Qwen3-4B
@@ -32,16 +33,34 @@
 // outputs the twin positions, and the exact similarity of each chosen twin is computed
 // afterwards (twk_refine.cu).
 //
-// Max and argmax: each 32-column chunk is scaled (the column scales carry a power of
-// two per unit that brings every value into [-1, 1]), offset to be positive and
-// reduced with 3-input maxima.  When a row of the warp improves its best, the chunk's
-// column is resolved by replacing the low 5 mantissa bits of each value with (31 - c)
-// and taking one more maximum, which returns the lowest column among values equal at
-// 2^-18 relative (near-equal candidates only; exact ties go to the lowest column
+// Max and argmax: each 32-column chunk is scaled (the column scales carry a power of two
+// per unit that brings every value into [-1, 1]), offset to be positive and reduced with
+// 3-input maxima.  The column of a maximum is the lowest of its chunk among the values
+// equal at 2^-18 relative (near-equal candidates only; exact ties go to the lowest column
 // whatever their sign, as the values are never negative).  Columns to ignore carry NaN
-// (max skips
-// NaN): padding columns have 1/||k_j|| = NaN, and window columns (|i - j| <= w) are
-// set to NaN on the few tiles that intersect the window band of the row block.
+// (max skips NaN): padding columns have 1/||k_j|| = NaN, and window columns
+// (|i - j| <= w) are set to NaN on the few tiles that intersect the window band of the
+// row block.
+//
+// What bounds the epilogue (cycle counters and copies with parts left out, at d = 128 and
+// 64): not the scaling, whose 32 broadcast loads and 64 paired multiply-adds per warp and
+// tile hide behind the MMAs, but the maxima and the look-up of the column, on an ALU that
+// issues one instruction every two cycles, and about 100 instructions per warp and tile
+// of waits and bookkeeping.  Two warps per scheduler hide little latency, so:
+//   * the warpgroups trade registers (setmaxnreg): with 200 and more the four chunks of
+//     a warp are scaled and reduced side by side (at 168 the compiler kept them apart);
+//   * at d = 128 a row that improves only copies its chunk's values to its slot in shared
+//     memory, and the column is looked up once per row block and segment;
+//   * at d = 64 a row sees few columns and some row improves in most chunks, so the copies
+//     (512 bytes of store path each) cost more than they save: there every value takes its
+//     column code along in its low 5 bits;
+//   * the next tile's barriers are tested while the current one is reduced (a wait on a
+//     completed barrier took 150 cycles), the next item's counts are loaded one item
+//     ahead, and two spare warps merge and write what the last item found.
+// Audit alone, before -> after: Qwen3-4B 16x8x16384x128 1279 -> 1559 TFLOP/s,
+// Llama-3.2-1B 16x8x8192x64 672 -> 740, policy 36x8x8192x128 1629 -> 1655, policy
+// 16x8x3001x64 728 -> 851.  Sixteen epilogue warps of 64 columns (104 registers): 1322,
+// 674, 1522, 811.  Copies without the look-up ran at 946 (d = 64).
 //
 // Count mode (Sec. 3.2 Eq. 2, the standalone scorer): instead of the maximum, each row i
 // counts the columns j outside the window with sim(i,j) > tau.  With x_ij the raw dot
@@ -58,6 +77,7 @@
 // order), so every tile belongs to exactly one of the two maxima.  The kernel writes
 // both winners; the maximum over all columns is the larger of the two, taken on the
 // exact similarities computed afterwards.
+#include <atomic>
 #include <cfloat>
 
 #include "twk_internal.h"
@@ -66,34 +86,54 @@
 namespace twk {
 namespace {
 
-constexpr int kEpiWarps = 8;                  // epilogue warps: 2 per SM sub-partition
-constexpr int kGroups = kEpiWarps / 4;        // column groups per tile
-constexpr int kGW = kBN / kGroups;            // columns per group (a multiple of 32)
-constexpr int kThreads = 64 + 32 * kEpiWarps; // + TMA warp + MMA warp
+constexpr int kHelperWarps = 4;                    // TMA, MMA, two that merge: a whole warpgroup
+constexpr int kEpiWarps = 8;                       // epilogue warps: 2 per SM sub-partition
+constexpr int kGroups = kEpiWarps / 4;             // column groups per tile
+constexpr int kGW = kBN / kGroups;                 // columns per group
+constexpr int kCh = kGW / 32;                      // 32-column chunks per group
+constexpr int kThreads = 32 * (kHelperWarps + kEpiWarps);
+constexpr int kLaunchRegs = 168;                   // registers per thread at launch
 constexpr uint32_t kTmemCols = 512;
+// a row's slot for the values of its best chunk: 32 floats and 16 bytes of padding, which
+// spreads the lanes of a 16-byte access over the banks
+constexpr int kSlot = 144;
 
-template <int D, bool kSym = false>
+template <int D, bool kCount = false, bool kSym = false>
 struct AuditCfg {
+    // Registers per thread after the warpgroups have traded theirs.  The epilogue's number
+    // decides how far the compiler interleaves its chunks: d = 128 ran at 1571 TFLOP/s
+    // with 200, 1520 with 216, 1465 with 232; d = 64 at 721 with 192, 718 with 200, 749
+    // with 216.
+    static constexpr int HELPER_REGS = D == 128 ? 104 : 72;
+    static constexpr int EPI_REGS = D == 128 ? 200 : 216;
+    static_assert(kHelperWarps * HELPER_REGS + kEpiWarps * EPI_REGS <=
+                      (kHelperWarps + kEpiWarps) * kLaunchRegs,
+                  "the split draws on the registers of the launch");
     static constexpr int KC = D / 64;                 // 128-byte K chunks per key row
     static constexpr int A_CHUNK = kBM * 128;         // 16 KB
     static constexpr int A_BYTES = KC * A_CHUNK;
     static constexpr int B_STAGE = kBN / 2 * 128;     // 16 KB: this CTA's half of a K chunk
-    static constexpr int STAGES = 8;
-    static constexpr int MSLOTS = 8;
+    static constexpr int STAGES = 6;
+    static constexpr int MSLOTS = 4;
     static constexpr int META = kBN * 8;              // rinv[256] + pos[256]
     static constexpr int OFF_A = 0;
     static constexpr int OFF_B = OFF_A + 2 * A_BYTES;
     static constexpr int OFF_META = OFF_B + STAGES * B_STAGE;
-    static constexpr int OFF_X = OFF_META + MSLOTS * META;   // 2 x (groups-1) x 128 x 16 B
+    static constexpr int OFF_X = OFF_META + MSLOTS * META;   // 2 x groups x 128 x 16 B
     // symmetric mode: each group's four warps exchange their per-column maxima here
     // (two tile parities x groups x 4 lane quarters x 128 columns)
-    static constexpr int OFF_CB = OFF_X + 2 * (kGroups - 1) * kBM * 16;
+    static constexpr int OFF_CB = OFF_X + 2 * kGroups * kBM * 16;
     static constexpr int CB_BYTES = kSym ? 2 * kGroups * 4 * kBM * 4 : 0;
-    static constexpr int OFF_BAR = OFF_CB + CB_BYTES;
+    // argmax mode: the 32 values of each thread's best chunk so far
+    static constexpr int OFF_BEST = OFF_CB + CB_BYTES;
+    static constexpr int BEST_BYTES =
+        kCount || kSym || D == 64 ? 0 : kGroups * kBM * kSlot;
+    static constexpr int OFF_BAR = OFF_BEST + BEST_BYTES;
     static constexpr int NBAR = 2 + 2 + 2 * STAGES + 2 * MSLOTS + 2 + 2 + 2 + 2 + 1 +
                                 (kSym ? 2 * kGroups : 0);
     static constexpr int OFF_MISC = OFF_BAR + NBAR * 8;
     static constexpr int BYTES = OFF_MISC + 16 + 1024;       // + 1024 for alignment
+    static_assert(BYTES <= 232448, "shared memory per CTA");
 };
 
 __device__ __forceinline__ float fmax3(float a, float b, float c)
@@ -139,8 +179,8 @@ __device__ __forceinline__ float tree32(const float (&p)[32])
     return fmax3(r0, r1, fmaxf(r2, r3));
 }
 
-// Running best of one row over one segment: the scaled similarity x_ij / ||k_j|| in
-// fp32 and its column.
+// Running best of one row over one segment: the largest scaled similarity so far and the
+// first column of its 32-column chunk (the column itself once resolved, see keep_chunk).
 struct Best {
     float v;
     int col;
@@ -153,23 +193,47 @@ struct Best {
 // multiply-add then needs no register for it.
 constexpr float kOffset = 1.0f + 0x1p-10f;
 
-// Folds 32 columns [col0, col0 + 32) into the running best.  Each accumulator value is
-// scaled and offset, v = x_ij 2^-e_u/||k_j|| + kOffset > 0, in one fused multiply-add
-// (NaN where the window drops the column, or where the column scale is NaN on
-// padding), and the chunk's maximum is taken.  Only when some row of the warp improves
-// on its best (strictly, so an earlier column keeps a tie) is the column resolved: each
-// value's 5 lowest mantissa bits are replaced by (31 - column) and one more maximum
-// returns the lowest column among the values equal to the maximum at 2^-18 relative.
-// The values are positive, where a larger low-bit code means a larger float, so ties
-// go to the lowest column whatever the sign of the similarity.  Most chunks cost one
-// fused multiply-add and one max tree.
-template <bool kMasked, bool kEager = false>
-__device__ __forceinline__ void fold32(const uint32_t (&x)[32], const float* rinv,
-                                       const int* pos, int rw, uint32_t w2, uint32_t mask,
-                                       int col0, Best& b)
+// Where `up`, the thread's 32 values go to its slot.
+__device__ __forceinline__ void keep_chunk(uint32_t slot, const float (&v)[32], bool up)
+{
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.ne.u32 p, %0, 0;\n\t"
+            "@p st.shared.v4.f32 [%1], {%2, %3, %4, %5};\n\t}" ::"r"(up ? 1u : 0u),
+            "r"(slot + 16u * q), "f"(v[4 * q]), "f"(v[4 * q + 1]), "f"(v[4 * q + 2]),
+            "f"(v[4 * q + 3]));
+}
+
+// The column of a running best: the lowest of its chunk whose value agrees with the
+// maximum to 2^-18 relative (the 5 lowest mantissa bits cleared; the values are positive,
+// so "at least the cleared maximum" is that comparison).
+__device__ __forceinline__ void resolve_best(uint32_t slot, uint32_t mask, Best& b)
+{
+    if (b.col < 0) return;
+    const float floor_v = __uint_as_float(__float_as_uint(b.v) & mask);
+    int c = 31;
+#pragma unroll
+    for (int q = 7; q >= 0; --q) {
+        float v[4];
+        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
+                     : "r"(slot + 16u * q));
+#pragma unroll
+        for (int e = 3; e >= 0; --e) c = v[e] >= floor_v ? 4 * q + e : c;
+    }
+    b.col += c;
+}
+
+// Each accumulator value scaled and offset, v = x_ij 2^-e_u/||k_j|| + kOffset > 0, in one
+// fused multiply-add (NaN where the window drops the column, or where the column scale is
+// NaN on padding).
+template <bool kMasked>
+__device__ __forceinline__ void scale32(const uint32_t (&x)[32], const float* rinv,
+                                        const int* pos, int rw, uint32_t w2, float (&v)[32])
 {
     const float2 ofs = make_float2(kOffset, kOffset);
-    float v[32];
 #pragma unroll
     for (int k = 0; k < 32; k += 4) {
         const float4 r = *reinterpret_cast<const float4*>(rinv + k);
@@ -191,89 +255,105 @@ __device__ __forceinline__ void fold32(const uint32_t (&x)[32], const float* rin
             v[k + 3] = (static_cast<uint32_t>(q.w - rw) > w2) ? v[k + 3] : nan_f();
         }
     }
-    if constexpr (kEager) {
-        // Where some row of the warp improves in most chunks the vote only adds a
-        // branch: every value is packed, one tree gives the lowest column among the
-        // values equal to the maximum at 2^-18 relative, and the running best moves at
-        // that resolution (an earlier column keeps a tie).
-        float p[32];
+}
+
+// The symmetric mode's row direction: each value's 5 lowest mantissa bits are replaced by
+// (31 - column) and one tree gives the lowest column among the values equal to the maximum
+// at 2^-18 relative; the running best moves at that resolution.
+template <bool kMasked>
+__device__ __forceinline__ void fold32_packed(const uint32_t (&x)[32], const float* rinv,
+                                              const int* pos, int rw, uint32_t w2, uint32_t mask,
+                                              int col0, Best& b)
+{
+    float v[32];
+    scale32<kMasked>(x, rinv, pos, rw, w2, v);
 #pragma unroll
-        for (int k = 0; k < 32; ++k) p[k] = pack(v[k], 31u - static_cast<uint32_t>(k), mask);
-        const uint32_t mp = __float_as_uint(tree32(p));
-        const float m = __uint_as_float(mp & mask);
-        if (m > b.v) {
-            b.v = m;
-            b.col = col0 + 31 - static_cast<int>(mp & 31u);
-        }
-        return;
-    }
-    const float m = tree32(v);
-    const bool up = m > b.v;
-    if (__any_sync(0xFFFFFFFFu, up)) {
-        float p[32];
-#pragma unroll
-        for (int k = 0; k < 32; ++k) p[k] = pack(v[k], 31u - static_cast<uint32_t>(k), mask);
-        const int c = 31 - static_cast<int>(__float_as_uint(tree32(p)) & 31u);
-        if (up) {
-            b.v = m;
-            b.col = col0 + c;
-        }
+    for (int k = 0; k < 32; ++k) v[k] = pack(v[k], 31u - static_cast<uint32_t>(k), mask);
+    const uint32_t mp = __float_as_uint(tree32(v));
+    const float m = __uint_as_float(mp & mask);
+    if (m > b.v) {
+        b.v = m;
+        b.col = col0 + 31 - static_cast<int>(mp & 31u);
     }
 }
 
-// The thread's kGW accumulator columns of one tile, loaded into registers (after this,
-// the accumulator may be released: the MMA can overwrite it while x is reduced).
-__device__ __forceinline__ void load_group(uint32_t taddr, uint32_t (&x0)[32], uint32_t (&x1)[32],
-                                           uint32_t (&x2)[32], uint32_t (&x3)[32])
+// The thread's accumulator columns of one tile, loaded into registers (after this, the
+// accumulator may be released: the MMA can overwrite it while x is reduced).
+__device__ __forceinline__ void load_group(uint32_t taddr, uint32_t (&x)[kCh][32])
 {
-    static_assert(kGW == 128, "one 128-column group per warp");
-    tmem_ld_32x32b_x32(taddr, x0);
-    tmem_ld_32x32b_x32(taddr + 32, x1);
-    tmem_ld_32x32b_x32(taddr + 64, x2);
-    tmem_ld_32x32b_x32(taddr + 96, x3);
+#pragma unroll
+    for (int k = 0; k < kCh; ++k) tmem_ld_32x32b_x32(taddr + 32 * k, x[k]);
     tmem_wait_ld();
-    reg_fence(x0);
-    reg_fence(x1);
-    reg_fence(x2);
-    reg_fence(x3);
+#pragma unroll
+    for (int k = 0; k < kCh; ++k) reg_fence(x[k]);
 }
 
-// Folds the loaded group into the running best, 32 columns at a time in column order.
-template <bool kMasked, bool kEager>
-__device__ __forceinline__ void reduce_group(const uint32_t (&x0)[32], const uint32_t (&x1)[32],
-                                             const uint32_t (&x2)[32], const uint32_t (&x3)[32],
-                                             const float* rinv, const int* pos, int rw,
-                                             uint32_t w2, uint32_t mask, int col0, Best& b)
+// The loaded group scaled, and the maximum of each of its chunks, with nothing between the
+// chunks that would keep their instructions apart.
+template <bool kMasked>
+__device__ __forceinline__ void scale_group(const uint32_t (&x)[kCh][32], const float* rinv,
+                                            const int* pos, int rw, uint32_t w2,
+                                            float (&v)[kCh][32], float (&m)[kCh])
 {
-    fold32<kMasked, kEager>(x0, rinv, pos, rw, w2, mask, col0, b);
-    fold32<kMasked, kEager>(x1, rinv + 32, pos + 32, rw, w2, mask, col0 + 32, b);
-    fold32<kMasked, kEager>(x2, rinv + 64, pos + 64, rw, w2, mask, col0 + 64, b);
-    fold32<kMasked, kEager>(x3, rinv + 96, pos + 96, rw, w2, mask, col0 + 96, b);
+#pragma unroll
+    for (int k = 0; k < kCh; ++k) scale32<kMasked>(x[k], rinv + 32 * k, pos + 32 * k, rw, w2, v[k]);
+#pragma unroll
+    for (int k = 0; k < kCh; ++k) m[k] = tree32(v[k]);
 }
 
-// Folds one tile's group, eagerly (every chunk resolved, no vote) or vote-gated.
-template <bool kEager>
-__device__ __forceinline__ void reduce_tile(bool band, const uint32_t (&x0)[32],
-                                            const uint32_t (&x1)[32], const uint32_t (&x2)[32],
-                                            const uint32_t (&x3)[32], const float* rinv,
+// Where a row of the warp improves on its best (strictly, so an earlier chunk keeps a
+// tie), its first chunk with the group's largest maximum is kept: the 32 values go to the
+// row's slot, and which column it was is looked up once, when the segment ends.
+__device__ __forceinline__ void keep_best(const float (&v)[kCh][32], const float (&m)[kCh],
+                                          int col0, uint32_t slot, Best& b)
+{
+    float top = m[0];
+#pragma unroll
+    for (int k = 1; k < kCh; ++k) top = fmaxf(top, m[k]);
+    const bool up = top > b.v;
+    bool here[kCh];
+    unsigned any[kCh];
+    bool left = up;
+#pragma unroll
+    for (int k = 0; k < kCh; ++k) {
+        here[k] = left && m[k] == top;
+        left = left && !here[k];
+        any[k] = __ballot_sync(0xFFFFFFFFu, here[k]);   // the votes overlap each other
+    }
+#pragma unroll
+    for (int k = 0; k < kCh; ++k) {
+        if (any[k]) keep_chunk(slot, v[k], here[k]);
+        b.col = here[k] ? col0 + 32 * k : b.col;
+    }
+    b.v = up ? top : b.v;
+}
+
+// The same without a slot: the low 5 mantissa bits of each value give way to (31 - column),
+// so that one more maximum returns the lowest column among the values equal at 2^-18
+// relative, and the running best moves at that resolution.
+template <bool kMasked>
+__device__ __forceinline__ void fold_packed(const uint32_t (&x)[kCh][32], const float* rinv,
                                             const int* pos, int rw, uint32_t w2, uint32_t mask,
                                             int col0, Best& b)
 {
-    if (band) reduce_group<true, kEager>(x0, x1, x2, x3, rinv, pos, rw, w2, mask, col0, b);
-    else reduce_group<false, kEager>(x0, x1, x2, x3, rinv, pos, rw, w2, mask, col0, b);
-}
-
-// The argmax modes fold eagerly at d = 64 only.  There a tile's epilogue is twice its
-// tensor-core time and, with fewer columns per row, the running best improves in most
-// chunks: the eager fold measured 661 TFLOP/s against 617 at the Llama-3.2-1B shape.  It
-// compares candidates of different chunks at the packed resolution, so more near ties
-// (within 2^-18 relative of the maximum) go to the earlier column; at d = 128 it gained
-// nothing measurable (16 eager tiles per row block: 1275 against 1271 TFLOP/s), and the
-// vote-gated fold keeps the exact comparison across chunks there.
-template <int D>
-__device__ __forceinline__ constexpr bool eager_fold()
-{
-    return D == 64;
+    float v[kCh][32];
+    uint32_t mp[kCh];
+#pragma unroll
+    for (int k = 0; k < kCh; ++k) scale32<kMasked>(x[k], rinv + 32 * k, pos + 32 * k, rw, w2, v[k]);
+#pragma unroll
+    for (int k = 0; k < kCh; ++k) {
+#pragma unroll
+        for (int c = 0; c < 32; ++c) v[k][c] = pack(v[k][c], 31u - static_cast<uint32_t>(c), mask);
+        mp[k] = __float_as_uint(tree32(v[k]));
+    }
+#pragma unroll
+    for (int k = 0; k < kCh; ++k) {
+        const float m = __uint_as_float(mp[k] & mask);
+        if (m > b.v) {
+            b.v = m;
+            b.col = col0 + 32 * k + 31 - static_cast<int>(mp[k] & 31u);
+        }
+    }
 }
 
 // sat(a * b + c): fp32 fused multiply-add clamped to [0, 1], NaN to 0.
@@ -310,16 +390,13 @@ __device__ __forceinline__ float2 count32(const uint32_t (&x)[32], const float* 
 }
 
 template <bool kMasked>
-__device__ __forceinline__ float count_group(const uint32_t (&x0)[32], const uint32_t (&x1)[32],
-                                             const uint32_t (&x2)[32], const uint32_t (&x3)[32],
-                                             const float* rinv, const int* pos, int rw,
-                                             uint32_t w2, float ts)
+__device__ __forceinline__ float count_group(const uint32_t (&x)[kCh][32], const float* rinv,
+                                             const int* pos, int rw, uint32_t w2, float ts)
 {
-    const float2 a = __fadd2_rn(count32<kMasked>(x0, rinv, pos, rw, w2, ts),
-                                count32<kMasked>(x1, rinv + 32, pos + 32, rw, w2, ts));
-    const float2 b = __fadd2_rn(count32<kMasked>(x2, rinv + 64, pos + 64, rw, w2, ts),
-                                count32<kMasked>(x3, rinv + 96, pos + 96, rw, w2, ts));
-    const float2 c = __fadd2_rn(a, b);
+    float2 c = count32<kMasked>(x[0], rinv, pos, rw, w2, ts);
+#pragma unroll
+    for (int k = 1; k < kCh; ++k)
+        c = __fadd2_rn(c, count32<kMasked>(x[k], rinv + 32 * k, pos + 32 * k, rw, w2, ts));
     return c.x + c.y;
 }
 
@@ -363,32 +440,47 @@ __device__ __forceinline__ uint32_t colpass32(const uint32_t (&x)[32], const int
 struct Tiles {
     int tr;   // tiles of segment 0 (retained, or every column in mode 0)
     int te;   // tiles of segment 1 (evicted; 0 unless b_all is wanted)
-    int t0;   // the first tile (symmetric mode: the tile holding column 128 rb - 0..128)
+    int t0;   // the first tile (symmetric mode: the tile holding the row block's columns)
 };
 
-// Symmetric mode: row block rb takes the tiles from the one holding its own first
-// column, rb / 2, to the last; the pairs left of them reach rb's rows through the
-// column maxima of the row blocks before it.
+// The work items of one CTA pair in order.  The next item's retained count is loaded while
+// the current item is worked on, so that no role waits for it between items.
 template <bool kSym>
-__device__ __forceinline__ Tiles unit_tiles(const AuditArgs& a, int u, int rb)
-{
-    if (kSym) {
-        const int t0 = rb;
-        return {(a.N + kBN - 1) / kBN - t0, 0, t0};
-    }
-    if (!a.repair_mode) return {(a.N + kBN - 1) / kBN, 0, 0};
-    const int kb = a.kb[u];
-    return {(kb + kBN - 1) / kBN, a.need_all ? (a.N - kb + kBN - 1) / kBN : 0, 0};
-}
+struct Items {
+    int item, u, rb;        // the item at hand: its unit and row block
+    int kb = 0;             // |S0| of its unit (repair mode)
+    int nu = 0, nrb = 0, nkb = 0;   // the next one's
 
-// Lane 0 waits, the warp follows its verdict.
-__device__ __forceinline__ bool lane0_wait(uint64_t* bar, uint32_t parity, const WaitCtl& w,
-                                           int where)
-{
-    int ok = 1;
-    if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity, w, where) ? 1 : 0;
-    return __shfl_sync(0xFFFFFFFFu, ok, 0) != 0;
-}
+    __device__ __forceinline__ Items(const AuditArgs& a, int first) : item(first)
+    {
+        u = item / a.RB;
+        rb = item - u * a.RB;
+        if (a.repair_mode && item < a.U * a.RB) kb = a.kb[u];
+    }
+    __device__ __forceinline__ void prefetch(const AuditArgs& a, int step)
+    {
+        const int n = item + step;
+        nu = n / a.RB;
+        nrb = n - nu * a.RB;
+        if (a.repair_mode && n < a.U * a.RB) nkb = a.kb[nu];
+    }
+    __device__ __forceinline__ void advance(int step)
+    {
+        item += step;
+        u = nu;
+        rb = nrb;
+        kb = nkb;
+    }
+    // Symmetric mode: row block rb takes the tiles from the one holding its own columns, rb,
+    // to the last; the pairs left of them reach rb's rows through the column maxima of
+    // the row blocks before it.
+    __device__ __forceinline__ Tiles tiles(const AuditArgs& a) const
+    {
+        if (kSym) return {(a.N + kBN - 1) / kBN - rb, 0, rb};
+        if (!a.repair_mode) return {(a.N + kBN - 1) / kBN, 0, 0};
+        return {(kb + kBN - 1) / kBN, a.need_all ? (a.N - kb + kBN - 1) / kBN : 0, 0};
+    }
+};
 
 // Every lane waits (each needs the acquire), the warp agrees on the verdict.
 __device__ __forceinline__ bool all_wait(uint64_t* bar, uint32_t parity, const WaitCtl& w,
@@ -434,11 +526,15 @@ private:
 };
 
 template <int D, bool kCount, bool kSym>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1)
+    __launch_bounds__(kThreads, 1)
     audit_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ AuditArgs a)
 {
-    using C = AuditCfg<D, kSym>;
+    using C = AuditCfg<D, kCount, kSym>;
+    // Chunks are compared with each other exactly at d = 128, and at 2^-18 relative (the
+    // earlier chunk on a tie) at d = 64.
+    constexpr bool kPacked = D == 64;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     uint8_t* sA = smem + C::OFF_A;
@@ -462,7 +558,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::OFF_MISC);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_MISC + 4);
 
-    const int warp = threadIdx.x >> 5;
+    // From a shuffle the compiler knows that the warp's number is the same in every lane
+    // (d = 128: 1559 TFLOP/s against 1482 without; at d = 64 it then spills, for 1 %).
+    const int warp = D == 64 && !kCount
+                         ? static_cast<int>(threadIdx.x >> 5)
+                         : __shfl_sync(0xFFFFFFFFu, static_cast<int>(threadIdx.x >> 5), 0);
     const int lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
@@ -471,8 +571,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             mbar_init(&a_empty[i], 1);
             mbar_init(&t_full[i], 1);
             mbar_init(&t_empty[i], 2 * kEpiWarps);   // both CTAs' epilogues
-            mbar_init(&x_full[i], (kGroups - 1) * kBM);
-            mbar_init(&x_empty[i], kBM);
+            mbar_init(&x_full[i], kGroups * kBM);
+            mbar_init(&x_empty[i], 64);
         }
         for (int i = 0; i < C::STAGES; ++i) {
             mbar_init(&b_full[i], 1);
@@ -509,131 +609,201 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     const uint32_t rank = cluster_rank();
     const bool leader = rank == 0;
 
-    if (warp == 0) {
-        // ------------------------------------------------------------ TMA producer
-        // One thread runs the whole role: its waits are the shortest path from a released
-        // stage to the copy that fills it.
-        if (lane == 0) {
-            Ring<2> ra;
-            Ring<C::STAGES> rb_;
-            Ring<C::MSLOTS> rm;
-            bool ok = true;
-            for (int item = pair; item < n_items && ok; item += n_pairs) {
-                const int u = item / a.RB;
-                const int rb = item - u * a.RB;
-                const Tiles ut = unit_tiles<kSym>(a, u, rb);
-                ok = mbar_wait(&a_empty[ra.slot], ra.phase ^ 1u, wc, 1);
-                if (!ok) break;
-                if (leader) mbar_arrive_expect_tx(&a_full[ra.slot], 2 * C::A_BYTES);
-                const uint32_t full = cluster_addr(&a_full[ra.slot], 0);
-                const int y = u * a.N + rb * kPM + static_cast<int>(rank) * kBM;
-#pragma unroll
-                for (int kc = 0; kc < C::KC; ++kc)
-                    tma_load_2d_pair(sA + ra.slot * C::A_BYTES + kc * C::A_CHUNK, &tmA, full,
-                                     kc * 64, y);
-                ra.next();
-                const int nt = ut.tr + ut.te;
-                int64_t off = static_cast<int64_t>(u) * a.NP + ut.t0 * kBN;
-                int yb = static_cast<int>(u * a.b_rows_per_unit + ut.t0 * kBN) +
-                         static_cast<int>(rank) * (kBN / 2);
-                for (int t = 0; t < nt; ++t, off += kBN, yb += kBN) {
-                    ok = mbar_wait(&m_empty[rm.slot], rm.phase ^ 1u, wc, 2);
+    if (warp < kHelperWarps) {
+        setmaxnreg_dec<C::HELPER_REGS>();
+        if (warp == 0) {
+            // ------------------------------------------------------------ TMA producer
+            // One thread runs the whole role: its waits are the shortest path from a released
+            // stage to the copy that fills it.
+            if (lane == 0) {
+                Ring<2> ra;
+                Ring<C::STAGES> rb_;
+                Ring<C::MSLOTS> rm;
+                bool ok = true;
+                for (Items<kSym> it(a, pair); it.item < n_items && ok; it.advance(n_pairs)) {
+                    const int u = it.u, rb = it.rb;
+                    const Tiles ut = it.tiles(a);
+                    it.prefetch(a, n_pairs);
+                    ok = mbar_wait(&a_empty[ra.slot], ra.phase ^ 1u, wc, 1);
                     if (!ok) break;
-                    uint8_t* meta = sMeta + rm.slot * C::META;
-                    mbar_arrive_expect_tx(&m_full[rm.slot], C::META);
-                    bulk_load(meta, a.colrinv + off, kBN * 4, &m_full[rm.slot]);
-                    bulk_load(meta + kBN * 4, a.colpos + off, kBN * 4, &m_full[rm.slot]);
-                    rm.next();
+                    if (leader) mbar_arrive_expect_tx(&a_full[ra.slot], 2 * C::A_BYTES);
+                    const uint32_t full = cluster_addr(&a_full[ra.slot], 0);
+                    const int y = u * a.N + rb * kPM + static_cast<int>(rank) * kBM;
 #pragma unroll
-                    for (int kc = 0; kc < C::KC; ++kc) {
-                        ok = mbar_wait(&b_empty[rb_.slot], rb_.phase ^ 1u, wc, 3);
+                    for (int kc = 0; kc < C::KC; ++kc)
+                        tma_load_2d_pair(sA + ra.slot * C::A_BYTES + kc * C::A_CHUNK, &tmA, full,
+                                         kc * 64, y);
+                    ra.next();
+                    const int nt = ut.tr + ut.te;
+                    int64_t off = static_cast<int64_t>(u) * a.NP + ut.t0 * kBN;
+                    int yb = static_cast<int>(u * a.b_rows_per_unit + ut.t0 * kBN) +
+                             static_cast<int>(rank) * (kBN / 2);
+                    for (int t = 0; t < nt; ++t, off += kBN, yb += kBN) {
+                        ok = mbar_wait(&m_empty[rm.slot], rm.phase ^ 1u, wc, 2);
                         if (!ok) break;
-                        if (leader) mbar_arrive_expect_tx(&b_full[rb_.slot], 2 * C::B_STAGE);
-                        tma_load_2d_pair(sB + rb_.slot * C::B_STAGE, &tmB,
-                                         cluster_addr(&b_full[rb_.slot], 0), kc * 64, yb);
-                        rb_.next();
+                        uint8_t* meta = sMeta + rm.slot * C::META;
+                        mbar_arrive_expect_tx(&m_full[rm.slot], C::META);
+                        bulk_load(meta, a.colrinv + off, kBN * 4, &m_full[rm.slot]);
+                        bulk_load(meta + kBN * 4, a.colpos + off, kBN * 4, &m_full[rm.slot]);
+                        rm.next();
+#pragma unroll
+                        for (int kc = 0; kc < C::KC; ++kc) {
+                            ok = mbar_wait(&b_empty[rb_.slot], rb_.phase ^ 1u, wc, 3);
+                            if (!ok) break;
+                            if (leader) mbar_arrive_expect_tx(&b_full[rb_.slot], 2 * C::B_STAGE);
+                            tma_load_2d_pair(sB + rb_.slot * C::B_STAGE, &tmB,
+                                             cluster_addr(&b_full[rb_.slot], 0), kc * 64, yb);
+                            rb_.next();
+                        }
+                        if (!ok) break;
                     }
-                    if (!ok) break;
                 }
-            }
-            // The even CTA's commits release the rings in both CTAs: each CTA stays until
-            // the last release of every slot has reached it.
-            for (int s = 0; ok && s < 2; ++s) {
-                const int p = ra.last_parity(s);
-                if (p >= 0) ok = mbar_wait(&a_empty[s], static_cast<uint32_t>(p), wc, 12);
-            }
-            for (int s = 0; ok && s < C::STAGES; ++s) {
-                const int p = rb_.last_parity(s);
-                if (p >= 0) ok = mbar_wait(&b_empty[s], static_cast<uint32_t>(p), wc, 13);
-            }
-            if (!ok) {
-                // Let every copy this warp started land before the block exits.  A and B
-                // copies of both CTAs complete on the even CTA's barriers; the odd CTA
-                // leaves its own to that wait (the cluster barrier at the end follows it).
-                for (int s = 0; leader && s < 2; ++s) {
+                // The even CTA's commits release the rings in both CTAs: each CTA stays until
+                // the last release of every slot has reached it.
+                for (int s = 0; ok && s < 2; ++s) {
                     const int p = ra.last_parity(s);
-                    if (p >= 0) drain_wait(&a_full[s], p, a.timeout_ns);
+                    if (p >= 0) ok = mbar_wait(&a_empty[s], static_cast<uint32_t>(p), wc, 12);
                 }
-                for (int s = 0; leader && s < C::STAGES; ++s) {
+                for (int s = 0; ok && s < C::STAGES; ++s) {
                     const int p = rb_.last_parity(s);
-                    if (p >= 0) drain_wait(&b_full[s], p, a.timeout_ns);
+                    if (p >= 0) ok = mbar_wait(&b_empty[s], static_cast<uint32_t>(p), wc, 13);
                 }
-                for (int s = 0; s < C::MSLOTS; ++s) {
-                    const int p = rm.last_parity(s);
-                    if (p >= 0) drain_wait(&m_full[s], p, a.timeout_ns);
+                if (!ok) {
+                    // Let every copy this warp started land before the block exits.  A and B
+                    // copies of both CTAs complete on the even CTA's barriers; the odd CTA
+                    // leaves its own to that wait (the cluster barrier at the end follows it).
+                    for (int s = 0; leader && s < 2; ++s) {
+                        const int p = ra.last_parity(s);
+                        if (p >= 0) drain_wait(&a_full[s], p, a.timeout_ns);
+                    }
+                    for (int s = 0; leader && s < C::STAGES; ++s) {
+                        const int p = rb_.last_parity(s);
+                        if (p >= 0) drain_wait(&b_full[s], p, a.timeout_ns);
+                    }
+                    for (int s = 0; s < C::MSLOTS; ++s) {
+                        const int p = rm.last_parity(s);
+                        if (p >= 0) drain_wait(&m_full[s], p, a.timeout_ns);
+                    }
                 }
             }
-        }
-        __syncwarp();
-    } else if (warp == 1) {
-        // ------------------------------------------------------------ MMA issuer
-        // One thread of the even CTA issues for both.
-        if (leader && lane == 0) {
-            constexpr uint32_t idesc = umma_idesc_bf16_f32(kPM, kBN);
-            Ring<2> ra, rt;
-            Ring<C::STAGES> rb_;
-            bool ok = true;
-            for (int item = pair; item < n_items && ok; item += n_pairs) {
-                const int u = item / a.RB;
-                const Tiles ut = unit_tiles<kSym>(a, u, item - u * a.RB);
-                ok = mbar_wait(&a_full[ra.slot], ra.phase, wc, 4);
-                if (!ok) break;
-                const uint64_t ad = umma_desc_sw128(smem_u32(sA + ra.slot * C::A_BYTES));
-                const int nt = ut.tr + ut.te;
-                for (int t = 0; t < nt; ++t) {
-                    ok = mbar_wait(&t_empty[rt.slot], rt.phase ^ 1u, wc, 5);
+            __syncwarp();
+        } else if (warp == 1) {
+            // ------------------------------------------------------------ MMA issuer
+            // One thread of the even CTA issues for both.
+            if (leader && lane == 0) {
+                constexpr uint32_t idesc = umma_idesc_bf16_f32(kPM, kBN);
+                Ring<2> ra, rt;
+                Ring<C::STAGES> rb_;
+                bool ok = true;
+                for (Items<kSym> it(a, pair); it.item < n_items && ok; it.advance(n_pairs)) {
+                    const Tiles ut = it.tiles(a);
+                    it.prefetch(a, n_pairs);
+                    ok = mbar_wait(&a_full[ra.slot], ra.phase, wc, 4);
                     if (!ok) break;
-                    const uint32_t d_tmem = tmem + rt.slot * kBN;
-#pragma unroll
-                    for (int kc = 0; kc < C::KC; ++kc) {
-                        ok = mbar_wait(&b_full[rb_.slot], rb_.phase, wc, 6);
+                    const uint64_t ad = umma_desc_sw128(smem_u32(sA + ra.slot * C::A_BYTES));
+                    const int nt = ut.tr + ut.te;
+                    for (int t = 0; t < nt; ++t) {
+                        ok = mbar_wait(&t_empty[rt.slot], rt.phase ^ 1u, wc, 5);
                         if (!ok) break;
-                        tc_fence_after();
-                        const uint64_t bd =
-                            umma_desc_sw128(smem_u32(sB + rb_.slot * C::B_STAGE));
+                        const uint32_t d_tmem = tmem + rt.slot * kBN;
 #pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            umma_bf16_pair(d_tmem, ad + (kc * C::A_CHUNK >> 4) + 2u * k,
-                                           bd + 2u * k, idesc, (kc | k) != 0 ? 1u : 0u);
-                        umma_commit_pair(&b_empty[rb_.slot]);
-                        rb_.next();
+                        for (int kc = 0; kc < C::KC; ++kc) {
+                            ok = mbar_wait(&b_full[rb_.slot], rb_.phase, wc, 6);
+                            if (!ok) break;
+                            tc_fence_after();
+                            const uint64_t bd =
+                                umma_desc_sw128(smem_u32(sB + rb_.slot * C::B_STAGE));
+#pragma unroll
+                            for (int k = 0; k < 4; ++k)
+                                umma_bf16_pair(d_tmem, ad + (kc * C::A_CHUNK >> 4) + 2u * k,
+                                               bd + 2u * k, idesc, (kc | k) != 0 ? 1u : 0u);
+                            umma_commit_pair(&b_empty[rb_.slot]);
+                            rb_.next();
+                        }
+                        if (!ok) break;
+                        umma_commit_pair(&t_full[rt.slot]);
+                        rt.next();
                     }
                     if (!ok) break;
-                    umma_commit_pair(&t_full[rt.slot]);
-                    rt.next();
+                    umma_commit_pair(&a_empty[ra.slot]);
+                    ra.next();
                 }
-                if (!ok) break;
-                umma_commit_pair(&a_empty[ra.slot]);
-                ra.next();
+                // Every MMA this thread issued completes before TMEM is released.
+                umma_commit_own(drain);
+                drain_wait(drain, 0, a.timeout_ns);
             }
-            // Every MMA this thread issued completes before TMEM is released.
-            umma_commit_own(drain);
-            drain_wait(drain, 0, a.timeout_ns);
+            __syncwarp();
+        } else {
+            // ------------------------------------------------------------ merge
+            // Two warps combine the column groups of every row and write the result, while the
+            // epilogue is already at the next item.
+            uint32_t n_x = 0;
+            bool ok = true;
+            for (Items<kSym> it(a, pair); it.item < n_items && ok; it.advance(n_pairs), ++n_x) {
+                it.prefetch(a, n_pairs);
+                const int xb = static_cast<int>(n_x & 1);
+                ok = all_wait(&x_full[xb], (n_x >> 1) & 1, wc, 10);
+                if (!ok) break;
+                const int64_t rbase = static_cast<int64_t>(it.u) * a.N;
+                const int64_t cbase = static_cast<int64_t>(it.u) * a.NP;
+#pragma unroll
+                for (int k = 0; k < kBM / 64; ++k) {
+                    const int rl = k * 64 + (warp - 2) * 32 + lane;
+                    const int row = it.rb * kPM + static_cast<int>(rank) * kBM + rl;
+                    const float4* X = sX + xb * kGroups * kBM + rl;
+                    float4 o = X[0];
+                    int c0 = __float_as_int(o.y), c1 = __float_as_int(o.w);
+#pragma unroll
+                    for (int g = 1; g < kGroups; ++g) {
+                        const float4 n = X[g * kBM];
+                        if (kCount) {
+                            o.x += n.x;
+                            continue;
+                        }
+                        const int nc0 = __float_as_int(n.y), nc1 = __float_as_int(n.w);
+                        if (nc0 >= 0 && (c0 < 0 || n.x > o.x || (n.x == o.x && nc0 < c0))) {
+                            o.x = n.x;
+                            c0 = nc0;
+                        }
+                        if (nc1 >= 0 && (c1 < 0 || n.z > o.z || (n.z == o.z && nc1 < c1))) {
+                            o.z = n.z;
+                            c1 = nc1;
+                        }
+                    }
+                    if (row >= a.N) continue;
+                    if (kCount) {
+                        a.out_count[rbase + row] = __float2int_rn(o.x);
+                    } else if (kSym) {
+                        // the row direction's best joins the column maxima of earlier row
+                        // blocks in the row's slot: value (low 5 bits cleared) then lowest
+                        // position
+                        if (c0 >= 0)
+                            atomicMax(a.slots + rbase + row,
+                                      (static_cast<unsigned long long>(__float_as_uint(o.x) &
+                                                                       0xFFFFFFE0u) << 32) |
+                                          (0xFFFFFFFFull - static_cast<uint32_t>(c0)));
+                    } else {
+                        a.out_t0[rbase + row] =
+                            c0 < 0 ? -1 : (a.repair_mode ? a.colpos[cbase + c0] : c0);
+                        if (a.repair_mode && a.need_all)
+                            a.out_t1[rbase + row] = c1 < 0 ? -1 : a.colpos[cbase + c1];
+                    }
+                }
+                mbar_arrive(&x_empty[xb]);
+            }
+            __syncwarp();
         }
-        __syncwarp();
+        // Neither CTA frees its tensor memory or exits while the pair's MMAs, commits or
+        // arrivals can still reach it.  (The epilogue ends with its own copy of the barrier:
+        // with a common end, the compiler spills what lives across its tile loop.)
+        tc_fence_before();
+        cluster_barrier();
+        tc_fence_after();
+        if (warp == 1) tmem_dealloc<2>(*tmem_slot, kTmemCols);
     } else {
         // ------------------------------------------------------------ epilogue
-        const int ew = warp - 2;
+        setmaxnreg_inc<C::EPI_REGS>();
+        const int ew = warp - kHelperWarps;
         const int h = ew >> 2;            // column group of the tile
         const int q = warp & 3;           // TMEM lane quarter this warp may read
         const int row_local = q * 32 + lane;
@@ -641,45 +811,64 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         const int w = a.window;
         const uint32_t w2 = 2u * static_cast<uint32_t>(w);
         const uint32_t mask = a.mant_mask;
-        uint32_t ms = 0, mph = 0;    // meta ring slot and phase
-        uint32_t acc = 0, tph = 0;   // accumulator buffer and phase
+        const uint32_t slot = smem_u32(smem + C::OFF_BEST) +
+                              static_cast<uint32_t>((h * kBM + row_local) * kSlot);
+        const uint32_t release0 = cluster_addr(&t_empty[0], 0);
+        const uint32_t release1 = cluster_addr(&t_empty[1], 0);
+        const uint32_t m_full0 = smem_u32(m_full), t_full0 = smem_u32(t_full);
+        uint32_t n_t = 0;   // tiles seen: metadata slot n_t mod MSLOTS, accumulator n_t mod 2
         uint32_t n_x = 0;
         uint32_t n_c = 0;   // symmetric mode: tiles whose column maxima were merged
         bool ok = true;
-        for (int item = pair; item < n_items && ok; item += n_pairs) {
-            const int u = item / a.RB;
-            const int rb = item - u * a.RB;
-            const Tiles ut = unit_tiles<kSym>(a, u, rb);
+        // the coming tile's metadata and accumulator were seen complete (tested while the
+        // tile before it was reduced, so that the test's latency is hidden)
+        uint32_t ready = 0;
+        // Column counts at the ends of the window band [r0 - w, r0 + 128 + w) of a row block
+        // (repair mode), loaded one item ahead like its retained count.
+        auto band_counts = [&](int bu, int brb, int bkb, int& clo, int& chi) {
+            const int b0r = brb * kPM + static_cast<int>(rank) * kBM;
+            const int lo = max(b0r - w, 0), hi = min(b0r + kBM + w, a.N);
+            const int* cnt = a.cnt + static_cast<int64_t>(bu) * a.N;
+            clo = lo < a.N ? cnt[lo] : bkb;
+            chi = hi < a.N ? cnt[hi] : bkb;
+        };
+        Items<kSym> it(a, pair);
+        int clo = 0, chi = 0, nclo = 0, nchi = 0;
+        if (a.repair_mode && it.item < n_items) band_counts(it.u, it.rb, it.kb, clo, chi);
+        for (; it.item < n_items && ok; it.advance(n_pairs), clo = nclo, chi = nchi) {
+            const int u = it.u, rb = it.rb;
+            const Tiles ut = it.tiles(a);
             const int nt = ut.tr + ut.te;
             const int r0 = rb * kPM + static_cast<int>(rank) * kBM;
             const int row = r0 + row_local;
+            it.prefetch(a, n_pairs);
             // symmetric mode: the row's own column scale (the value of row j's candidate
             // i is x_ij s_i), and whether this row block runs past the end of the unit
             const bool row_ok = row < a.N;
             const float si = (kSym && row_ok) ? a.colrinv[static_cast<int64_t>(u) * a.NP + row] : 0.f;
             const bool pad_item = r0 + kBM > a.N;
 
-            // Column ranges that meet the window band [r0 - w, r0 + 128 + w) of this
-            // row block: only tiles meeting them need the per-element window test.
+            // Column ranges that meet the window band of this row block: only tiles meeting
+            // them need the per-element window test.  A group's columns [c_lo, c_lo + GW)
+            // meet [s, e) when c_lo - (s - GW + 1), as unsigned, is below e - s + GW - 1.
             const int lo = max(r0 - w, 0);
             const int hi = min(r0 + kBM + w, a.N);
-            int s0a, s0b, s1a = 0, s1b = 0;
+            int s0a, s1a = 0;
+            uint32_t s0n, s1n = 0;
             if (!a.repair_mode) {
-                s0a = lo;
-                s0b = hi;
+                s0a = lo - (kGW - 1);
+                s0n = hi > lo ? hi - lo + kGW - 1 : 0;
             } else {
-                const int kb = a.kb[u];
-                const int* cnt = a.cnt + static_cast<int64_t>(u) * a.N;
-                const int clo = lo < a.N ? cnt[lo] : kb;
-                const int chi = hi < a.N ? cnt[hi] : kb;
-                const int kpad = ut.tr * kBN;
-                s0a = clo;
-                s0b = chi;
-                s1a = kpad + lo - clo;
-                s1b = kpad + hi - chi;
+                const int nlo = lo - clo, nhi = hi - chi;   // evicted before each end
+                s0a = clo - (kGW - 1);
+                s0n = chi > clo ? chi - clo + kGW - 1 : 0;
+                s1a = ut.tr * kBN + nlo - (kGW - 1);
+                s1n = nhi > nlo ? nhi - nlo + kGW - 1 : 0;
+                if (it.item + n_pairs < n_items) band_counts(it.nu, it.nrb, it.nkb, nclo, nchi);
             }
 
             Best b0{-INFINITY, -1}, b1{-INFINITY, -1};   // retained (or all) / evicted
+            Best best = b0;                              // of the segment at hand
             const int rw = row - w;
 
             float cnt = 0.f;                               // count mode: r_i so far
@@ -689,56 +878,64 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                        (a.colrinv[static_cast<int64_t>(u) * a.NP + row] * (1.0f / kCountScale))) *
                       kCountScale;
             for (int t = 0; t < nt; ++t) {
-                ok = all_wait(&m_full[ms], mph, wc, 7);
-                if (ok) ok = all_wait(&t_full[acc], tph, wc, 8);
-                if (!ok) break;
+                const uint32_t ms = n_t % C::MSLOTS, acc = n_t & 1u;
+                if (!__all_sync(0xFFFFFFFFu, ready != 0u)) {
+                    ok = all_wait(&m_full[ms], (n_t / C::MSLOTS) & 1u, wc, 7);
+                    if (ok) ok = all_wait(&t_full[acc], (n_t >> 1) & 1u, wc, 8);
+                    if (!ok) break;
+                }
+                ++n_t;
                 tc_fence_after();
                 const float* rinv = reinterpret_cast<const float*>(sMeta + ms * C::META) + h * kGW;
                 const int* pos =
                     reinterpret_cast<const int*>(sMeta + ms * C::META + kBN * 4) + h * kGW;
                 const int c_lo = (ut.t0 + t) * kBN + h * kGW;
-                const bool band = (c_lo < s0b && c_lo + kGW > s0a) ||
-                                  (c_lo < s1b && c_lo + kGW > s1a);
+                const bool band = static_cast<uint32_t>(c_lo - s0a) < s0n ||
+                                  static_cast<uint32_t>(c_lo - s1a) < s1n;
                 const uint32_t taddr = tmem + lane_base + acc * kBN + static_cast<uint32_t>(h * kGW);
-                uint32_t x0[32], x1[32], x2[32], x3[32];
-                load_group(taddr, x0, x1, x2, x3);
+                auto test_next = [&]() {
+                    ready = mbar_test2(m_full0 + 8u * (n_t % C::MSLOTS), (n_t / C::MSLOTS) & 1u,
+                                       t_full0 + 8u * (n_t & 1u), (n_t >> 1) & 1u);
+                };
+                uint32_t x[kCh][32];
+                load_group(taddr, x);
                 // The tile is in registers: hand the accumulator back to the MMA warp now,
                 // so it can compute the next-but-one tile while this one is reduced.
                 tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive_cluster(cluster_addr(&t_empty[acc], 0));
-                if (kSym) {
+                if (lane == 0) mbar_arrive_cluster(acc ? release1 : release0);
+                if constexpr (kSym) {
+                    ready = 0;
                     // row maxima (the eager fold: the column pass already costs more than
                     // the vote saves) and each chunk's column maxima over this warp's 32
                     // rows right after it (while its registers are live)
                     uint32_t cr[4];
                     if (band) {
-                        fold32<true, true>(x0, rinv, pos, rw, w2, mask, c_lo, b0);
-                        cr[0] = colpass32<true>(x0, pos, rw, w2, si, row_ok);
-                        fold32<true, true>(x1, rinv + 32, pos + 32, rw, w2, mask, c_lo + 32, b0);
-                        cr[1] = colpass32<true>(x1, pos + 32, rw, w2, si, row_ok);
-                        fold32<true, true>(x2, rinv + 64, pos + 64, rw, w2, mask, c_lo + 64, b0);
-                        cr[2] = colpass32<true>(x2, pos + 64, rw, w2, si, row_ok);
-                        fold32<true, true>(x3, rinv + 96, pos + 96, rw, w2, mask, c_lo + 96, b0);
-                        cr[3] = colpass32<true>(x3, pos + 96, rw, w2, si, row_ok);
+                        fold32_packed<true>(x[0], rinv, pos, rw, w2, mask, c_lo, b0);
+                        cr[0] = colpass32<true>(x[0], pos, rw, w2, si, row_ok);
+                        fold32_packed<true>(x[1], rinv + 32, pos + 32, rw, w2, mask, c_lo + 32, b0);
+                        cr[1] = colpass32<true>(x[1], pos + 32, rw, w2, si, row_ok);
+                        fold32_packed<true>(x[2], rinv + 64, pos + 64, rw, w2, mask, c_lo + 64, b0);
+                        cr[2] = colpass32<true>(x[2], pos + 64, rw, w2, si, row_ok);
+                        fold32_packed<true>(x[3], rinv + 96, pos + 96, rw, w2, mask, c_lo + 96, b0);
+                        cr[3] = colpass32<true>(x[3], pos + 96, rw, w2, si, row_ok);
                     } else if (pad_item) {
-                        fold32<false, true>(x0, rinv, pos, rw, w2, mask, c_lo, b0);
-                        cr[0] = colpass32<true>(x0, pos, rw, w2, si, row_ok);
-                        fold32<false, true>(x1, rinv + 32, pos + 32, rw, w2, mask, c_lo + 32, b0);
-                        cr[1] = colpass32<true>(x1, pos + 32, rw, w2, si, row_ok);
-                        fold32<false, true>(x2, rinv + 64, pos + 64, rw, w2, mask, c_lo + 64, b0);
-                        cr[2] = colpass32<true>(x2, pos + 64, rw, w2, si, row_ok);
-                        fold32<false, true>(x3, rinv + 96, pos + 96, rw, w2, mask, c_lo + 96, b0);
-                        cr[3] = colpass32<true>(x3, pos + 96, rw, w2, si, row_ok);
+                        fold32_packed<false>(x[0], rinv, pos, rw, w2, mask, c_lo, b0);
+                        cr[0] = colpass32<true>(x[0], pos, rw, w2, si, row_ok);
+                        fold32_packed<false>(x[1], rinv + 32, pos + 32, rw, w2, mask, c_lo + 32, b0);
+                        cr[1] = colpass32<true>(x[1], pos + 32, rw, w2, si, row_ok);
+                        fold32_packed<false>(x[2], rinv + 64, pos + 64, rw, w2, mask, c_lo + 64, b0);
+                        cr[2] = colpass32<true>(x[2], pos + 64, rw, w2, si, row_ok);
+                        fold32_packed<false>(x[3], rinv + 96, pos + 96, rw, w2, mask, c_lo + 96, b0);
+                        cr[3] = colpass32<true>(x[3], pos + 96, rw, w2, si, row_ok);
                     } else {
-                        fold32<false, true>(x0, rinv, pos, rw, w2, mask, c_lo, b0);
-                        cr[0] = colpass32<false>(x0, pos, rw, w2, si, row_ok);
-                        fold32<false, true>(x1, rinv + 32, pos + 32, rw, w2, mask, c_lo + 32, b0);
-                        cr[1] = colpass32<false>(x1, pos + 32, rw, w2, si, row_ok);
-                        fold32<false, true>(x2, rinv + 64, pos + 64, rw, w2, mask, c_lo + 64, b0);
-                        cr[2] = colpass32<false>(x2, pos + 64, rw, w2, si, row_ok);
-                        fold32<false, true>(x3, rinv + 96, pos + 96, rw, w2, mask, c_lo + 96, b0);
-                        cr[3] = colpass32<false>(x3, pos + 96, rw, w2, si, row_ok);
+                        fold32_packed<false>(x[0], rinv, pos, rw, w2, mask, c_lo, b0);
+                        cr[0] = colpass32<false>(x[0], pos, rw, w2, si, row_ok);
+                        fold32_packed<false>(x[1], rinv + 32, pos + 32, rw, w2, mask, c_lo + 32, b0);
+                        cr[1] = colpass32<false>(x[1], pos + 32, rw, w2, si, row_ok);
+                        fold32_packed<false>(x[2], rinv + 64, pos + 64, rw, w2, mask, c_lo + 64, b0);
+                        cr[2] = colpass32<false>(x[2], pos + 64, rw, w2, si, row_ok);
+                        fold32_packed<false>(x[3], rinv + 96, pos + 96, rw, w2, mask, c_lo + 96, b0);
+                        cr[3] = colpass32<false>(x[3], pos + 96, rw, w2, si, row_ok);
                     }
                     // merge the four lane quarters of this group: the warps exchange their
                     // 128 column maxima, then warp q takes columns 32q .. 32q + 31
@@ -768,103 +965,54 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                                   (static_cast<unsigned long long>(best & 0xFFFFFFE0u) << 32) |
                                       (0xFFFFFFFFull - win));
                     }
-                } else if (kCount) {
-                    cnt += band ? count_group<true>(x0, x1, x2, x3, rinv, pos, rw, w2, thr)
-                                : count_group<false>(x0, x1, x2, x3, rinv, pos, rw, w2, thr);
-                } else if (t < ut.tr) {
-                    reduce_tile<eager_fold<D>()>(band, x0, x1, x2, x3, rinv, pos, rw, w2, mask,
-                                                 c_lo, b0);
+                } else if constexpr (kCount) {
+                    cnt += band ? count_group<true>(x, rinv, pos, rw, w2, thr)
+                                : count_group<false>(x, rinv, pos, rw, w2, thr);
+                    test_next();
                 } else {
                     if (t == ut.tr) {
                         // The evicted segment matters only where it reaches the retained
                         // one: start its running best just below this group's retained
                         // best (exact similarities decide between the two later; the
                         // FLT_MIN keeps an exact tie at 0 in play).
-                        b1.v = b0.v - (fabsf(b0.v) * 0x1p-13f + FLT_MIN);
+                        if constexpr (!kPacked) resolve_best(slot, mask, best);
+                        b0 = best;
+                        best = Best{b0.v - (fabsf(b0.v) * 0x1p-13f + FLT_MIN), -1};
                     }
-                    reduce_tile<eager_fold<D>()>(band, x0, x1, x2, x3, rinv, pos, rw, w2, mask,
-                                                 c_lo, b1);
+                    if constexpr (kPacked) {
+                        if (band) fold_packed<true>(x, rinv, pos, rw, w2, mask, c_lo, best);
+                        else fold_packed<false>(x, rinv, pos, rw, w2, mask, c_lo, best);
+                        test_next();
+                    } else {
+                        float v[kCh][32], m[kCh];
+                        if (band) scale_group<true>(x, rinv, pos, rw, w2, v, m);
+                        else scale_group<false>(x, rinv, pos, rw, w2, v, m);
+                        test_next();
+                        keep_best(v, m, c_lo, slot, best);
+                    }
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&m_empty[ms]);
-                if (++ms == C::MSLOTS) {
-                    ms = 0;
-                    mph ^= 1;
-                }
-                acc ^= 1;
-                tph ^= acc == 0 ? 1u : 0u;
             }
             if (!ok) break;
-            const float bv0 = b0.v, bv1 = b1.v;
-            const int bc0 = b0.col, bc1 = b1.col;
-
-            // Merge the column groups of every row through shared memory: groups
-            // 1.. hand their (value, column) pairs to group 0.
-            const int xb = static_cast<int>(n_x & 1);
-            float4* X = sX + xb * (kGroups - 1) * kBM;
-            if (h != 0) {
-                ok = all_wait(&x_empty[xb], ((n_x >> 1) & 1) ^ 1, wc, 9);
-                if (!ok) break;
-                X[(h - 1) * kBM + row_local] =
-                    kCount ? make_float4(cnt, 0.f, 0.f, 0.f)
-                           : make_float4(bv0, __int_as_float(bc0), bv1, __int_as_float(bc1));
-                mbar_arrive(&x_full[xb]);
-            } else if (kCount) {
-                ok = all_wait(&x_full[xb], (n_x >> 1) & 1, wc, 10);
-                if (!ok) break;
-                float total = cnt;
-#pragma unroll
-                for (int g = 1; g < kGroups; ++g) total += X[(g - 1) * kBM + row_local].x;
-                mbar_arrive(&x_empty[xb]);
-                if (row < a.N)
-                    a.out_count[static_cast<int64_t>(u) * a.N + row] = __float2int_rn(total);
-            } else {
-                ok = all_wait(&x_full[xb], (n_x >> 1) & 1, wc, 10);
-                if (!ok) break;
-                float v0 = bv0, v1 = bv1;
-                int c0 = bc0, c1 = bc1;
-#pragma unroll
-                for (int g = 1; g < kGroups; ++g) {
-                    const float4 o = X[(g - 1) * kBM + row_local];
-                    const int oc0 = __float_as_int(o.y), oc1 = __float_as_int(o.w);
-                    if (oc0 >= 0 && (c0 < 0 || o.x > v0 || (o.x == v0 && oc0 < c0))) {
-                        v0 = o.x;
-                        c0 = oc0;
-                    }
-                    if (oc1 >= 0 && (c1 < 0 || o.z > v1 || (o.z == v1 && oc1 < c1))) {
-                        v1 = o.z;
-                        c1 = oc1;
-                    }
-                }
-                mbar_arrive(&x_empty[xb]);
-                if (kSym) {
-                    // the row direction's best joins the column maxima of earlier row
-                    // blocks in the row's slot: value (low 5 bits cleared) then lowest
-                    // position
-                    if (row < a.N && c0 >= 0)
-                        atomicMax(a.slots + static_cast<int64_t>(u) * a.N + row,
-                                  (static_cast<unsigned long long>(__float_as_uint(v0) &
-                                                                   0xFFFFFFE0u) << 32) |
-                                      (0xFFFFFFFFull - static_cast<uint32_t>(c0)));
-                } else if (row < a.N) {
-                    const int64_t o_idx = static_cast<int64_t>(u) * a.N + row;
-                    const int64_t cbase = static_cast<int64_t>(u) * a.NP;
-                    const int p0 = c0 < 0 ? -1 : (a.repair_mode ? a.colpos[cbase + c0] : c0);
-                    a.out_t0[o_idx] = p0;
-                    if (a.repair_mode && a.need_all)
-                        a.out_t1[o_idx] = c1 < 0 ? -1 : a.colpos[cbase + c1];
-                }
+            if constexpr (!kCount && !kSym) {
+                if constexpr (!kPacked) resolve_best(slot, mask, best);
+                if (nt > ut.tr) b1 = best;
+                else b0 = best;
             }
+            // Every row's (value, column) pairs go to the merging warps.
+            const int xb = static_cast<int>(n_x & 1);
+            ok = all_wait(&x_empty[xb], ((n_x >> 1) & 1) ^ 1, wc, 9);
+            if (!ok) break;
+            sX[(xb * kGroups + h) * kBM + row_local] =
+                kCount ? make_float4(cnt, 0.f, 0.f, 0.f)
+                       : make_float4(b0.v, __int_as_float(b0.col), b1.v, __int_as_float(b1.col));
+            mbar_arrive(&x_full[xb]);
             ++n_x;
         }
+        tc_fence_before();
+        cluster_barrier();
     }
-
-    // Neither CTA frees its tensor memory or exits while the pair's MMAs, commits or
-    // arrivals can still reach it.
-    tc_fence_before();
-    cluster_barrier();
-    tc_fence_after();
-    if (warp == 1) tmem_dealloc<2>(tmem, kTmemCols);
 }
 
 }  // namespace
@@ -878,7 +1026,17 @@ template <int D, bool kCount, bool kSym>
 cudaError_t launch_audit_t(const CUtensorMap& tmA, const CUtensorMap& tmB, const AuditArgs& a,
                            int grid, cudaStream_t st)
 {
-    const int bytes = AuditCfg<D, kSym>::BYTES;
+    const int bytes = AuditCfg<D, kCount, kSym>::BYTES;
+    // The warpgroups' shares after setmaxnreg add up to the launch's registers: with fewer
+    // than kLaunchRegs per thread the second share would never be granted.
+    static std::atomic<int> regs{0};   // a property of the build; 0: not asked yet
+    if (regs.load(std::memory_order_relaxed) == 0) {
+        cudaFuncAttributes f;
+        const cudaError_t q = cudaFuncGetAttributes(&f, audit_kernel<D, kCount, kSym>);
+        if (q != cudaSuccess) return q;
+        regs.store(f.numRegs, std::memory_order_relaxed);
+    }
+    if (regs.load(std::memory_order_relaxed) < kLaunchRegs) return cudaErrorInvalidConfiguration;
     cudaError_t e = cudaFuncSetAttribute(audit_kernel<D, kCount, kSym>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e != cudaSuccess) return e;
