@@ -76,9 +76,8 @@ struct RepairArgs {
     int cluster;                // literal variant: CTAs per unit (1, 2, 4, 8 or 16)
 };
 
-// CTAs per unit of the literal repair's selection: the largest power of two that keeps
-// all units in one wave of two CTAs per SM, slices of at least 256 positions, at most
-// 16.
+// CTAs per unit of the literal repair's selection: a power of two up to 8 (see the
+// definition for where the lines lie).
 int select_cluster_size(int U, int N, int sms);
 
 // The count mode's column scales are 1/||k|| times this power of two: one saturated

@@ -11,10 +11,11 @@
 //   orphan k); a unit whose mask has a byte > 1 or whose popcount differs from its
 //   budget gets status, nswaps = -1 and S1 = S0.
 //
-// The literal rule (select_kernel<C>) runs each unit on a cluster of C CTAs (C = 1, 2,
-// 4, 8 or 16, chosen so that every SM has work): see "cluster selection" below.  Its
-// scratch is caller workspace ([U][N] keys and positions, twice) and 48 KB of dynamic
-// shared memory per CTA.
+// The literal rule (select_kernel<C>) runs each unit on a cluster of C CTAs (C = 1 to 8 by
+// select_cluster_size; 16 can be forced): by buckets in shared memory where the swap list
+// fits (see "bucket path" below), else by a radix select and sorts over the workspace
+// ("cluster selection").  Its scratch is caller workspace ([U][N] keys and positions,
+// twice) and 72 KB of dynamic shared memory per CTA.
 //
 // Dedup variant (dedup_kernel, given the twin of every position; one 512-thread block
 // per unit): evicting a donor keeps its twin, so a twin pair never loses both members.
@@ -31,6 +32,7 @@
 #include <cooperative_groups.h>
 
 #include "twk_internal.h"
+#include "twk_ptx.cuh"
 
 namespace twk {
 namespace {
@@ -493,7 +495,9 @@ __device__ __forceinline__ T* peer(T* p, int rank)
 }
 
 struct ClusterShared {
-    int cnt[4];          // this CTA's orphans, donors, retained count, invalid-byte flag
+    int cnt[8];          // this CTA's orphans, donors, retained count, invalid-byte flag;
+                         // bucket path: smallest and largest orphan, then donor, as_int order
+    int all[8];          // bucket path: the same over the cluster
     int lcnt[2];         // compaction: this CTA's items below the cut and at it
     int hist[2][256];    // this CTA's digit histogram, alternating between passes
     int tot[8];          // cluster-wide values derived by thread 0
@@ -572,6 +576,350 @@ __host__ __device__ inline int slice_len(int N, int C)
     return (q + kEA - 1) / kEA * kEA;
 }
 
+// ---- bucket path -------------------------------------------------------------------
+//
+// The usual case of the selection: no list is written to memory and nothing is sorted by
+// comparisons across the CTA.  Three passes read the slice's b and mask (coalesced, in any
+// order):
+//   1. S1 = S0, the counts, and the smallest and largest b of each side;
+//   2. a histogram of each side over kBk equal intervals of its range, summed over the
+//      cluster; its prefix sums give every bucket's first rank.  Buckets whose first rank
+//      is below m hold the m most severe items (and the rest of the bucket at the cut);
+//   3. their items go to the bucket's place in the shared memory of the CTA that owns the
+//      bucket (buckets are dealt out by first rank, so that each CTA gets about 1/C).
+// An item's rank is its bucket's first rank plus the number of items of its bucket ordered
+// before it, counted one by one.  The intervals are taken on b rounded toward zero to fp32,
+// which keeps the order, so the ranks are those of the (key, position) order whatever the
+// values.  Where the shares would not fit in shared memory or a bucket is too full to count
+// through (many equal values), the general path below does the whole unit instead.
+// Why: the selection is bound by latency, the round trips of its passes and barriers.  The
+// general path's radix select takes up to eight passes over lists in memory with several
+// block barriers each, and its bitonic sort was 58 of 182 thousand cycles per unit at 16384
+// positions.  General -> buckets, with the cluster size each was given: 288 units of 16384
+// positions 120 -> 60 us, 8 of 8192 67 -> 22, 8 of 4096 57 -> 17, 8 of 131072 295 -> 82,
+// 128 of 8192 64 -> 25.
+constexpr int kBk = 1024;      // buckets per side
+constexpr int kCap = 3072;     // items per side a CTA holds (36 KB): two CTAs per SM fit
+constexpr int kMaxBucket = 256;
+
+// A float's bits as an int with the float's order.
+__device__ __forceinline__ int as_int(float f)
+{
+    const int i = __float_as_int(f);
+    return i ^ ((i >> 31) & 0x7FFFFFFF);
+}
+__device__ __forceinline__ float from_int(int i)
+{
+    return __int_as_float(i ^ ((i >> 31) & 0x7FFFFFFF));
+}
+
+// A double's bits (not a NaN's) as an fp32 value, rounded toward zero: monotone, in integer
+// operations.  Beyond fp32's range it is 0 or the largest fp32 value.
+__device__ __forceinline__ float narrow(uint64_t u)
+{
+    const uint32_t hi = static_cast<uint32_t>(u >> 32), lo = static_cast<uint32_t>(u);
+    const int e = static_cast<int>((hi >> 20) & 0x7FFu) - 896;
+    const uint32_t mant = ((hi & 0xFFFFFu) << 3) | (lo >> 29);
+    const uint32_t mag = e <= 0 ? 0u : e >= 255 ? 0x7F7FFFFFu : (static_cast<uint32_t>(e) << 23) | mant;
+    return __uint_as_float((hi & 0x80000000u) | mag);
+}
+
+// Bucket of a value in [lo, lo + (kBk - 1) / scale]; non-decreasing in f.  (A range too wide
+// for fp32 has scale 0, and every value falls into bucket 0.)
+__device__ __forceinline__ int bucket_of(float f, float lo, float scale)
+{
+    return min(kBk - 1, max(0, static_cast<int>((f - lo) * scale)));
+}
+
+// The b whose severity key (side 0: orphans, 1: donors) is k, as the double's bits.
+__device__ __forceinline__ uint64_t bits_of_key(uint64_t k, int side)
+{
+    const uint64_t o = side ? ~k : k;
+    return (o >> 63) ? (o & 0x7FFFFFFFFFFFFFFFull) : ~o;
+}
+
+// What a position is: 0 an orphan, 1 a donor, 2 neither.
+__device__ __forceinline__ int side_of(uint32_t m, double bi, uint64_t ki, int i,
+                                       const RepairArgs& a, uint64_t ktau)
+{
+    if (is_nan_bits(bi)) return 2;
+    if (m == 0u) return ki < ktau ? 0 : 2;
+    const bool prot = i < a.n_sink || i >= a.N - a.n_recent;
+    return !prot && ki >= ktau ? 1 : 2;
+}
+
+// Accesses to the same shared-memory object in CTA `rank` of the cluster, by 32-bit
+// shared::cluster addresses (generic pointers made the kernel spill).
+__device__ __forceinline__ int peer_add(int* p, int rank, int v)
+{
+    int old;
+    asm volatile("atom.relaxed.cluster.shared::cluster.add.s32 %0, [%1], %2;"
+                 : "=r"(old)
+                 : "r"(cluster_addr(p, static_cast<uint32_t>(rank))), "r"(v)
+                 : "memory");
+    return old;
+}
+__device__ __forceinline__ void peer_store(uint64_t* p, int rank, uint64_t v)
+{
+    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(
+                     cluster_addr(p, static_cast<uint32_t>(rank))),
+                 "l"(v)
+                 : "memory");
+}
+__device__ __forceinline__ void peer_store(int* p, int rank, int v)
+{
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(
+                     cluster_addr(p, static_cast<uint32_t>(rank))),
+                 "r"(v)
+                 : "memory");
+}
+
+// Runs the unit by buckets; every thread of the cluster calls it.  False (and, apart from
+// S1 = S0, nothing written) where the unit is left to the general path.
+template <int C>
+__device__ bool select_by_buckets(Shared& s, ClusterShared& cs, uint64_t* sk, int* si,
+                                  const RepairArgs& a, int u, int r)
+{
+    const int64_t off = static_cast<int64_t>(u) * a.N;
+    const uint8_t* S0 = a.mask + off;
+    const double* b = a.b + off;
+    uint8_t* S1 = a.out_mask + off;
+    const int slice = slice_len(a.N, C);
+    const int lo = min(a.N, r * slice), hi = min(a.N, lo + slice);
+    const uint64_t ktau = ordered(a.tau);
+    constexpr int kP = C == 1 ? 8 : 4;   // positions per thread and step
+    const int tid = threadIdx.x, lane = tid & 31;
+    int* base = &s.warp_cnt[0][0];   // [2][kBk] first rank of each bucket
+    int* cur = base + 2 * kBk;       // [2][kBk] counts, then the next free place
+    static_assert(sizeof(s.warp_cnt) == 4 * kBk * sizeof(int), "bucket arrays fill warp_cnt");
+
+    // the thread's kP positions of one step: c0 + tid, + kT, ...
+    auto load = [&](int c0, uint32_t (&mv)[kP], double (&bv)[kP]) {
+#pragma unroll
+        for (int j = 0; j < kP; ++j) {
+            const int i = c0 + j * kT + tid;
+            mv[j] = i < hi ? S0[i] : 255u;
+            bv[j] = i < hi ? b[i] : 0.0;
+        }
+    };
+
+    // 1. counts and ranges
+    int bad = 0, cnt = 0, n[2] = {0, 0};
+    int mn[2] = {0x7FFFFFFF, 0x7FFFFFFF}, mx[2] = {-0x7FFFFFFF - 1, -0x7FFFFFFF - 1};
+    for (int c0 = lo; c0 < hi; c0 += kT * kP) {
+        uint32_t mv[kP];
+        double bv[kP];
+        load(c0, mv, bv);
+#pragma unroll
+        for (int j = 0; j < kP; ++j) {
+            const int i = c0 + j * kT + tid;
+            if (i >= hi) continue;
+            S1[i] = static_cast<uint8_t>(mv[j]);
+            bad |= mv[j] > 1u;
+            cnt += mv[j] != 0u;
+            const int x = side_of(mv[j], bv[j], ordered(bv[j]), i, a, ktau);
+            const int f = as_int(narrow(static_cast<uint64_t>(__double_as_longlong(bv[j]))));
+#pragma unroll
+            for (int y = 0; y < 2; ++y) {
+                n[y] += x == y;
+                mn[y] = x == y ? min(mn[y], f) : mn[y];
+                mx[y] = x == y ? max(mx[y], f) : mx[y];
+            }
+        }
+    }
+    if (tid < 8) cs.cnt[tid] = tid < 4 ? 0 : (tid & 1) ? -0x7FFFFFFF - 1 : 0x7FFFFFFF;
+    for (int i = tid; i < 2 * kBk; i += kT) cur[i] = 0;
+    __syncthreads();
+    bad = __reduce_or_sync(0xFFFFFFFFu, bad);
+    cnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
+#pragma unroll
+    for (int y = 0; y < 2; ++y) {
+        n[y] = __reduce_add_sync(0xFFFFFFFFu, n[y]);
+        mn[y] = __reduce_min_sync(0xFFFFFFFFu, mn[y]);
+        mx[y] = __reduce_max_sync(0xFFFFFFFFu, mx[y]);
+    }
+    if (lane == 0) {
+        atomicAdd(&cs.cnt[0], n[0]);
+        atomicAdd(&cs.cnt[1], n[1]);
+        atomicAdd(&cs.cnt[2], cnt);
+        atomicOr(&cs.cnt[3], bad);
+#pragma unroll
+        for (int y = 0; y < 2; ++y) {
+            atomicMin(&cs.cnt[4 + 2 * y], mn[y]);
+            atomicMax(&cs.cnt[5 + 2 * y], mx[y]);
+        }
+    }
+    cluster_sync<C>();
+    if (tid < 8) {   // totals and ranges over the cluster, identical in every CTA
+        const bool mini = tid == 4 || tid == 6, maxi = tid == 5 || tid == 7;
+        int v = mini ? 0x7FFFFFFF : maxi ? -0x7FFFFFFF - 1 : 0;
+        for (int q = 0; q < C; ++q) {
+            const int* rc = peer<C>(cs.cnt, q);   // cnt[4], then ends[4]
+            const int x = rc[tid];
+            v = mini ? min(v, x) : maxi ? max(v, x) : tid == 3 ? v | x : v + x;
+        }
+        cs.all[tid] = v;
+    }
+    __syncthreads();
+    const int* tot = cs.all;
+    const int* ends = cs.all + 4;
+    int status = 0;
+    if (tot[3]) status = 1;                                  // TWINKV_ERR_INVALID_ARG
+    else if (a.budget && a.budget[u] != tot[2]) status = 3;  // TWINKV_ERR_BUDGET
+    const int m = status ? 0 : min(tot[0], tot[1]);
+    if (m == 0) {
+        cluster_sync<C>();   // every CTA has read the counts before any CTA exits
+        if (r == 0 && tid == 0) {
+            a.out_nswaps[u] = status ? -1 : 0;
+            if (a.out_status) a.out_status[u] = status;
+        }
+        return true;
+    }
+    float from[2], scale[2];
+#pragma unroll
+    for (int y = 0; y < 2; ++y) {
+        from[y] = from_int(ends[2 * y]);
+        const float w = from_int(ends[2 * y + 1]) - from[y];
+        scale[y] = w > 0.f && w <= 3.4e38f ? (kBk - 1) / w : 0.f;
+        if (!(scale[y] <= 3.4e38f)) scale[y] = 0.f;
+    }
+    // side x's bucket, most severe first (donors from the largest b down)
+    auto bucket = [&](int x, uint64_t bits) {
+        const int k = bucket_of(narrow(bits), x ? from[1] : from[0], x ? scale[1] : scale[0]);
+        return x ? kBk - 1 - k : k;
+    };
+
+    // 2. histogram, summed over the cluster, and its prefix sums
+    for (int c0 = lo; c0 < hi; c0 += kT * kP) {
+        uint32_t mv[kP];
+        double bv[kP];
+        load(c0, mv, bv);
+#pragma unroll
+        for (int j = 0; j < kP; ++j) {
+            const int i = c0 + j * kT + tid;
+            const int x = i < hi ? side_of(mv[j], bv[j], ordered(bv[j]), i, a, ktau) : 2;
+            if (x < 2)
+                atomicAdd(&cur[x * kBk + bucket(x, static_cast<uint64_t>(
+                                                       __double_as_longlong(bv[j])))],
+                          1);
+        }
+    }
+    // maxima, then minima (beyond every place, yet far from overflow for a CTA without items)
+    if (tid < 8) cs.tot[tid] = (tid & 4) ? 1 << 30 : 0;
+    if (tid == 0) s.sel_digit = s.sel_before = 0;
+    cluster_sync<C>();
+    constexpr int kPer = 2 * kBk / kT;   // buckets per thread; side 0: the lower half of the block
+    static_assert(kPer * kT == 2 * kBk && kW % 2 == 0, "whole warps per side");
+    const int b0 = tid * kPer, side = b0 / kBk;
+    int c[kPer], sum = 0;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        c[k] = 0;
+#pragma unroll 1
+        for (int q = 0; q < C; ++q) c[k] += peer<C>(cur, q)[b0 + k];
+        sum += c[k];
+    }
+    int incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) s.wsum[0][tid >> 5] = incl;
+    cluster_sync<C>();   // (every CTA has read this one's counts)
+    int run = incl - sum;
+    for (int w = side * (kW / 2); w < (tid >> 5); ++w) run += s.wsum[0][w];
+    int full = 0, last = 0;   // the fullest bucket in play, and the end of the last one
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        base[b0 + k] = run;
+        cur[b0 + k] = run;
+        if (run < m) {
+            full = max(full, c[k]);
+            last = max(last, run + c[k]);
+        }
+        run += c[k];
+    }
+    atomicMax(&cs.tot[0], full);
+    atomicMax(&cs.tot[1 + side], last);
+    cluster_sync<C>();
+    full = cs.tot[0];
+    const int end[2] = {cs.tot[1], cs.tot[2]};   // items in play per side
+    const int share = (max(end[0], end[1]) + C - 1) / C;
+    if (full > kMaxBucket || share + full > kCap) return false;   // alike in every CTA
+
+    // 3. the items in play to their buckets' owners
+    for (int c0 = lo; c0 < hi; c0 += kT * kP) {
+        uint32_t mv[kP];
+        double bv[kP];
+        load(c0, mv, bv);
+#pragma unroll
+        for (int j = 0; j < kP; ++j) {
+            const int i = c0 + j * kT + tid;
+            const uint64_t ki = ordered(bv[j]);
+            const int x = i < hi ? side_of(mv[j], bv[j], ki, i, a, ktau) : 2;
+            if (x == 2) continue;
+            const int k = x * kBk + bucket(x, static_cast<uint64_t>(__double_as_longlong(bv[j])));
+            if (base[k] >= m) continue;
+            const int t = C == 1 ? 0 : base[k] / share;
+            if constexpr (C == 1) {
+                const int at = x * kCap + atomicAdd(&cur[k], 1);
+                sk[at] = x ? ~ki : ki;
+                si[at] = i;
+            } else {
+                const int at = x * kCap + peer_add(cur + k, t, 1) % kCap;
+                peer_store(sk + at, t, x ? ~ki : ki);
+                peer_store(si + at, t, i);
+            }
+        }
+    }
+    // this CTA's own items: the places from its first bucket's to its last one's end
+    int g0[2] = {0, 0}, g1[2] = {end[0], end[1]};
+    if constexpr (C > 1) {
+#pragma unroll 1
+        for (int k = threadIdx.x; k < 2 * kBk; k += kT) {
+            const int x = k / kBk, bk = base[k];
+            const int ek = (k + 1) % kBk ? base[k + 1] : x ? tot[1] : tot[0];
+            if (ek > bk && bk < m && bk / share == r) {
+                atomicMin(&cs.tot[4 + x], bk);
+                atomicMax(x ? &s.sel_before : &s.sel_digit, ek);
+            }
+        }
+    }
+    cluster_sync<C>();
+    if constexpr (C > 1) {
+        g0[0] = cs.tot[4];
+        g0[1] = cs.tot[5];
+        g1[0] = s.sel_digit;
+        g1[1] = s.sel_before;
+    }
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        int* swaps = a.out_swaps + static_cast<int64_t>(u) * 2 * (a.N / 2);
+        for (int g = g0[x] + tid; g < g1[x]; g += kT) {
+            const uint64_t key = sk[x * kCap + g % kCap];
+            const int pos = si[x * kCap + g % kCap];
+            const int k = bucket(x, bits_of_key(key, x));
+            const int from_g = base[x * kBk + k];
+            const int to_g = k + 1 < kBk ? base[x * kBk + k + 1] : tot[x];
+            int rank = from_g;
+            for (int h = from_g; h < to_g; ++h) {
+                const int at = x * kCap + h % kCap;
+                rank += before(sk[at], si[at], key, pos) ? 1 : 0;
+            }
+            if (rank < m) {
+                swaps[2 * rank + (x ? 0 : 1)] = pos;
+                S1[pos] = x ? 0 : 1;
+            }
+        }
+    }
+    if (r == 0 && tid == 0) {
+        a.out_nswaps[u] = m;
+        if (a.out_status) a.out_status[u] = 0;
+    }
+    return true;
+}
+
 template <int C>
 __global__ void __launch_bounds__(kT, 2) select_kernel(const RepairArgs a)
 {
@@ -587,6 +935,10 @@ __global__ void __launch_bounds__(kT, 2) select_kernel(const RepairArgs a)
     int r = 0;
     if constexpr (C > 1) r = static_cast<int>(cg::this_cluster().block_rank());
     const int u = static_cast<int>(blockIdx.x / C);
+    if (select_by_buckets<C>(s, cs, sk_o, reinterpret_cast<int*>(sk_o + 2 * kCap), a, u, r))
+        return;
+    cluster_sync<C>();   // what the attempt left in shared memory is free
+
     const int N = a.N;
     const int64_t off = static_cast<int64_t>(u) * N;
     const uint8_t* S0 = a.mask + off;
@@ -1176,7 +1528,8 @@ template <int C>
 cudaError_t config_select(const RepairArgs& a, cudaStream_t st, cudaLaunchConfig_t& cfg,
                           cudaLaunchAttribute* at)
 {
-    const size_t bytes = 2 * static_cast<size_t>(kChunk) * 12;   // the two shares
+    const size_t bytes = 2 * static_cast<size_t>(kCap) * 12;   // the two sides' items
+    static_assert(kCap >= kChunk, "the general path's shares fit too");
     cudaError_t e = cudaFuncSetAttribute(select_kernel<C>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(bytes));
@@ -1226,11 +1579,16 @@ cudaError_t try_select(const RepairArgs& a, cudaStream_t st, bool* launched)
 
 int select_cluster_size(int U, int N, int sms)
 {
-    // the largest cluster that keeps every unit in one wave of two CTAs per SM (more
-    // CTAs than that queue behind each other), slices of at least 256 positions, at
-    // most 16 CTAs
+    // More CTAs per unit while each has an SM to itself and 4096 positions or more: below
+    // that the cluster's barriers cost more than the shorter passes save, and a second CTA
+    // on an SM halves both (us per selection with C = 1 / 2 / 4 / 8: 8 units of 4096
+    // positions 17 / 19 / 18 / 21, 8 of 32768 193 / 55 / 36 / 31, 72 of 8192 25 / 22 / 27 /
+    // 79, 288 of 16384 61 / 80 / 112 / 286).  Slices above 24576 positions are split
+    // whatever the number of units, since their swap lists seldom fit one CTA's buckets
+    // (8 units of 131072 by the general path 1127 / 617 / 350, by buckets at C = 8 82).
     int C = 1;
-    while (C < 16 && static_cast<int64_t>(U) * (2 * C) <= 2LL * sms && N / (2 * C) >= 256)
+    while (C < 8 && ((static_cast<int64_t>(U) * (2 * C) <= sms && N / (2 * C) >= 4096) ||
+                     N / C > 24576))
         C <<= 1;
     return C;
 }
