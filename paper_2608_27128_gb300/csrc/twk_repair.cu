@@ -582,9 +582,9 @@ __host__ __device__ inline int slice_len(int N, int C)
 // comparisons across the CTA.  Three passes read the slice's b and mask (coalesced, in any
 // order):
 //   1. S1 = S0, the counts, and the smallest and largest b of each side;
-//   2. a histogram of each side over kBk equal intervals of its range, summed over the
-//      cluster; its prefix sums give every bucket's first rank.  Buckets whose first rank
-//      is below m hold the m most severe items (and the rest of the bucket at the cut);
+//   2. a histogram of each side over kBk intervals of its range, summed over the cluster;
+//      its prefix sums give every bucket's first rank.  Buckets whose first rank is below m
+//      hold the m most severe items (and the rest of the bucket at the cut);
 //   3. their items go to the bucket's place in the shared memory of the CTA that owns the
 //      bucket (buckets are dealt out by first rank, so that each CTA gets about 1/C).
 // An item's rank is its bucket's first rank plus the number of items of its bucket ordered
@@ -596,8 +596,8 @@ __host__ __device__ inline int slice_len(int N, int C)
 // general path's radix select takes up to eight passes over lists in memory with several
 // block barriers each, and its bitonic sort was 58 of 182 thousand cycles per unit at 16384
 // positions.  General -> buckets, with the cluster size each was given: 288 units of 16384
-// positions 120 -> 60 us, 8 of 8192 67 -> 22, 8 of 4096 57 -> 17, 8 of 131072 295 -> 82,
-// 128 of 8192 64 -> 25.
+// positions 120 -> 64 us, 8 of 8192 67 -> 23, 8 of 4096 57 -> 16, 8 of 131072 128 -> 65,
+// 128 of 8192 64 -> 27.
 constexpr int kBk = 1024;      // buckets per side
 constexpr int kCap = 3072;     // items per side a CTA holds (36 KB): two CTAs per SM fit
 constexpr int kMaxBucket = 256;
@@ -624,11 +624,36 @@ __device__ __forceinline__ float narrow(uint64_t u)
     return __uint_as_float((hi & 0x80000000u) | mag);
 }
 
-// Bucket of a value in [lo, lo + (kBk - 1) / scale]; non-decreasing in f.  (A range too wide
-// for fp32 has scale 0, and every value falls into bucket 0.)
-__device__ __forceinline__ int bucket_of(float f, float lo, float scale)
+// How a side's values map to buckets.  d is a value's distance from the side's most severe
+// end, w the whole range: half of the buckets divide w evenly, the other half divide the
+// 16 octaves below w, and a value's bucket is the sum of its two shares.  Evenly spread
+// values keep a bucket each per 1/512 of the range, and the twins that crowd within 1e-5 to
+// 1e-3 of the largest b spread over the octaves (with 1024 even intervals they filled one
+// bucket, and the Llama-3.2-1B cache's units went to the general path, 60 us).
+// Non-decreasing in d (each operation is).
+struct Buckets {
+    float end;     // the most severe value, as fp32
+    float inv;     // (kBk / 2 - 1) / w, or 0: every value in bucket 0
+    int floor;     // bits of w 2^-16, as an int
+};
+
+__device__ __forceinline__ Buckets make_buckets(float severe, float mild)
 {
-    return min(kBk - 1, max(0, static_cast<int>((f - lo) * scale)));
+    const float w = fabsf(mild - severe);
+    Buckets k{severe, (kBk / 2 - 1) / w, __float_as_int(w) - (16 << 23)};
+    if (!(w > 0.f && w <= 3.4e38f && k.inv <= 3.4e38f)) {
+        k.inv = 0.f;
+        k.floor = 0x7FFFFFFF;
+    }
+    return k;
+}
+
+__device__ __forceinline__ int bucket_of(float f, const Buckets& k)
+{
+    const float d = fabsf(f - k.end);
+    const int over = max(0, __float_as_int(d) - max(k.floor, 0));   // 2^23 per octave
+    const float v = __fmaf_rn(d, k.inv, static_cast<float>(k.inv == 0.f ? 0 : over) * 0x1p-18f);
+    return min(kBk - 1, static_cast<int>(v));
 }
 
 // The b whose severity key (side 0: orphans, 1: donors) is k, as the double's bits.
@@ -775,18 +800,11 @@ __device__ bool select_by_buckets(Shared& s, ClusterShared& cs, uint64_t* sk, in
         }
         return true;
     }
-    float from[2], scale[2];
-#pragma unroll
-    for (int y = 0; y < 2; ++y) {
-        from[y] = from_int(ends[2 * y]);
-        const float w = from_int(ends[2 * y + 1]) - from[y];
-        scale[y] = w > 0.f && w <= 3.4e38f ? (kBk - 1) / w : 0.f;
-        if (!(scale[y] <= 3.4e38f)) scale[y] = 0.f;
-    }
-    // side x's bucket, most severe first (donors from the largest b down)
+    // side x's bucket: orphans from the smallest b up, donors from the largest down
+    const Buckets bo = make_buckets(from_int(ends[0]), from_int(ends[1]));
+    const Buckets bd = make_buckets(from_int(ends[3]), from_int(ends[2]));
     auto bucket = [&](int x, uint64_t bits) {
-        const int k = bucket_of(narrow(bits), x ? from[1] : from[0], x ? scale[1] : scale[0]);
-        return x ? kBk - 1 - k : k;
+        return bucket_of(narrow(bits), x ? bd : bo);
     };
 
     // 2. histogram, summed over the cluster, and its prefix sums

@@ -35,7 +35,7 @@ def _check(b, S0, tau):
 
 
 @pytest.mark.parametrize("cluster", [1, 2, 4, 8])
-@pytest.mark.parametrize("kind", ["near", "wide", "special", "one value"])
+@pytest.mark.parametrize("kind", ["near", "crowded", "wide", "special", "one value"])
 def test_values(kind, cluster, monkeypatch):
     monkeypatch.setenv("TWINKV_SELECT_CLUSTER", str(cluster))
     rng = np.random.default_rng([len(kind), cluster])
@@ -44,6 +44,9 @@ def test_values(kind, cluster, monkeypatch):
     if kind == "near":
         b = np.where(rng.random((U, N)) < 0.3, 1.0 - 4e-4 * rng.random((U, N)),
                      0.3 + 0.05 * rng.standard_normal((U, N)))
+    elif kind == "crowded":     # the largest b within 1e-3 of 1, the rest of the donors far off
+        b = np.minimum(1.0, np.where(rng.random((U, N)) < 0.3, 1.0 - rng.exponential(1e-4, (U, N)),
+                                     0.5 + 0.1 * rng.standard_normal((U, N))))
     elif kind == "wide":
         b = rng.uniform(-1, 1, (U, N)) * 10.0 ** rng.integers(-320, 308, (U, N))
     elif kind == "special":
