@@ -208,20 +208,12 @@ twinkv_status check_ws(const twinkv_shape& s, int op, void* ws, size_t bytes, La
     return TWINKV_OK;
 }
 
-// bf16 view of the keys (rounding float32 keys into the workspace first).
-twinkv_status keys_bf16(const void* keys, const twinkv_shape& s, void* ws, const Layout& L,
-                        cudaStream_t st, const uint16_t** out)
+// The bf16 keys the later stages read: the caller's, or for float32 keys the rounded copy in
+// the workspace, which the prep kernels write.
+uint16_t* keys_bf16(const void* keys, const twinkv_shape& s, void* ws, const Layout& L)
 {
-    if (s.dtype == TWINKV_BF16) {
-        *out = static_cast<const uint16_t*>(keys);
-        return TWINKV_OK;
-    }
-    uint16_t* k16 = at<uint16_t>(ws, L.keys16);
-    ProfScope p(TWINKV_KERNEL_PREP, st);
-    const int64_t n = static_cast<int64_t>(s.L) * s.H * s.N * s.d;
-    const cudaError_t e = launch_round_bf16(static_cast<const float*>(keys), k16, n, st);
-    *out = k16;
-    return cuda_status(e);
+    return s.dtype == TWINKV_F32 ? at<uint16_t>(ws, L.keys16)
+                                 : static_cast<uint16_t*>(const_cast<void*>(keys));
 }
 
 twinkv_status run_audit(const DeviceInfo& dev, const twinkv_shape& s, const uint16_t* keys16,
@@ -576,8 +568,8 @@ twinkv_status redundancy_impl(const void* keys, twinkv_shape s, int32_t window, 
     if ((r = device_info(&dev)) != TWINKV_OK) return r;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
 
-    const uint16_t* k16 = nullptr;
-    if ((r = keys_bf16(keys, s, workspace, L, st, &k16)) != TWINKV_OK) return r;
+    uint16_t* const k16 = keys_bf16(keys, s, workspace, L);
+    const bool f32 = s.dtype == TWINKV_F32;
     const int U = s.L * s.H;
     const int64_t NP = column_stride(s.N);
     float* colrinv = at<float>(workspace, L.colrinv);
@@ -588,8 +580,8 @@ twinkv_status redundancy_impl(const void* keys, twinkv_shape s, int32_t window, 
         ProfScope p(TWINKV_KERNEL_PREP, st);
         unsigned* ukk = at<unsigned>(workspace, L.ukk);
         if (cudaMemsetAsync(ukk, 0, static_cast<size_t>(U) * 4, st) != cudaSuccess ||
-            launch_norms_identity(k16, U, s.N, s.d, NP, colrinv, colpos, norm2, st, 1.0f, ukk) !=
-                cudaSuccess ||
+            launch_norms_identity(keys, f32, k16, U, s.N, s.d, NP, colrinv, colpos, norm2, st,
+                                  1.0f, ukk) != cudaSuccess ||
             launch_scale_columns(colrinv, U, NP, ukk, st) != cudaSuccess ||
             (symmetric && cudaMemsetAsync(slots, 0, static_cast<size_t>(U) * s.N * 8, st) !=
                               cudaSuccess))
@@ -659,8 +651,8 @@ twinkv_status twinkv_policy(const void* keys, twinkv_shape s, const int32_t* bud
     if ((r = device_info(&dev)) != TWINKV_OK) return r;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
 
-    const uint16_t* k16 = nullptr;
-    if ((r = keys_bf16(keys, s, workspace, L, st, &k16)) != TWINKV_OK) return r;
+    uint16_t* const k16 = keys_bf16(keys, s, workspace, L);
+    const bool f32 = s.dtype == TWINKV_F32;
     const int U = s.L * s.H;
     const int64_t NP = column_stride(s.N);
     float* colrinv = at<float>(workspace, L.colrinv);
@@ -669,9 +661,8 @@ twinkv_status twinkv_policy(const void* keys, twinkv_shape s, const int32_t* bud
     int* count = out_count ? out_count : at<int>(workspace, L.rcount);
     {
         ProfScope pr(TWINKV_KERNEL_PREP, st);
-        if (launch_norms_identity(k16, U, s.N, s.d, NP, colrinv, colpos, norm2, st,
-                                  kCountScale) !=
-            cudaSuccess)
+        if (launch_norms_identity(keys, f32, k16, U, s.N, s.d, NP, colrinv, colpos, norm2, st,
+                                  kCountScale) != cudaSuccess)
             return TWINKV_ERR_CUDA;
     }
     AuditArgs a;
@@ -712,21 +703,20 @@ twinkv_status prep_stages(const void* keys, const twinkv_shape& s, const uint8_t
                           void* workspace, const Layout& L, cudaStream_t st,
                           const uint16_t** k16)
 {
-    twinkv_status r;
-    if ((r = keys_bf16(keys, s, workspace, L, st, k16)) != TWINKV_OK) return r;
+    uint16_t* const rows = keys_bf16(keys, s, workspace, L);
+    *k16 = rows;
     const int U = s.L * s.H;
     const int64_t NP = column_stride(s.N);
+    unsigned* ukk = at<unsigned>(workspace, L.ukk);
     {
         ProfScope pr(TWINKV_KERNEL_PREP, st);
         if (launch_scan(retained_mask, U, s.N, at<int>(workspace, L.cnt),
-                        at<int>(workspace, L.kb), st) != cudaSuccess)
+                        at<int>(workspace, L.kb), ukk, st) != cudaSuccess)
             return TWINKV_ERR_CUDA;
     }
     ProfScope pr(TWINKV_KERNEL_PREP, st);
-    unsigned* ukk = at<unsigned>(workspace, L.ukk);
-    if (cudaMemsetAsync(ukk, 0, static_cast<size_t>(U) * 4, st) != cudaSuccess ||
-        launch_gather(*k16, retained_mask, at<int>(workspace, L.cnt), at<int>(workspace, L.kb),
-                      U, s.N, s.d, NP, at<uint16_t>(workspace, L.kp),
+    if (launch_gather(keys, s.dtype == TWINKV_F32, rows, retained_mask, at<int>(workspace, L.cnt),
+                      at<int>(workspace, L.kb), U, s.N, s.d, NP, at<uint16_t>(workspace, L.kp),
                       at<float>(workspace, L.colrinv), at<int>(workspace, L.colpos),
                       at<float4>(workspace, L.norm2), ukk, st) != cudaSuccess ||
         launch_scale_columns(at<float>(workspace, L.colrinv), U, NP, ukk, st) != cudaSuccess)

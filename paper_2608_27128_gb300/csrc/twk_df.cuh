@@ -67,15 +67,27 @@ __device__ __forceinline__ void quarter_dot(const uint16_t* __restrict__ a,
     }
 }
 
-// a . b by the kParts consecutive lanes of a group (every lane passes its part): the
-// lanes' parts are summed as ((q0 + q1) + (q2 + q3)), and every lane of the group returns
-// the same double-float.  All dot products, norms included, go through this routine.
-template <int D>
-__device__ __forceinline__ DFPair group_dot_df(const uint16_t* __restrict__ a,
-                                             const uint16_t* __restrict__ b, int part)
+// The same for a . a with the lane's 16-byte chunks already in registers.
+template <int Q>
+__device__ __forceinline__ void quarter_square(const uint4 (&v)[Q], float& hi, float& lo)
 {
-    float hi, lo;
-    quarter_dot<D>(a, b, part, hi, lo);
+    hi = 0.f;
+    lo = 0.f;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        const uint32_t w[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float e = __uint_as_float(w[k] << 16), o = __uint_as_float(w[k] & 0xFFFF0000u);
+            two_sum_acc(hi, lo, __fmul_rn(e, e));
+            two_sum_acc(hi, lo, __fmul_rn(o, o));
+        }
+    }
+}
+
+// The lanes' parts of one dot product summed as ((q0 + q1) + (q2 + q3)).
+__device__ __forceinline__ DFPair group_sum(float hi, float lo)
+{
 #pragma unroll
     for (int o = 1; o < kParts; o <<= 1) {
         const float h2 = __shfl_xor_sync(0xFFFFFFFFu, hi, o);
@@ -83,6 +95,18 @@ __device__ __forceinline__ DFPair group_dot_df(const uint16_t* __restrict__ a,
         df_add(hi, lo, h2, l2);
     }
     return DFPair{hi, lo};
+}
+
+// a . b by the kParts consecutive lanes of a group (every lane passes its part): the
+// lanes' parts are summed as ((q0 + q1) + (q2 + q3)), and every lane of the group returns
+// the same double-float.  All dot products, norms included, take their terms in this order.
+template <int D>
+__device__ __forceinline__ DFPair group_dot_df(const uint16_t* __restrict__ a,
+                                             const uint16_t* __restrict__ b, int part)
+{
+    float hi, lo;
+    quarter_dot<D>(a, b, part, hi, lo);
+    return group_sum(hi, lo);
 }
 
 // The same two dot products a . b0 and a . b1 at once, one in each half of paired

@@ -1,4 +1,5 @@
-// twk_prep.cu -- O(N d) preparation for the audit (TwinKV, arXiv 2608.27128):
+// twk_prep.cu -- O(N d) preparation for the audit (TwinKV, arXiv 2608.27128), one pass over
+// the keys, bound by memory:
 //   * float32 keys -> bf16 (round to nearest even),
 //   * per key k . k and 1/||k|| (the l2 normalisation of Sec. 3.2 Eq. 1, applied later
 //     as a scale; a zero key gets 0, so it has similarity 0 with every key),
@@ -6,6 +7,8 @@
 //     position order, padded to a 256-column tile, then evicted keys in position order,
 //     with per-column 1/||k|| (NaN on padding columns, which the audit then ignores)
 //     and per-column original position.
+#include <algorithm>
+
 #include <cuda_bf16.h>
 
 #include "twk_df.cuh"
@@ -16,24 +19,55 @@ namespace {
 
 __device__ __forceinline__ float nan_f() { return __uint_as_float(0x7FFFFFFFu); }
 
-__global__ void round_bf16_kernel(const float* __restrict__ in, uint16_t* __restrict__ out,
-                                  int64_t n)
-{
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-    for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
-         i += stride)
-        out[i] = __bfloat16_as_ushort(__float2bfloat16_rn(in[i]));
-}
-
 constexpr int kPrepThreads = 256;
 constexpr int kKeysPerBlock = kPrepThreads / kParts;   // NP is a multiple of this
 
+// A lane's 16-byte chunks part, part + kParts, ... of a key's bf16 row, from bf16 keys or
+// from float32 ones rounded to nearest even (8 floats per chunk).
+template <int D>
+__device__ __forceinline__ void load_key(const uint16_t* __restrict__ keys, int64_t row, int part,
+                                         uint4 (&v)[D / 8 / kParts])
+{
+    const uint4* src = reinterpret_cast<const uint4*>(keys + row * D) + part;
+#pragma unroll
+    for (int q = 0; q < D / 8 / kParts; ++q) v[q] = __ldg(src + q * kParts);
+}
+
+__device__ __forceinline__ uint32_t round2(float a, float b)
+{
+    return static_cast<uint32_t>(__bfloat16_as_ushort(__float2bfloat16_rn(a))) |
+           static_cast<uint32_t>(__bfloat16_as_ushort(__float2bfloat16_rn(b))) << 16;
+}
+
+template <int D>
+__device__ __forceinline__ void load_key(const float* __restrict__ keys, int64_t row, int part,
+                                         uint4 (&v)[D / 8 / kParts])
+{
+    const float4* src = reinterpret_cast<const float4*>(keys + row * D) + 2 * part;
+#pragma unroll
+    for (int q = 0; q < D / 8 / kParts; ++q) {
+        const float4 f = __ldg(src + 2 * q * kParts), g = __ldg(src + 2 * q * kParts + 1);
+        v[q] = make_uint4(round2(f.x, f.y), round2(f.z, f.w), round2(g.x, g.y), round2(g.z, g.w));
+    }
+}
+
+template <int D>
+__device__ __forceinline__ void store_key(uint16_t* out, int64_t row, int part,
+                                          const uint4 (&v)[D / 8 / kParts])
+{
+    uint4* dst = reinterpret_cast<uint4*>(out + row * D) + part;
+#pragma unroll
+    for (int q = 0; q < D / 8 / kParts; ++q) dst[q * kParts] = v[q];
+}
+
 // The norm record of one key, computed by its kParts-lane group: k.k and 1/||k|| as
 // double-floats (for the exact similarity values) and 1/||k|| in fp32 (for the audit).
-template <int D>
-__device__ __forceinline__ float4 key_norms(const uint16_t* key, int part, float& rinv32)
+template <int Q>
+__device__ __forceinline__ float4 key_norms(const uint4 (&v)[Q], float& rinv32)
 {
-    const DF sq = group_dot_df<D>(key, key, part);
+    float hi, lo;
+    quarter_square(v, hi, lo);
+    const DF sq = group_sum(hi, lo);
     const DF rn = sq.h > 0.f ? df_rsqrt(sq) : DF{0.f, 0.f};
     rinv32 = rn.h;
     return make_float4(sq.h, sq.l, rn.h, rn.l);
@@ -60,83 +94,125 @@ __device__ __forceinline__ void unit_max_kk(unsigned* unit_kk, int64_t u, float 
 // Mode 0 (keys as given): per column p of unit blockIdx.y, colrinv = rscale/||k_p||
 // (rscale a power of two, so the scaling is exact) and colpos = p, NaN / -1 on the
 // padding columns [N, NP); norms[u][p] = the norm record; unit_kk[u] (if given) =
-// the unit's largest k.k.  Grid (NP / kKeysPerBlock, U), kParts lanes per column.
-template <int D>
+// the unit's largest k.k.  float32 keys also leave their rounded rows in keys16: one pass
+// over them, where a separate rounding pass wrote the bf16 keys for this one to read back
+// (16 units of 5003 x 128: 50 -> 18 us with the launches).  Grid (NP / kKeysPerBlock, U),
+// kParts lanes per column.
+template <int D, typename Key>
 __global__ void __launch_bounds__(kPrepThreads)
-    norms_identity_kernel(const uint16_t* __restrict__ keys, int N, int64_t NP,
+    norms_identity_kernel(const Key* __restrict__ keys, int N, int64_t NP,
                           float* __restrict__ colrinv, int* __restrict__ colpos,
-                          float4* __restrict__ norms, float rscale, unsigned* unit_kk)
+                          float4* __restrict__ norms, float rscale, unsigned* unit_kk,
+                          uint16_t* __restrict__ keys16)
 {
     const int part = threadIdx.x % kParts;
     const int p = blockIdx.x * kKeysPerBlock + threadIdx.x / kParts;
     const int64_t u = blockIdx.y;
-    // every lane takes part in the shuffles of group_dot_df: padding columns use key 0
-    const int pk = p < N ? p : 0;
+    // every lane takes part in the shuffles of the norms: padding columns use key 0
+    const int64_t row = u * N + (p < N ? p : 0);
+    uint4 v[D / 8 / kParts];
+    load_key<D>(keys, row, part, v);
+    if constexpr (sizeof(Key) == 4)
+        if (p < N) store_key<D>(keys16, row, part, v);
     float r32;
-    const float4 nr = key_norms<D>(keys + (u * N + pk) * D, part, r32);
+    const float4 nr = key_norms(v, r32);
     if (part == 0) {
         colrinv[u * NP + p] = p < N ? r32 * rscale : nan_f();
         colpos[u * NP + p] = p < N ? p : -1;
-        if (p < N) norms[u * N + p] = nr;
+        if (p < N) norms[row] = nr;
     }
     if (unit_kk) unit_max_kk(unit_kk, u, (part == 0 && p < N) ? nr.x : 0.f);
 }
 
-// Mode 1, step 1: cnt[u][p] = number of retained positions before p; kb[u] = |S0|.
-// One block per unit; a mask byte counts as retained when non-zero.
+constexpr int kScanBytes = 16;   // mask bytes per thread and step
+
+// Mode 1, step 1: cnt[u][p] = number of retained positions before p; kb[u] = |S0|;
+// unit_kk[u] = 0.  One block per unit; a mask byte counts as retained when non-zero.  A
+// thread takes 16 consecutive positions, so that a block covers 16384 per step of one
+// barrier (with one position per thread and four barriers per step of 1024, the prep of 8
+// units of 131072 x 128 took 189 us, now 118; 128 units of 8192 x 64 69 -> 62).
 __global__ void scan_kernel(const uint8_t* __restrict__ mask, int N, int* __restrict__ cnt,
-                            int* __restrict__ kb)
+                            int* __restrict__ kb, unsigned* __restrict__ unit_kk)
 {
-    __shared__ int warp_tot[32];
-    __shared__ int carry;
+    __shared__ int warp_tot[2][32];
     const int u = blockIdx.x;
     const uint8_t* m = mask + static_cast<int64_t>(u) * N;
     int* c = cnt + static_cast<int64_t>(u) * N;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    for (int base = 0; base < N; base += blockDim.x) {
-        const int p = base + threadIdx.x;
-        const int f = (p < N && m[p] != 0) ? 1 : 0;
+    const bool vec = N % kScanBytes == 0 && (reinterpret_cast<uintptr_t>(mask) & 15) == 0;
+    int carry = 0, step = 0;
+    for (int base = 0; base < N; base += blockDim.x * kScanBytes, step ^= 1) {
+        const int p0 = base + threadIdx.x * kScanBytes;
+        uint32_t keep = 0;   // bit j: position p0 + j is retained
+        if (vec) {
+            if (p0 < N) {
+                const uint4 v = *reinterpret_cast<const uint4*>(m + p0);
+                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int j = 0; j < kScanBytes; ++j)
+                    keep |= ((w[j / 4] >> (8 * (j % 4))) & 255u) != 0u ? 1u << j : 0u;
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < kScanBytes; ++j)
+                if (p0 + j < N && m[p0 + j] != 0) keep |= 1u << j;
+        }
+        const int f = __popc(keep);
         int x = f;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int y = __shfl_up_sync(0xFFFFFFFFu, x, o);
             if (lane >= o) x += y;
         }
-        if (lane == 31) warp_tot[wid] = x;
+        if (lane == 31) warp_tot[step][wid] = x;
         __syncthreads();
-        if (wid == 0) {
-            int t = lane < nw ? warp_tot[lane] : 0;
+        const int t = lane < nw ? warp_tot[step][lane] : 0;
+        const int all = __reduce_add_sync(0xFFFFFFFFu, t);
+        const int mine = __reduce_add_sync(0xFFFFFFFFu, lane < wid ? t : 0);
+        int run = carry + mine + x - f;
+        carry += all;
+        if (vec) {   // N, and so every row of cnt, is a multiple of 16 entries
+            if (p0 < N) {
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(0xFFFFFFFFu, t, o);
-                if (lane >= o) t += y;
+                for (int j = 0; j < kScanBytes; j += 4) {
+                    int4 o;
+                    o.x = run;
+                    o.y = o.x + ((keep >> j) & 1u);
+                    o.z = o.y + ((keep >> (j + 1)) & 1u);
+                    o.w = o.z + ((keep >> (j + 2)) & 1u);
+                    run = o.w + ((keep >> (j + 3)) & 1u);
+                    *reinterpret_cast<int4*>(c + p0 + j) = o;
+                }
             }
-            if (lane < nw) warp_tot[lane] = t;   // inclusive prefix of warp totals
+        } else {
+#pragma unroll
+            for (int j = 0; j < kScanBytes; ++j) {
+                if (p0 + j < N) c[p0 + j] = run;
+                run += (keep >> j) & 1u;
+            }
         }
-        __syncthreads();
-        const int before = carry + (wid > 0 ? warp_tot[wid - 1] : 0) + (x - f);
-        if (p < N) c[p] = before;
-        __syncthreads();
-        if (threadIdx.x == 0) carry += warp_tot[nw - 1];
-        __syncthreads();
+        // the next step writes the other half of warp_tot; the one after it follows the
+        // next step's barrier
     }
-    if (threadIdx.x == 0) kb[u] = carry;
+    if (threadIdx.x == 0) {
+        kb[u] = carry;
+        unit_kk[u] = 0u;
+    }
 }
 
 // Mode 1, step 2: slot p < N of unit blockIdx.y is key p: its kParts-lane group copies
 // it to its column of the retained-first layout (retained keys in position order, then
 // from the next tile boundary the evicted ones), with 1/||k_p|| (fp32) and p as column
-// metadata, and writes its norm record.  Slots p >= N are the padding columns
-// [K, Kpad) and [Kpad + N - K, NP): zero keys, NaN, -1.  unit_kk[u] = the unit's
-// largest k.k.  Grid (NP / kKeysPerBlock, U).
-template <int D>
+// metadata, and writes its norm record (and, for float32 keys, its rounded row).  Slots
+// p >= N are the padding columns [K, Kpad) and [Kpad + N - K, NP): zero keys, NaN, -1.
+// unit_kk[u] = the unit's largest k.k.  Grid (NP / kKeysPerBlock, U).
+template <int D, typename Key>
 __global__ void __launch_bounds__(kPrepThreads)
-    gather_kernel(const uint16_t* __restrict__ keys, const uint8_t* __restrict__ mask,
+    gather_kernel(const Key* __restrict__ keys, const uint8_t* __restrict__ mask,
                   const int* __restrict__ cnt, const int* __restrict__ kb, int N, int64_t NP,
                   uint16_t* __restrict__ kp, float* __restrict__ colrinv,
-                  int* __restrict__ colpos, float4* __restrict__ norms, unsigned* unit_kk)
+                  int* __restrict__ colpos, float4* __restrict__ norms, unsigned* unit_kk,
+                  uint16_t* __restrict__ keys16)
 {
     constexpr int Q = D / 8 / kParts;   // 16-byte chunks per lane
     const int part = threadIdx.x % kParts;
@@ -144,28 +220,30 @@ __global__ void __launch_bounds__(kPrepThreads)
     const int64_t u = blockIdx.y;
     const int k = kb[u];
     const int kpad = ((k + kBN - 1) / kBN) * kBN;
-    const int pk = p < N ? p : 0;   // every lane takes part in the shuffles
-    const uint16_t* key = keys + (u * N + pk) * D;
-    float r32;
-    const float4 nr = key_norms<D>(key, part, r32);
+    const int64_t row = u * N + (p < N ? p : 0);   // every lane takes part in the shuffles
+    uint4 v[Q];
+    load_key<D>(keys, row, part, v);
     int col;
     if (p < N) {
-        const int before = cnt[u * N + p];
-        col = mask[u * N + p] ? before : kpad + (p - before);
+        const int before = cnt[row];
+        col = mask[row] ? before : kpad + (p - before);
     } else {
         const int r = p - N;
         col = r < kpad - k ? k + r : kpad + (N - k) + (r - (kpad - k));
     }
-    // the lane's 16-byte chunks part, part + kParts, ... (those its dot product read)
-    const uint4* src = reinterpret_cast<const uint4*>(key) + part;
-    uint4* dst = reinterpret_cast<uint4*>(kp + (u * NP + col) * D) + part;
+    if constexpr (sizeof(Key) == 4)
+        if (p < N) store_key<D>(keys16, row, part, v);
+    float r32;
+    const float4 nr = key_norms(v, r32);
+    if (p >= N) {
 #pragma unroll
-    for (int q = 0; q < Q; ++q)
-        dst[q * kParts] = p < N ? __ldg(src + q * kParts) : make_uint4(0u, 0u, 0u, 0u);
+        for (int q = 0; q < Q; ++q) v[q] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    store_key<D>(kp, u * NP + col, part, v);
     if (part == 0) {
         colrinv[u * NP + col] = p < N ? r32 : nan_f();
         colpos[u * NP + col] = p < N ? p : -1;
-        if (p < N) norms[u * N + p] = nr;
+        if (p < N) norms[row] = nr;
     }
     unit_max_kk(unit_kk, u, (part == 0 && p < N) ? nr.x : 0.f);
 }
@@ -188,29 +266,24 @@ __global__ void __launch_bounds__(kPrepThreads)
     colrinv[u * NP + c] = ldexpf(colrinv[u * NP + c], -e);
 }
 
-
 }  // namespace
 
-cudaError_t launch_round_bf16(const float* in, uint16_t* out, int64_t n, cudaStream_t st)
-{
-    int64_t blocks = (n + 255) / 256;
-    if (blocks > 65535LL * 16) blocks = 65535LL * 16;
-    if (blocks < 1) blocks = 1;
-    round_bf16_kernel<<<static_cast<int>(blocks), 256, 0, st>>>(in, out, n);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_norms_identity(const uint16_t* keys, int U, int N, int d, int64_t NP,
-                                  float* colrinv, int* colpos, float4* norms, cudaStream_t st,
-                                  float rscale, unsigned* unit_kk)
+cudaError_t launch_norms_identity(const void* keys, bool f32, uint16_t* keys16, int U, int N,
+                                  int d, int64_t NP, float* colrinv, int* colpos,
+                                  float4* norms, cudaStream_t st, float rscale,
+                                  unsigned* unit_kk)
 {
     const dim3 grid(static_cast<unsigned>(NP / kKeysPerBlock), U);
-    if (d == 128)
-        norms_identity_kernel<128><<<grid, kPrepThreads, 0, st>>>(keys, N, NP, colrinv, colpos,
-                                                                   norms, rscale, unit_kk);
-    else
-        norms_identity_kernel<64><<<grid, kPrepThreads, 0, st>>>(keys, N, NP, colrinv, colpos,
-                                                                  norms, rscale, unit_kk);
+    auto go = [&](auto kernel, auto* k) {
+        kernel<<<grid, kPrepThreads, 0, st>>>(k, N, NP, colrinv, colpos, norms, rscale, unit_kk,
+                                              keys16);
+    };
+    const float* kf = static_cast<const float*>(keys);
+    const uint16_t* kh = static_cast<const uint16_t*>(keys);
+    if (f32 && d == 128) go(norms_identity_kernel<128, float>, kf);
+    else if (f32) go(norms_identity_kernel<64, float>, kf);
+    else if (d == 128) go(norms_identity_kernel<128, uint16_t>, kh);
+    else go(norms_identity_kernel<64, uint16_t>, kh);
     return cudaGetLastError();
 }
 
@@ -222,24 +295,31 @@ cudaError_t launch_scale_columns(float* colrinv, int U, int64_t NP, const unsign
     return cudaGetLastError();
 }
 
-cudaError_t launch_scan(const uint8_t* mask, int U, int N, int* cnt, int* kb, cudaStream_t st)
+cudaError_t launch_scan(const uint8_t* mask, int U, int N, int* cnt, int* kb, unsigned* unit_kk,
+                        cudaStream_t st)
 {
-    scan_kernel<<<U, 1024, 0, st>>>(mask, N, cnt, kb);
+    // one step where 1024 threads cover the unit, in no more warps than it needs
+    const int threads = std::min(1024, (N + 32 * kScanBytes - 1) / (32 * kScanBytes) * 32);
+    scan_kernel<<<U, threads, 0, st>>>(mask, N, cnt, kb, unit_kk);
     return cudaGetLastError();
 }
 
-cudaError_t launch_gather(const uint16_t* keys, const uint8_t* mask, const int* cnt,
-                          const int* kb, int U, int N, int d, int64_t NP, uint16_t* kp,
-                          float* colrinv, int* colpos, float4* norms, unsigned* unit_kk,
-                          cudaStream_t st)
+cudaError_t launch_gather(const void* keys, bool f32, uint16_t* keys16, const uint8_t* mask,
+                          const int* cnt, const int* kb, int U, int N, int d, int64_t NP,
+                          uint16_t* kp, float* colrinv, int* colpos, float4* norms,
+                          unsigned* unit_kk, cudaStream_t st)
 {
     const dim3 grid(static_cast<unsigned>(NP / kKeysPerBlock), U);
-    if (d == 128)
-        gather_kernel<128><<<grid, kPrepThreads, 0, st>>>(keys, mask, cnt, kb, N, NP, kp,
-                                                           colrinv, colpos, norms, unit_kk);
-    else
-        gather_kernel<64><<<grid, kPrepThreads, 0, st>>>(keys, mask, cnt, kb, N, NP, kp,
-                                                          colrinv, colpos, norms, unit_kk);
+    auto go = [&](auto kernel, auto* k) {
+        kernel<<<grid, kPrepThreads, 0, st>>>(k, mask, cnt, kb, N, NP, kp, colrinv, colpos, norms,
+                                              unit_kk, keys16);
+    };
+    const float* kf = static_cast<const float*>(keys);
+    const uint16_t* kh = static_cast<const uint16_t*>(keys);
+    if (f32 && d == 128) go(gather_kernel<128, float>, kf);
+    else if (f32) go(gather_kernel<64, float>, kf);
+    else if (d == 128) go(gather_kernel<128, uint16_t>, kh);
+    else go(gather_kernel<64, uint16_t>, kh);
     return cudaGetLastError();
 }
 
