@@ -582,7 +582,7 @@ twinkv_status redundancy_impl(const void* keys, twinkv_shape s, int32_t window, 
         if (cudaMemsetAsync(ukk, 0, static_cast<size_t>(U) * 4, st) != cudaSuccess ||
             launch_norms_identity(keys, f32, k16, U, s.N, s.d, NP, colrinv, colpos, norm2, st,
                                   1.0f, ukk) != cudaSuccess ||
-            launch_scale_columns(colrinv, U, NP, ukk, st) != cudaSuccess ||
+            launch_scale_columns(colrinv, U, NP, ukk, nullptr, st) != cudaSuccess ||
             (symmetric && cudaMemsetAsync(slots, 0, static_cast<size_t>(U) * s.N * 8, st) !=
                               cudaSuccess))
             return TWINKV_ERR_CUDA;
@@ -700,7 +700,7 @@ namespace {
 // prefix counts, and the retained-first column layout with its metadata and the norm
 // records.  *k16 receives the bf16 keys.
 twinkv_status prep_stages(const void* keys, const twinkv_shape& s, const uint8_t* retained_mask,
-                          void* workspace, const Layout& L, cudaStream_t st,
+                          bool need_all, void* workspace, const Layout& L, cudaStream_t st,
                           const uint16_t** k16)
 {
     uint16_t* const rows = keys_bf16(keys, s, workspace, L);
@@ -718,8 +718,9 @@ twinkv_status prep_stages(const void* keys, const twinkv_shape& s, const uint8_t
     if (launch_gather(keys, s.dtype == TWINKV_F32, rows, retained_mask, at<int>(workspace, L.cnt),
                       at<int>(workspace, L.kb), U, s.N, s.d, NP, at<uint16_t>(workspace, L.kp),
                       at<float>(workspace, L.colrinv), at<int>(workspace, L.colpos),
-                      at<float4>(workspace, L.norm2), ukk, st) != cudaSuccess ||
-        launch_scale_columns(at<float>(workspace, L.colrinv), U, NP, ukk, st) != cudaSuccess)
+                      at<float4>(workspace, L.norm2), ukk, need_all, st) != cudaSuccess ||
+        launch_scale_columns(at<float>(workspace, L.colrinv), U, NP, ukk,
+                             need_all ? nullptr : at<int>(workspace, L.kb), st) != cudaSuccess)
         return TWINKV_ERR_CUDA;
     return TWINKV_OK;
 }
@@ -778,7 +779,8 @@ twinkv_status audit_stages(const DeviceInfo* dev, const void* keys, const twinkv
                            void* workspace, const Layout& L, cudaStream_t st)
 {
     const uint16_t* k16 = nullptr;
-    const twinkv_status r = prep_stages(keys, s, retained_mask, workspace, L, st, &k16);
+    const twinkv_status r = prep_stages(keys, s, retained_mask, out_score_all || out_twin_all,
+                                        workspace, L, st, &k16);
     if (r != TWINKV_OK) return r;
     return main_stages(dev, k16, s, p, bret, t0, out_score_all, out_twin_all, workspace, L, st);
 }
@@ -1024,7 +1026,7 @@ twinkv_status twinkv_repair_host(const void* keys, twinkv_shape s, const uint8_t
         const Layout Lc = layout(sc, TWINKV_OP_REPAIR);
         char* wsb = base + A.ws + b * A.ws_bytes;
         const uint16_t* k16 = nullptr;
-        if ((r = prep_stages(kbuf, sc, d_mask + u0 * N, wsb, Lc, st, &k16)) != TWINKV_OK)
+        if ((r = prep_stages(kbuf, sc, d_mask + u0 * N, need_all, wsb, Lc, st, &k16)) != TWINKV_OK)
             return fail(r);
         r = main_stages(dev, k16, sc, p, d_bret + u0 * N, d_tret + u0 * N,
                         need_all ? d_sall + u0 * N : nullptr, need_all ? d_tall + u0 * N : nullptr,

@@ -89,25 +89,26 @@ constexpr int kDedupMaxN = 1 << 19;
 
 // prep kernels
 // keys: bf16 patterns, or (f32) float32, whose rounded rows also go to keys16 [U][N][d].
-// NP must be a multiple of 64 (column_stride gives a multiple of 256).
+// NP must be a multiple of 256 (as column_stride gives).
 // rscale: a power of two that multiplies every colrinv (1 except for the count mode)
 // unit_kk (zeroed by the caller, or null): receives each unit's largest k.k, as float bits.
 cudaError_t launch_norms_identity(const void* keys, bool f32, uint16_t* keys16, int U, int N,
                                   int d, int64_t NP, float* colrinv, int* colpos,
                                   float4* norms, cudaStream_t st, float rscale = 1.0f,
                                   unsigned* unit_kk = nullptr);
-// Also zeroes unit_kk for launch_gather.
+// Also zeroes unit_kk for launch_gather.  `evicted`: the evicted segment is wanted too.
 cudaError_t launch_scan(const uint8_t* mask, int U, int N, int* cnt, int* kb, unsigned* unit_kk,
                         cudaStream_t st);
 cudaError_t launch_gather(const void* keys, bool f32, uint16_t* keys16, const uint8_t* mask,
                           const int* cnt, const int* kb, int U, int N, int d, int64_t NP,
                           uint16_t* kp, float* colrinv, int* colpos, float4* norms,
-                          unsigned* unit_kk, cudaStream_t st);
+                          unsigned* unit_kk, bool evicted, cudaStream_t st);
 // colrinv of every unit times 2^-e_u, 2^e_u the smallest power of two >= the unit's
 // largest ||k|| (unit_kk as written by the kernels above), so that the audit's scaled
 // similarities lie in [-1, 1] (argmax mode; not for the count mode's scales).
+// kb (or null): only the retained segments.
 cudaError_t launch_scale_columns(float* colrinv, int U, int64_t NP, const unsigned* unit_kk,
-                                 cudaStream_t st);
+                                 const int* kb, cudaStream_t st);
 
 // exact similarity of the chosen twins
 // norms[r] = {k.k hi, k.k lo, 1/||k|| hi, 1/||k|| lo} (double-float pairs) per key, as

@@ -20,7 +20,13 @@ namespace {
 __device__ __forceinline__ float nan_f() { return __uint_as_float(0x7FFFFFFFu); }
 
 constexpr int kPrepThreads = 256;
-constexpr int kKeysPerBlock = kPrepThreads / kParts;   // NP is a multiple of this
+constexpr int kKeysPerStep = kPrepThreads / kParts;
+// Keys per lane group: their loads are issued together, so that 64 bytes per thread are in
+// flight, and the block's reduction and atomic serve them all.
+template <int D>
+constexpr int kKeys = 256 / D;
+template <int D>
+constexpr int kKeysPerBlock = kKeysPerStep * kKeys<D>;   // NP is a multiple of this
 
 // A lane's 16-byte chunks part, part + kParts, ... of a key's bf16 row, from bf16 keys or
 // from float32 ones rounded to nearest even (8 floats per chunk).
@@ -96,7 +102,7 @@ __device__ __forceinline__ void unit_max_kk(unsigned* unit_kk, int64_t u, float 
 // padding columns [N, NP); norms[u][p] = the norm record; unit_kk[u] (if given) =
 // the unit's largest k.k.  float32 keys also leave their rounded rows in keys16: one pass
 // over them, where a separate rounding pass wrote the bf16 keys for this one to read back
-// (16 units of 5003 x 128: 50 -> 18 us with the launches).  Grid (NP / kKeysPerBlock, U),
+// (16 units of 5003 x 128: 50 -> 18 us with the launches).  Grid (NP / kKeysPerBlock<D>, U),
 // kParts lanes per column.
 template <int D, typename Key>
 __global__ void __launch_bounds__(kPrepThreads)
@@ -105,23 +111,35 @@ __global__ void __launch_bounds__(kPrepThreads)
                           float4* __restrict__ norms, float rscale, unsigned* unit_kk,
                           uint16_t* __restrict__ keys16)
 {
+    constexpr int Q = D / 8 / kParts, K = kKeys<D>;
     const int part = threadIdx.x % kParts;
-    const int p = blockIdx.x * kKeysPerBlock + threadIdx.x / kParts;
+    const int p0 = blockIdx.x * kKeysPerBlock<D> + threadIdx.x / kParts;
     const int64_t u = blockIdx.y;
-    // every lane takes part in the shuffles of the norms: padding columns use key 0
-    const int64_t row = u * N + (p < N ? p : 0);
-    uint4 v[D / 8 / kParts];
-    load_key<D>(keys, row, part, v);
-    if constexpr (sizeof(Key) == 4)
-        if (p < N) store_key<D>(keys16, row, part, v);
-    float r32;
-    const float4 nr = key_norms(v, r32);
-    if (part == 0) {
-        colrinv[u * NP + p] = p < N ? r32 * rscale : nan_f();
-        colpos[u * NP + p] = p < N ? p : -1;
-        if (p < N) norms[row] = nr;
+    uint4 v[K][Q];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        // every lane takes part in the shuffles of the norms: padding columns use key 0
+        const int p = p0 + k * kKeysPerStep;
+        load_key<D>(keys, u * N + (p < N ? p : 0), part, v[k]);
     }
-    if (unit_kk) unit_max_kk(unit_kk, u, (part == 0 && p < N) ? nr.x : 0.f);
+    float top = 0.f;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int p = p0 + k * kKeysPerStep;
+        if constexpr (sizeof(Key) == 4)
+            if (p < N) store_key<D>(keys16, u * N + p, part, v[k]);
+        float r32;
+        const float4 nr = key_norms(v[k], r32);
+        if (part == 0) {
+            colrinv[u * NP + p] = p < N ? r32 * rscale : nan_f();
+            colpos[u * NP + p] = p < N ? p : -1;
+            if (p < N) {
+                norms[u * N + p] = nr;
+                top = fmaxf(top, nr.x);
+            }
+        }
+    }
+    if (unit_kk) unit_max_kk(unit_kk, u, top);
 }
 
 constexpr int kScanBytes = 16;   // mask bytes per thread and step
@@ -205,61 +223,83 @@ __global__ void scan_kernel(const uint8_t* __restrict__ mask, int N, int* __rest
 // from the next tile boundary the evicted ones), with 1/||k_p|| (fp32) and p as column
 // metadata, and writes its norm record (and, for float32 keys, its rounded row).  Slots
 // p >= N are the padding columns [K, Kpad) and [Kpad + N - K, NP): zero keys, NaN, -1.
-// unit_kk[u] = the unit's largest k.k.  Grid (NP / kKeysPerBlock, U).
+// Without `evicted` (b_i(all) is not wanted) the audit reads the columns [0, Kpad) only, and
+// only those are written: half of the copy at a ratio of 0.5 (128 units of 8192 x 64:
+// prep 62 -> 45 us; 144 of 8192 x 128, 30 % kept: 110 -> 70).
+// unit_kk[u] = the unit's largest k.k.  Grid (NP / kKeysPerBlock<D>, U).
 template <int D, typename Key>
 __global__ void __launch_bounds__(kPrepThreads)
     gather_kernel(const Key* __restrict__ keys, const uint8_t* __restrict__ mask,
                   const int* __restrict__ cnt, const int* __restrict__ kb, int N, int64_t NP,
                   uint16_t* __restrict__ kp, float* __restrict__ colrinv,
                   int* __restrict__ colpos, float4* __restrict__ norms, unsigned* unit_kk,
-                  uint16_t* __restrict__ keys16)
+                  uint16_t* __restrict__ keys16, bool evicted)
 {
-    constexpr int Q = D / 8 / kParts;   // 16-byte chunks per lane
+    constexpr int Q = D / 8 / kParts, K = kKeys<D>;
     const int part = threadIdx.x % kParts;
-    const int p = blockIdx.x * kKeysPerBlock + threadIdx.x / kParts;
+    const int p0 = blockIdx.x * kKeysPerBlock<D> + threadIdx.x / kParts;
     const int64_t u = blockIdx.y;
-    const int k = kb[u];
-    const int kpad = ((k + kBN - 1) / kBN) * kBN;
-    const int64_t row = u * N + (p < N ? p : 0);   // every lane takes part in the shuffles
-    uint4 v[Q];
-    load_key<D>(keys, row, part, v);
-    int col;
-    if (p < N) {
-        const int before = cnt[row];
-        col = mask[row] ? before : kpad + (p - before);
-    } else {
-        const int r = p - N;
-        col = r < kpad - k ? k + r : kpad + (N - k) + (r - (kpad - k));
-    }
-    if constexpr (sizeof(Key) == 4)
-        if (p < N) store_key<D>(keys16, row, part, v);
-    float r32;
-    const float4 nr = key_norms(v, r32);
-    if (p >= N) {
+    const int kept = kb[u];
+    const int kpad = ((kept + kBN - 1) / kBN) * kBN;
+    uint4 v[K][Q];
+    int before[K], in[K];
 #pragma unroll
-        for (int q = 0; q < Q; ++q) v[q] = make_uint4(0u, 0u, 0u, 0u);
+    for (int k = 0; k < K; ++k) {
+        const int p = p0 + k * kKeysPerStep;
+        const int64_t row = u * N + (p < N ? p : 0);   // every lane takes part in the shuffles
+        load_key<D>(keys, row, part, v[k]);
+        before[k] = cnt[row];
+        in[k] = mask[row];
     }
-    store_key<D>(kp, u * NP + col, part, v);
-    if (part == 0) {
-        colrinv[u * NP + col] = p < N ? r32 : nan_f();
-        colpos[u * NP + col] = p < N ? p : -1;
-        if (p < N) norms[row] = nr;
+    float top = 0.f;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int p = p0 + k * kKeysPerStep;
+        int col;
+        if (p < N) {
+            col = in[k] ? before[k] : kpad + (p - before[k]);
+        } else {
+            const int r = p - N;
+            col = r < kpad - kept ? kept + r : kpad + (N - kept) + (r - (kpad - kept));
+        }
+        if constexpr (sizeof(Key) == 4)
+            if (p < N) store_key<D>(keys16, u * N + p, part, v[k]);
+        float r32;
+        const float4 nr = key_norms(v[k], r32);
+        if (p >= N) {
+#pragma unroll
+            for (int q = 0; q < Q; ++q) v[k][q] = make_uint4(0u, 0u, 0u, 0u);
+        }
+        const bool read = evicted || col < kpad;
+        if (read) store_key<D>(kp, u * NP + col, part, v[k]);
+        if (part == 0) {
+            if (read) {
+                colrinv[u * NP + col] = p < N ? r32 : nan_f();
+                colpos[u * NP + col] = p < N ? p : -1;
+            }
+            if (p < N) {
+                norms[u * N + p] = nr;
+                top = fmaxf(top, nr.x);
+            }
+        }
     }
-    unit_max_kk(unit_kk, u, (part == 0 && p < N) ? nr.x : 0.f);
+    unit_max_kk(unit_kk, u, top);
 }
 
 // colrinv[u][c] *= 2^-e_u, the power of two with 2^e_u >= the largest ||k|| of unit u
 // (from unit_kk), so that every scaled similarity x_ij * colrinv_j = sim(i,j) ||k_i||
 // 2^-e_u lies in [-1, 1].  Exact (a power of two); NaN padding stays NaN.  A unit of
-// zero keys keeps its scale.  Grid (NP / kPrepThreads, U).
+// zero keys keeps its scale.  Given kb, only the retained columns, padded to a tile, are
+// scaled.  Grid (NP / kPrepThreads, U).
 __global__ void __launch_bounds__(kPrepThreads)
     scale_columns_kernel(float* __restrict__ colrinv, int64_t NP,
-                         const unsigned* __restrict__ unit_kk)
+                         const unsigned* __restrict__ unit_kk, const int* __restrict__ kb)
 {
     const int64_t u = blockIdx.y;
     const int64_t c = static_cast<int64_t>(blockIdx.x) * kPrepThreads + threadIdx.x;
     const float kk = __uint_as_float(unit_kk[u]);
-    if (c >= NP || !(kk > 0.f)) return;
+    const int64_t cols = kb ? (static_cast<int64_t>(kb[u]) + kBN - 1) / kBN * kBN : NP;
+    if (c >= cols || !(kk > 0.f)) return;
     int E;
     (void)frexpf(kk, &E);               // kk < 2^E, so ||k|| < 2^ceil(E / 2)
     const int e = (E + 1) >> 1;          // ceil(E / 2), also for E <= 0
@@ -273,7 +313,8 @@ cudaError_t launch_norms_identity(const void* keys, bool f32, uint16_t* keys16, 
                                   float4* norms, cudaStream_t st, float rscale,
                                   unsigned* unit_kk)
 {
-    const dim3 grid(static_cast<unsigned>(NP / kKeysPerBlock), U);
+    const int per = d == 128 ? kKeysPerBlock<128> : kKeysPerBlock<64>;
+    const dim3 grid(static_cast<unsigned>(NP / per), U);
     auto go = [&](auto kernel, auto* k) {
         kernel<<<grid, kPrepThreads, 0, st>>>(k, N, NP, colrinv, colpos, norms, rscale, unit_kk,
                                               keys16);
@@ -288,10 +329,10 @@ cudaError_t launch_norms_identity(const void* keys, bool f32, uint16_t* keys16, 
 }
 
 cudaError_t launch_scale_columns(float* colrinv, int U, int64_t NP, const unsigned* unit_kk,
-                                 cudaStream_t st)
+                                 const int* kb, cudaStream_t st)
 {
     const dim3 grid(static_cast<unsigned>((NP + kPrepThreads - 1) / kPrepThreads), U);
-    scale_columns_kernel<<<grid, kPrepThreads, 0, st>>>(colrinv, NP, unit_kk);
+    scale_columns_kernel<<<grid, kPrepThreads, 0, st>>>(colrinv, NP, unit_kk, kb);
     return cudaGetLastError();
 }
 
@@ -307,12 +348,13 @@ cudaError_t launch_scan(const uint8_t* mask, int U, int N, int* cnt, int* kb, un
 cudaError_t launch_gather(const void* keys, bool f32, uint16_t* keys16, const uint8_t* mask,
                           const int* cnt, const int* kb, int U, int N, int d, int64_t NP,
                           uint16_t* kp, float* colrinv, int* colpos, float4* norms,
-                          unsigned* unit_kk, cudaStream_t st)
+                          unsigned* unit_kk, bool evicted, cudaStream_t st)
 {
-    const dim3 grid(static_cast<unsigned>(NP / kKeysPerBlock), U);
+    const int per = d == 128 ? kKeysPerBlock<128> : kKeysPerBlock<64>;
+    const dim3 grid(static_cast<unsigned>(NP / per), U);
     auto go = [&](auto kernel, auto* k) {
         kernel<<<grid, kPrepThreads, 0, st>>>(k, mask, cnt, kb, N, NP, kp, colrinv, colpos, norms,
-                                              unit_kk, keys16);
+                                              unit_kk, keys16, evicted);
     };
     const float* kf = static_cast<const float*>(keys);
     const uint16_t* kh = static_cast<const uint16_t*>(keys);
