@@ -596,6 +596,7 @@ __global__ void __cluster_dims__(2, 1, 1)
     tc_fence_before();
     cluster_barrier();   // barriers of both CTAs initialised, tensor memory allocated
     tc_fence_after();
+    wait_for_previous();
     const uint32_t tmem = *tmem_slot;
 
     WaitCtl wc;
@@ -1040,8 +1041,8 @@ cudaError_t launch_audit_t(const CUtensorMap& tmA, const CUtensorMap& tmB, const
     cudaError_t e = cudaFuncSetAttribute(audit_kernel<D, kCount, kSym>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e != cudaSuccess) return e;
-    audit_kernel<D, kCount, kSym><<<grid, kThreads, bytes, st>>>(tmA, tmB, a);
-    return cudaGetLastError();
+    return launch_dependent(audit_kernel<D, kCount, kSym>, dim3(grid), kThreads, bytes, st, tmA,
+                            tmB, a);
 }
 
 cudaError_t launch_audit(int d, AuditMode mode, const CUtensorMap& tmA, const CUtensorMap& tmB,
@@ -1064,6 +1065,7 @@ namespace {
 __global__ void slots_to_twins_kernel(const unsigned long long* __restrict__ slots, int64_t n,
                                       int* __restrict__ twin)
 {
+    wait_for_previous();
     const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const unsigned long long sv = slots[i];
@@ -1075,8 +1077,8 @@ cudaError_t launch_slots_to_twins(const unsigned long long* slots, int64_t n, in
                                   cudaStream_t st)
 {
     const int64_t blocks = (n + 255) / 256;
-    slots_to_twins_kernel<<<static_cast<unsigned>(blocks), 256, 0, st>>>(slots, n, twin);
-    return cudaGetLastError();
+    return launch_dependent(slots_to_twins_kernel, dim3(static_cast<unsigned>(blocks)), 256, 0, st,
+                            slots, n, twin);
 }
 
 // ---------------------------------------------------------------- wait probe

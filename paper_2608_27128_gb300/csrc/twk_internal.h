@@ -87,6 +87,30 @@ constexpr float kCountScale = 0x1p32f;
 // Largest N the dedup variant accepts: its walk keeps 2 bits per donor in shared memory.
 constexpr int kDedupMaxN = 1 << 19;
 
+// Every kernel that follows another one of the library on a stream is launched as its
+// programmatic dependent: its blocks are set up while the last ones before it still run, and
+// wait (wait_for_previous in twk_ptx.cuh) before they touch memory.  Each kernel waits at its
+// start, in every thread, so that a kernel's end implies the end of all before it.  A call is
+// five or six kernels of 4 to 10 us on a small cache, where the gaps between them count:
+// one layer 1x8x4096x128 59 -> 49 us per call, policy 16x8x3001x64 198 -> 192, redundancy
+// 2x8x5003x128 125 -> 119, host repair 9x8x8192x128 1003 -> 981.
+template <typename... Params, typename... Args>
+cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem,
+                             cudaStream_t st, Args... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
 // prep kernels
 // keys: bf16 patterns, or (f32) float32, whose rounded rows also go to keys16 [U][N][d].
 // NP must be a multiple of 256 (as column_stride gives).

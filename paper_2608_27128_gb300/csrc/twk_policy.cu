@@ -16,6 +16,7 @@
 //      to it, in position order (warp ballots + a block scan), writing the mask.
 // Counts are read from global memory (N int32 per pass); nothing else is stored.
 #include "twk_internal.h"
+#include "twk_ptx.cuh"
 
 namespace twk {
 namespace {
@@ -66,6 +67,7 @@ __global__ void __launch_bounds__(kPT, 1)
                          int* __restrict__ status)
 {
     static_assert(kPW == 32, "one warp holds the per-warp totals");
+    wait_for_previous();
     __shared__ PolicyShared s;
     const int u = blockIdx.x;
     const int* count = count_all + static_cast<int64_t>(u) * N;
@@ -140,9 +142,8 @@ cudaError_t launch_policy_select(const int* count, int U, int N, const int* budg
                                  int n_recent, uint8_t* out_mask, int* out_status,
                                  cudaStream_t st)
 {
-    policy_select_kernel<<<U, kPT, 0, st>>>(count, N, budget, n_sink, n_recent, out_mask,
-                                            out_status);
-    return cudaGetLastError();
+    return launch_dependent(policy_select_kernel, dim3(U), kPT, 0, st, count, N, budget, n_sink,
+                            n_recent, out_mask, out_status);
 }
 
 }  // namespace twk

@@ -13,6 +13,7 @@
 
 #include "twk_df.cuh"
 #include "twk_internal.h"
+#include "twk_ptx.cuh"
 
 namespace twk {
 namespace {
@@ -111,6 +112,7 @@ __global__ void __launch_bounds__(kPrepThreads)
                           float4* __restrict__ norms, float rscale, unsigned* unit_kk,
                           uint16_t* __restrict__ keys16)
 {
+    wait_for_previous();
     constexpr int Q = D / 8 / kParts, K = kKeys<D>;
     const int part = threadIdx.x % kParts;
     const int p0 = blockIdx.x * kKeysPerBlock<D> + threadIdx.x / kParts;
@@ -152,6 +154,7 @@ constexpr int kScanBytes = 16;   // mask bytes per thread and step
 __global__ void scan_kernel(const uint8_t* __restrict__ mask, int N, int* __restrict__ cnt,
                             int* __restrict__ kb, unsigned* __restrict__ unit_kk)
 {
+    wait_for_previous();
     __shared__ int warp_tot[2][32];
     const int u = blockIdx.x;
     const uint8_t* m = mask + static_cast<int64_t>(u) * N;
@@ -235,6 +238,7 @@ __global__ void __launch_bounds__(kPrepThreads)
                   int* __restrict__ colpos, float4* __restrict__ norms, unsigned* unit_kk,
                   uint16_t* __restrict__ keys16, bool evicted)
 {
+    wait_for_previous();
     constexpr int Q = D / 8 / kParts, K = kKeys<D>;
     const int part = threadIdx.x % kParts;
     const int p0 = blockIdx.x * kKeysPerBlock<D> + threadIdx.x / kParts;
@@ -295,6 +299,7 @@ __global__ void __launch_bounds__(kPrepThreads)
     scale_columns_kernel(float* __restrict__ colrinv, int64_t NP,
                          const unsigned* __restrict__ unit_kk, const int* __restrict__ kb)
 {
+    wait_for_previous();
     const int64_t u = blockIdx.y;
     const int64_t c = static_cast<int64_t>(blockIdx.x) * kPrepThreads + threadIdx.x;
     const float kk = __uint_as_float(unit_kk[u]);
@@ -332,8 +337,8 @@ cudaError_t launch_scale_columns(float* colrinv, int U, int64_t NP, const unsign
                                  const int* kb, cudaStream_t st)
 {
     const dim3 grid(static_cast<unsigned>((NP + kPrepThreads - 1) / kPrepThreads), U);
-    scale_columns_kernel<<<grid, kPrepThreads, 0, st>>>(colrinv, NP, unit_kk, kb);
-    return cudaGetLastError();
+    return launch_dependent(scale_columns_kernel, grid, kPrepThreads, 0, st, colrinv, NP, unit_kk,
+                            kb);
 }
 
 cudaError_t launch_scan(const uint8_t* mask, int U, int N, int* cnt, int* kb, unsigned* unit_kk,
@@ -353,16 +358,15 @@ cudaError_t launch_gather(const void* keys, bool f32, uint16_t* keys16, const ui
     const int per = d == 128 ? kKeysPerBlock<128> : kKeysPerBlock<64>;
     const dim3 grid(static_cast<unsigned>(NP / per), U);
     auto go = [&](auto kernel, auto* k) {
-        kernel<<<grid, kPrepThreads, 0, st>>>(k, mask, cnt, kb, N, NP, kp, colrinv, colpos, norms,
-                                              unit_kk, keys16, evicted);
+        return launch_dependent(kernel, grid, kPrepThreads, 0, st, k, mask, cnt, kb, N, NP, kp,
+                                colrinv, colpos, norms, unit_kk, keys16, evicted);
     };
     const float* kf = static_cast<const float*>(keys);
     const uint16_t* kh = static_cast<const uint16_t*>(keys);
-    if (f32 && d == 128) go(gather_kernel<128, float>, kf);
-    else if (f32) go(gather_kernel<64, float>, kf);
-    else if (d == 128) go(gather_kernel<128, uint16_t>, kh);
-    else go(gather_kernel<64, uint16_t>, kh);
-    return cudaGetLastError();
+    if (f32 && d == 128) return go(gather_kernel<128, float>, kf);
+    if (f32) return go(gather_kernel<64, float>, kf);
+    if (d == 128) return go(gather_kernel<128, uint16_t>, kh);
+    return go(gather_kernel<64, uint16_t>, kh);
 }
 
 }  // namespace twk

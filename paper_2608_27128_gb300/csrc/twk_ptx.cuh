@@ -193,6 +193,17 @@ __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* map)
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
 
+// ---------------------------------------------------------------- dependent launches
+
+// Waits until the kernel before this one on its stream has ended and its writes are visible
+// (at once where the launch was not a programmatic dependent), and lets the next kernel's
+// blocks be set up as soon as every block of this one has started.
+__device__ __forceinline__ void wait_for_previous()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // ---------------------------------------------------------------- registers
 // Every warp of a warpgroup gives up or takes registers (kRegs per thread afterwards).
 

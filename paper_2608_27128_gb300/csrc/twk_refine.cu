@@ -18,6 +18,7 @@
 // (i, j) bit for bit and exactly 1 for a duplicate.
 #include "twk_df.cuh"
 #include "twk_internal.h"
+#include "twk_ptx.cuh"
 
 namespace twk {
 namespace {
@@ -80,6 +81,7 @@ __global__ void __launch_bounds__(kRefineThreads, kMinBlocks)
                   const int* __restrict__ twin0, int* __restrict__ twin1,
                   double* __restrict__ b0, double* __restrict__ b1)
 {
+    wait_for_previous();
     const int part = threadIdx.x % kParts;
     const int i = blockIdx.x * kRowsPerBlock + threadIdx.x / kParts;
     const bool live = i < N;
@@ -131,15 +133,12 @@ cudaError_t launch_refine(const uint16_t* keys, int U, int N, int d, const float
                           cudaStream_t st, bool beside_audit)
 {
     const dim3 grid((N + kRowsPerBlock - 1) / kRowsPerBlock, U);
-    if (d == 128 && beside_audit)
-        refine_kernel<128, 6><<<grid, kRefineThreads, 0, st>>>(keys, N, norms, twin0, twin1, b0, b1);
-    else if (d == 128)
-        refine_kernel<128, 5><<<grid, kRefineThreads, 0, st>>>(keys, N, norms, twin0, twin1, b0, b1);
-    else if (beside_audit)
-        refine_kernel<64, 6><<<grid, kRefineThreads, 0, st>>>(keys, N, norms, twin0, twin1, b0, b1);
-    else
-        refine_kernel<64, 5><<<grid, kRefineThreads, 0, st>>>(keys, N, norms, twin0, twin1, b0, b1);
-    return cudaGetLastError();
+    auto go = [&](auto kernel) {
+        return launch_dependent(kernel, grid, kRefineThreads, 0, st, keys, N, norms, twin0, twin1,
+                                b0, b1);
+    };
+    if (d == 128) return beside_audit ? go(refine_kernel<128, 6>) : go(refine_kernel<128, 5>);
+    return beside_audit ? go(refine_kernel<64, 6>) : go(refine_kernel<64, 5>);
 }
 
 }  // namespace twk

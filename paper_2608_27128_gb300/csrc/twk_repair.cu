@@ -953,6 +953,7 @@ __global__ void __launch_bounds__(kT, 2) select_kernel(const RepairArgs a)
     int r = 0;
     if constexpr (C > 1) r = static_cast<int>(cg::this_cluster().block_rank());
     const int u = static_cast<int>(blockIdx.x / C);
+    wait_for_previous();
     if (select_by_buckets<C>(s, cs, sk_o, reinterpret_cast<int*>(sk_o + 2 * kCap), a, u, r))
         return;
     cluster_sync<C>();   // what the attempt left in shared memory is free
@@ -1361,6 +1362,7 @@ __global__ void __launch_bounds__(kT, 2) select_kernel(const RepairArgs a)
 __global__ void __launch_bounds__(kT, 2) dedup_kernel(const RepairArgs a)   // 2 blocks/SM
 {
     __shared__ Shared s;
+    wait_for_previous();
     const int u = blockIdx.x;
     const int N = a.N;
     const int64_t off = static_cast<int64_t>(u) * N;
@@ -1561,12 +1563,14 @@ cudaError_t config_select(const RepairArgs& a, cudaStream_t st, cudaLaunchConfig
     cfg.blockDim = dim3(kT);
     cfg.dynamicSmemBytes = bytes;
     cfg.stream = st;
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = C;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // as launch_dependent
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = C;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = C > 1 ? 1 : 0;   // one CTA per unit: a plain launch
+    cfg.numAttrs = C > 1 ? 2 : 1;   // one CTA per unit: no cluster
     return cudaSuccess;
 }
 
@@ -1577,7 +1581,7 @@ cudaError_t try_select(const RepairArgs& a, cudaStream_t st, bool* launched)
 {
     *launched = false;
     cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     cudaError_t e = config_select<C>(a, st, cfg, at);
     if (e != cudaSuccess) return e;
     if (C > 1) {
@@ -1636,8 +1640,7 @@ cudaError_t launch_repair(const RepairArgs& a, cudaStream_t st)
     const cudaError_t e = cudaFuncSetAttribute(
         dedup_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
     if (e != cudaSuccess) return e;
-    dedup_kernel<<<a.U, kT, bytes, st>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(dedup_kernel, dim3(a.U), kT, bytes, st, a);
 }
 
 }  // namespace twk
