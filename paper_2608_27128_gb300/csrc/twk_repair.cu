@@ -19,6 +19,7 @@
 //
 // Dedup variant (dedup_kernel, given the twin of every position; one 512-thread block
 // per unit): evicting a donor keeps its twin, so a twin pair never loses both members.
+// Where all donors fit, by buckets too, with the walk in rounds (dedup_swap); else:
 // All donors are sorted; each gets the donor rank of its twin (through a position ->
 // rank table in the workspace); one thread then walks the ranks in severity order with
 // two bits of state per rank in shared memory (evicted, pinned): a donor is skipped
@@ -29,6 +30,8 @@
 // from the top) and sorted: up to 4096 items by a bitonic network in shared memory,
 // more by a stable LSD radix sort (8-bit digits, warp match + per-warp digit counts; a
 // digit position shared by every key is skipped).
+#include <algorithm>
+
 #include <cooperative_groups.h>
 
 #include "twk_internal.h"
@@ -699,9 +702,14 @@ __device__ __forceinline__ void peer_store(int* p, int rank, int v)
                  : "memory");
 }
 
+__device__ void dedup_swap(Shared& s, uint64_t* sk, int* si, const Buckets& bd,
+                           const RepairArgs& a, int u, const int* end, int n_o, uint64_t ktau,
+                           const int (&rank)[2][kCap / kT]);
+
 // Runs the unit by buckets; every thread of the cluster calls it.  False (and, apart from
-// S1 = S0, nothing written) where the unit is left to the general path.
-template <int C>
+// S1 = S0, nothing written) where the unit is left to the general path.  kDedup (C = 1): every
+// donor is in play, not only the m most severe, and dedup_swap ends the unit.
+template <int C, bool kDedup = false>
 __device__ bool select_by_buckets(Shared& s, ClusterShared& cs, uint64_t* sk, int* si,
                                   const RepairArgs& a, int u, int r)
 {
@@ -800,6 +808,9 @@ __device__ bool select_by_buckets(Shared& s, ClusterShared& cs, uint64_t* sk, in
         }
         return true;
     }
+    // ranks in play per side; lists that cannot fit are left at once
+    const int lim_o = m, lim_d = kDedup ? tot[1] : m;
+    if (max(lim_o, lim_d) > C * kCap) return false;
     // side x's bucket: orphans from the smallest b up, donors from the largest down
     const Buckets bo = make_buckets(from_int(ends[0]), from_int(ends[1]));
     const Buckets bd = make_buckets(from_int(ends[3]), from_int(ends[2]));
@@ -852,7 +863,7 @@ __device__ bool select_by_buckets(Shared& s, ClusterShared& cs, uint64_t* sk, in
     for (int k = 0; k < kPer; ++k) {
         base[b0 + k] = run;
         cur[b0 + k] = run;
-        if (run < m) {
+        if (run < (side ? lim_d : lim_o)) {
             full = max(full, c[k]);
             last = max(last, run + c[k]);
         }
@@ -878,7 +889,7 @@ __device__ bool select_by_buckets(Shared& s, ClusterShared& cs, uint64_t* sk, in
             const int x = i < hi ? side_of(mv[j], bv[j], ki, i, a, ktau) : 2;
             if (x == 2) continue;
             const int k = x * kBk + bucket(x, static_cast<uint64_t>(__double_as_longlong(bv[j])));
-            if (base[k] >= m) continue;
+            if (base[k] >= (x ? lim_d : lim_o)) continue;
             const int t = C == 1 ? 0 : base[k] / share;
             if constexpr (C == 1) {
                 const int at = x * kCap + atomicAdd(&cur[k], 1);
@@ -911,31 +922,156 @@ __device__ bool select_by_buckets(Shared& s, ClusterShared& cs, uint64_t* sk, in
         g1[0] = s.sel_digit;
         g1[1] = s.sel_before;
     }
+    // the rank of the item at place g of side x
+    auto rank_of = [&](int x, int g) {
+        const uint64_t key = sk[x * kCap + g % kCap];
+        const int pos = si[x * kCap + g % kCap];
+        const int k = bucket(x, bits_of_key(key, x));
+        const int from_g = base[x * kBk + k];
+        const int to_g = k + 1 < kBk ? base[x * kBk + k + 1] : tot[x];
+        int rank = from_g;
+        for (int h = from_g; h < to_g; ++h) {
+            const int at = x * kCap + h % kCap;
+            rank += before(sk[at], si[at], key, pos) ? 1 : 0;
+        }
+        return rank;
+    };
+    if constexpr (kDedup) {
+        int rank[2][kCap / kT];
 #pragma unroll
-    for (int x = 0; x < 2; ++x) {
+        for (int x = 0; x < 2; ++x)
+#pragma unroll
+            for (int j = 0; j < kCap / kT; ++j) {
+                const int g = tid + j * kT;
+                rank[x][j] = g < end[x] ? rank_of(x, g) : -1;
+            }
+        dedup_swap(s, sk, si, bd, a, u, end, tot[0], ktau, rank);
+    } else {
         int* swaps = a.out_swaps + static_cast<int64_t>(u) * 2 * (a.N / 2);
-        for (int g = g0[x] + tid; g < g1[x]; g += kT) {
-            const uint64_t key = sk[x * kCap + g % kCap];
-            const int pos = si[x * kCap + g % kCap];
-            const int k = bucket(x, bits_of_key(key, x));
-            const int from_g = base[x * kBk + k];
-            const int to_g = k + 1 < kBk ? base[x * kBk + k + 1] : tot[x];
-            int rank = from_g;
-            for (int h = from_g; h < to_g; ++h) {
-                const int at = x * kCap + h % kCap;
-                rank += before(sk[at], si[at], key, pos) ? 1 : 0;
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+            for (int g = g0[x] + tid; g < g1[x]; g += kT) {
+                const int rank = rank_of(x, g), pos = si[x * kCap + g % kCap];
+                if (rank < m) {
+                    swaps[2 * rank + (x ? 0 : 1)] = pos;
+                    S1[pos] = x ? 0 : 1;
+                }
             }
-            if (rank < m) {
-                swaps[2 * rank + (x ? 0 : 1)] = pos;
-                S1[pos] = x ? 0 : 1;
-            }
+        if (r == 0 && tid == 0) {
+            a.out_nswaps[u] = m;
+            if (a.out_status) a.out_status[u] = 0;
         }
     }
-    if (r == 0 && tid == 0) {
+    return true;
+}
+
+// The end of the dedup variant's bucket path: the walk over the donors in severity order as
+// rounds over all of them.  A donor conflicts with its twin, and with the donors whose twin
+// it is; it is evicted unless a more severe one that it conflicts with is.  In each round an
+// edge (donor, its twin) whose more severe end is evicted rejects the other end, one whose
+// more severe end is undecided holds the other end back, and every undecided donor that
+// nothing holds back is evicted: the same set as the walk's.  Twins are mostly mutual, so a
+// few rounds decide all; a chain longer than kRounds is finished by one thread in rank
+// order.  (The walk by one thread took about half of the kernel's 78 us at 144 units of 8192.)
+// rank: the ranks of the thread's items, places tid + j kT.  The keys at sk are no longer
+// needed: their memory takes the lists by rank.
+constexpr int kRounds = 64;
+
+__device__ void dedup_swap(Shared& s, uint64_t* sk, int* si, const Buckets& bd,
+                           const RepairArgs& a, int u, const int* end, int n_o, uint64_t ktau,
+                           const int (&rank)[2][kCap / kT])
+{
+    const int tid = threadIdx.x, N = a.N, n_d = end[1];
+    const int64_t off = static_cast<int64_t>(u) * N;
+    const int* base = &s.warp_cnt[0][0] + kBk;   // the donors' buckets
+    uint8_t* state = reinterpret_cast<uint8_t*>(&s.warp_cnt[0][0] + 2 * kBk);   // by rank
+    uint8_t* held = state + kCap;
+    static_assert(2 * kCap <= 2 * kBk * 4, "state and held take the place of the cursors");
+    int* orph = reinterpret_cast<int*>(sk);   // [kCap] orphans by rank
+    int* don = orph + kCap;                   // [kCap] donors by rank
+    int* rank_at = don + kCap;                // [kCap] rank of the donor at each place
+    int* twin = rank_at + kCap;               // [kCap] by rank: the rank of the donor's twin
+    __syncthreads();                          // every rank has been counted
+#pragma unroll
+    for (int j = 0; j < kCap / kT; ++j) {
+        const int g = tid + j * kT;
+        if (rank[0][j] >= 0) orph[rank[0][j]] = si[g];
+        if (rank[1][j] >= 0) {
+            don[rank[1][j]] = si[kCap + g];
+            rank_at[g] = rank[1][j];
+        }
+    }
+    for (int k = tid; k < n_d; k += kT) state[k] = 0;   // 1: evicted, 2: rejected
+    __syncthreads();
+    for (int k = tid; k < n_d; k += kT) {
+        const int t = a.twin[off + don[k]];
+        int r = -1;
+        if (t >= 0 && t < N) {
+            const double bt = a.b[off + t];
+            if (side_of(a.mask[off + t], bt, ordered(bt), t, a, ktau) == 1) {
+                const int bk = bucket_of(narrow(static_cast<uint64_t>(__double_as_longlong(bt))), bd);
+                const int to = bk + 1 < kBk ? base[bk + 1] : n_d;
+                for (int g = base[bk]; g < to; ++g)
+                    if (si[kCap + g] == t) r = rank_at[g];
+            }
+        }
+        twin[k] = r == k ? -1 : r;
+    }
+    __syncthreads();
+    int undecided = 1;
+    for (int round = 0; round < kRounds && undecided; ++round) {
+        for (int k = tid; k < n_d; k += kT) held[k] = 0;
+        __syncthreads();
+        for (int k = tid; k < n_d; k += kT) {
+            const int t = twin[k];
+            if (t < 0) continue;
+            const int first = state[min(k, t)];
+            if (first == 1) state[max(k, t)] = 2;
+            else if (first == 0) held[max(k, t)] = 1;
+        }
+        __syncthreads();
+        int left = 0;
+        for (int k = tid; k < n_d; k += kT)
+            if (state[k] == 0) {
+                if (held[k]) left = 1;
+                else state[k] = 1;
+            }
+        undecided = __syncthreads_or(left);
+    }
+    if (undecided) {
+        if (tid == 0)
+            for (int k = 0; k < n_d; ++k) {
+                const int t = twin[k];
+                if (state[k] == 0) state[k] = t >= 0 && t < k && state[t] == 1 ? 2 : 1;
+                if (state[k] == 1 && t > k) state[t] = 2;
+            }
+        __syncthreads();
+    }
+    // the first n_o evictions in rank order
+    int* out = rank_at;
+    int total = 0;
+    for (int c0 = 0; c0 < n_d; c0 += kT) {
+        const int k = c0 + tid;
+        const int f = k < n_d && state[k] == 1;
+        int p, q, to, tq;
+        scan2(s, f, 0, p, q, to, tq);
+        if (f) out[total + p] = don[k];
+        total += to;
+    }
+    __syncthreads();
+    const int m = min(total, n_o);
+    uint8_t* S1 = a.out_mask + off;
+    int* swaps = a.out_swaps + static_cast<int64_t>(u) * 2 * (N / 2);
+    for (int k = tid; k < m; k += kT) {
+        swaps[2 * k] = out[k];
+        swaps[2 * k + 1] = orph[k];
+        S1[out[k]] = 0;
+        S1[orph[k]] = 1;
+    }
+    if (tid == 0) {
         a.out_nswaps[u] = m;
         if (a.out_status) a.out_status[u] = 0;
     }
-    return true;
 }
 
 template <int C>
@@ -1362,8 +1498,14 @@ __global__ void __launch_bounds__(kT, 2) select_kernel(const RepairArgs a)
 __global__ void __launch_bounds__(kT, 2) dedup_kernel(const RepairArgs a)   // 2 blocks/SM
 {
     __shared__ Shared s;
+    __shared__ ClusterShared cs;
+    extern __shared__ __align__(16) uint32_t dyn[];
     wait_for_previous();
     const int u = blockIdx.x;
+    if (uint64_t* keys = reinterpret_cast<uint64_t*>(dyn); select_by_buckets<1, true>(
+            s, cs, keys, reinterpret_cast<int*>(keys + 2 * kCap), a, u, 0))
+        return;
+    __syncthreads();   // what the attempt left in shared memory is free
     const int N = a.N;
     const int64_t off = static_cast<int64_t>(u) * N;
     const uint8_t* S0 = a.mask + off;
@@ -1469,7 +1611,6 @@ __global__ void __launch_bounds__(kT, 2) dedup_kernel(const RepairArgs a)   // 2
     __syncthreads();
 
     // 4. the m most severe orphans and donors, in severity order
-    extern __shared__ __align__(16) uint32_t dyn[];
     uint64_t* sk = reinterpret_cast<uint64_t*>(
         reinterpret_cast<unsigned char*>(dyn) + sort_smem_offset(N));
     int* si = reinterpret_cast<int*>(sk + kSortMax);
@@ -1636,7 +1777,7 @@ cudaError_t launch_repair(const RepairArgs& a, cudaStream_t st)
         return cudaSuccess;
     }
     if (a.N > kDedupMaxN) return cudaErrorInvalidValue;
-    const size_t bytes = dedup_kernel_smem_bytes(a.N);
+    const size_t bytes = std::max(dedup_kernel_smem_bytes(a.N), 2 * static_cast<size_t>(kCap) * 12);
     const cudaError_t e = cudaFuncSetAttribute(
         dedup_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
     if (e != cudaSuccess) return e;
