@@ -1,23 +1,14 @@
 // twk_df.cuh -- double-float arithmetic (an unevaluated sum of two floats) and the one
-// dot-product routine behind every exact similarity value of the TwinKV pass: bf16 x
+// dot-product scheme behind every exact similarity value of the TwinKV pass: bf16 x
 // bf16 products are exact in fp32 and are accumulated with Knuth's TwoSum, four lanes
 // per dot product, each over every fourth 16-byte chunk, combined in a fixed tree.  Every
-// dot product (norms included) goes through group_dot_df, so identical keys give
+// dot product (norms included) takes its terms in the same order, so identical keys give
 // identical values and the value of k_i . k_j equals that of k_j . k_i bit for bit.
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
 
 namespace twk {
-
-__device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float p)
-{
-    const float s = __fadd_rn(hi, p);
-    const float bp = __fsub_rn(s, hi);
-    const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bp)), __fsub_rn(p, bp));
-    hi = s;
-    lo = __fadd_rn(lo, e);
-}
 
 // An unevaluated sum hi + lo of two floats (a double-float).
 struct DFPair {
@@ -38,83 +29,9 @@ __device__ __forceinline__ void df_add(float& hi, float& lo, float hi2, float lo
 
 constexpr int kParts = 4;   // threads per dot product, each over every fourth 16-byte chunk
 
-// One lane's part of a . b for two bf16 rows of length D: the 16-byte chunks part,
-// part + kParts, part + 2 kParts, ... (so that the kParts lanes of a dot product read
-// kParts * 16 contiguous bytes per load), terms in increasing t.
-template <int D>
-__device__ __forceinline__ void quarter_dot(const uint16_t* __restrict__ a,
-                                            const uint16_t* __restrict__ b, int part,
-                                            float& hi, float& lo)
-{
-    constexpr int Q = D / 8 / kParts;   // 16-byte chunks per lane
-    const uint4* a4 = reinterpret_cast<const uint4*>(a) + part;
-    const uint4* b4 = reinterpret_cast<const uint4*>(b) + part;
-    hi = 0.f;
-    lo = 0.f;
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-        const uint4 va = __ldg(a4 + q * kParts);
-        const uint4 vb = __ldg(b4 + q * kParts);
-        const uint32_t wa[4] = {va.x, va.y, va.z, va.w};
-        const uint32_t wb[4] = {vb.x, vb.y, vb.z, vb.w};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            // element 2k (low half) then 2k+1 (high half) of this 16-byte chunk
-            two_sum_acc(hi, lo, __fmul_rn(__uint_as_float(wa[k] << 16), __uint_as_float(wb[k] << 16)));
-            two_sum_acc(hi, lo, __fmul_rn(__uint_as_float(wa[k] & 0xFFFF0000u),
-                                          __uint_as_float(wb[k] & 0xFFFF0000u)));
-        }
-    }
-}
-
-// The same for a . a with the lane's 16-byte chunks already in registers.
-template <int Q>
-__device__ __forceinline__ void quarter_square(const uint4 (&v)[Q], float& hi, float& lo)
-{
-    hi = 0.f;
-    lo = 0.f;
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-        const uint32_t w[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const float e = __uint_as_float(w[k] << 16), o = __uint_as_float(w[k] & 0xFFFF0000u);
-            two_sum_acc(hi, lo, __fmul_rn(e, e));
-            two_sum_acc(hi, lo, __fmul_rn(o, o));
-        }
-    }
-}
-
-// The lanes' parts of one dot product summed as ((q0 + q1) + (q2 + q3)).
-__device__ __forceinline__ DFPair group_sum(float hi, float lo)
-{
-#pragma unroll
-    for (int o = 1; o < kParts; o <<= 1) {
-        const float h2 = __shfl_xor_sync(0xFFFFFFFFu, hi, o);
-        const float l2 = __shfl_xor_sync(0xFFFFFFFFu, lo, o);
-        df_add(hi, lo, h2, l2);
-    }
-    return DFPair{hi, lo};
-}
-
-// a . b by the kParts consecutive lanes of a group (every lane passes its part): the
-// lanes' parts are summed as ((q0 + q1) + (q2 + q3)), and every lane of the group returns
-// the same double-float.  All dot products, norms included, take their terms in this order.
-template <int D>
-__device__ __forceinline__ DFPair group_dot_df(const uint16_t* __restrict__ a,
-                                             const uint16_t* __restrict__ b, int part)
-{
-    float hi, lo;
-    quarter_dot<D>(a, b, part, hi, lo);
-    return group_sum(hi, lo);
-}
-
-// The same two dot products a . b0 and a . b1 at once, one in each half of paired
-// (f32x2) instructions: each half performs exactly the scalar sequence of
-// group_dot_df, with the same rounding, term order and combine tree, so each result
-// equals group_dot_df's bit for bit.
 __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 
+// (hi, lo) + p in both halves: Knuth's TwoSum on the high parts, its error added to lo.
 __device__ __forceinline__ void two_sum_acc2(float2& hi, float2& lo, float2 p)
 {
     const float2 s = __fadd2_rn(hi, p);
@@ -125,17 +42,69 @@ __device__ __forceinline__ void two_sum_acc2(float2& hi, float2& lo, float2 p)
     lo = __fadd2_rn(lo, e);
 }
 
-__device__ __forceinline__ void df_add2(float2& hi, float2& lo, float2 hi2, float2 lo2)
+// The two bf16 elements of a word, in order, as fp32.
+__device__ __forceinline__ float2 unpack2(uint32_t w)
 {
-    const float2 s = __fadd2_rn(hi, hi2);
-    const float2 bp = __fadd2_rn(s, neg2(hi));
-    float2 e = __fadd2_rn(__fadd2_rn(hi, neg2(__fadd2_rn(s, neg2(bp)))), __fadd2_rn(hi2, neg2(bp)));
-    e = __fadd2_rn(e, __fadd2_rn(lo, lo2));
-    hi = __fadd2_rn(s, e);
-    lo = __fadd2_rn(e, neg2(__fadd2_rn(hi, neg2(s))));
+    return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
 }
 
-// b1 is read only where use1 (elsewhere its terms are zero and r1 is meaningless).
+// One lane's part of a dot product of two bf16 rows of length D: the 16-byte chunks part,
+// part + kParts, part + 2 kParts, ... (so that the kParts lanes of a dot product read
+// kParts * 16 contiguous bytes per load), even and odd elements in the two halves of paired
+// (f32x2) instructions, terms in increasing order.
+struct DotAcc {
+    float2 hi = make_float2(0.f, 0.f), lo = make_float2(0.f, 0.f);
+
+    __device__ __forceinline__ void add(const uint4& a, const uint4& b)
+    {
+        const uint32_t wa[4] = {a.x, a.y, a.z, a.w}, wb[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) two_sum_acc2(hi, lo, __fmul2_rn(unpack2(wa[k]), unpack2(wb[k])));
+    }
+
+    // The halves, then the lanes' parts as ((q0 + q1) + (q2 + q3)); every lane of the group
+    // returns the same double-float.
+    __device__ __forceinline__ DFPair sum() const
+    {
+        float h = hi.x, l = lo.x;
+        df_add(h, l, hi.y, lo.y);
+#pragma unroll
+        for (int o = 1; o < kParts; o <<= 1) {
+            const float h2 = __shfl_xor_sync(0xFFFFFFFFu, h, o);
+            const float l2 = __shfl_xor_sync(0xFFFFFFFFu, l, o);
+            df_add(h, l, h2, l2);
+        }
+        return DFPair{h, l};
+    }
+};
+
+// a . b by the kParts consecutive lanes of a group (every lane passes its part).  All dot
+// products, norms included, take their terms in this order.
+template <int D>
+__device__ __forceinline__ DFPair group_dot_df(const uint16_t* __restrict__ a,
+                                               const uint16_t* __restrict__ b, int part)
+{
+    constexpr int Q = D / 8 / kParts;   // 16-byte chunks per lane
+    const uint4* a4 = reinterpret_cast<const uint4*>(a) + part;
+    const uint4* b4 = reinterpret_cast<const uint4*>(b) + part;
+    DotAcc s;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) s.add(__ldg(a4 + q * kParts), __ldg(b4 + q * kParts));
+    return s.sum();
+}
+
+// a . a with the lane's chunks already in registers.
+template <int Q>
+__device__ __forceinline__ DFPair group_square_df(const uint4 (&v)[Q])
+{
+    DotAcc s;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) s.add(v[q], v[q]);
+    return s.sum();
+}
+
+// a . b0 and a . b1 at once, each exactly as group_dot_df gives it.  b1 is read only where
+// use1 (elsewhere its terms are zero and r1 is meaningless).
 template <int D>
 __device__ __forceinline__ void group_dot2_df(const uint16_t* __restrict__ a,
                                               const uint16_t* __restrict__ b0,
@@ -146,37 +115,17 @@ __device__ __forceinline__ void group_dot2_df(const uint16_t* __restrict__ a,
     const uint4* a4 = reinterpret_cast<const uint4*>(a) + part;
     const uint4* c4 = reinterpret_cast<const uint4*>(b0) + part;
     const uint4* d4 = reinterpret_cast<const uint4*>(b1) + part;
-    float2 hi = make_float2(0.f, 0.f), lo = make_float2(0.f, 0.f);
+    DotAcc s0, s1;
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
         const uint4 va = __ldg(a4 + q * kParts);
         const uint4 vc = __ldg(c4 + q * kParts);
         const uint4 vd = use1 ? __ldg(d4 + q * kParts) : make_uint4(0u, 0u, 0u, 0u);
-        const uint32_t wa[4] = {va.x, va.y, va.z, va.w};
-        const uint32_t wc[4] = {vc.x, vc.y, vc.z, vc.w};
-        const uint32_t wd[4] = {vd.x, vd.y, vd.z, vd.w};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const float lo_a = __uint_as_float(wa[k] << 16);
-            const float hi_a = __uint_as_float(wa[k] & 0xFFFF0000u);
-            two_sum_acc2(hi, lo, __fmul2_rn(make_float2(lo_a, lo_a),
-                                            make_float2(__uint_as_float(wc[k] << 16),
-                                                        __uint_as_float(wd[k] << 16))));
-            two_sum_acc2(hi, lo, __fmul2_rn(make_float2(hi_a, hi_a),
-                                            make_float2(__uint_as_float(wc[k] & 0xFFFF0000u),
-                                                        __uint_as_float(wd[k] & 0xFFFF0000u))));
-        }
+        s0.add(va, vc);
+        s1.add(va, vd);
     }
-#pragma unroll
-    for (int o = 1; o < kParts; o <<= 1) {
-        const float2 h2 = make_float2(__shfl_xor_sync(0xFFFFFFFFu, hi.x, o),
-                                      __shfl_xor_sync(0xFFFFFFFFu, hi.y, o));
-        const float2 l2 = make_float2(__shfl_xor_sync(0xFFFFFFFFu, lo.x, o),
-                                      __shfl_xor_sync(0xFFFFFFFFu, lo.y, o));
-        df_add2(hi, lo, h2, l2);
-    }
-    r0 = DFPair{hi.x, lo.x};
-    r1 = DFPair{hi.y, lo.y};
+    r0 = s0.sum();
+    r1 = s1.sum();
 }
 
 // ---- double-float (unevaluated fp32 pair) helpers --------------------------------

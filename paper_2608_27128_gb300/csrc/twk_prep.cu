@@ -22,10 +22,11 @@ __device__ __forceinline__ float nan_f() { return __uint_as_float(0x7FFFFFFFu); 
 
 constexpr int kPrepThreads = 256;
 constexpr int kKeysPerStep = kPrepThreads / kParts;
-// Keys per lane group: their loads are issued together, so that 64 bytes per thread are in
-// flight, and the block's reduction and atomic serve them all.
+// Keys per lane group: 64 bytes of loads per thread are in flight, and the block's reduction
+// and atomic serve them all (twice as many keys, or blocks of 128 threads, measured within
+// 3 % either way).
 template <int D>
-constexpr int kKeys = 256 / D;
+constexpr int kKeys = 128 / D;
 template <int D>
 constexpr int kKeysPerBlock = kKeysPerStep * kKeys<D>;   // NP is a multiple of this
 
@@ -72,9 +73,7 @@ __device__ __forceinline__ void store_key(uint16_t* out, int64_t row, int part,
 template <int Q>
 __device__ __forceinline__ float4 key_norms(const uint4 (&v)[Q], float& rinv32)
 {
-    float hi, lo;
-    quarter_square(v, hi, lo);
-    const DF sq = group_sum(hi, lo);
+    const DF sq = group_square_df(v);
     const DF rn = sq.h > 0.f ? df_rsqrt(sq) : DF{0.f, 0.f};
     rinv32 = rn.h;
     return make_float4(sq.h, sq.l, rn.h, rn.l);
@@ -228,7 +227,7 @@ __global__ void scan_kernel(const uint8_t* __restrict__ mask, int N, int* __rest
 // p >= N are the padding columns [K, Kpad) and [Kpad + N - K, NP): zero keys, NaN, -1.
 // Without `evicted` (b_i(all) is not wanted) the audit reads the columns [0, Kpad) only, and
 // only those are written: half of the copy at a ratio of 0.5 (128 units of 8192 x 64:
-// prep 62 -> 45 us; 144 of 8192 x 128, 30 % kept: 110 -> 70).
+// prep 61 -> 58 us; 144 of 8192 x 128, 30 % kept: 110 -> 91).
 // unit_kk[u] = the unit's largest k.k.  Grid (NP / kKeysPerBlock<D>, U).
 template <int D, typename Key>
 __global__ void __launch_bounds__(kPrepThreads)

@@ -64,7 +64,7 @@ __device__ __forceinline__ DF cosine(DF dot, float4 ni, float4 nj)
     return DF{h, static_cast<float>(x - static_cast<double>(h))};
 }
 
-constexpr int kRefineThreads = 256;
+constexpr int kRefineThreads = 128;
 constexpr int kRowsPerBlock = kRefineThreads / kParts;
 
 // For every row (u, i): b0 = sim(i, twin0), -1 where twin0 is -1 (empty candidate
@@ -72,11 +72,17 @@ constexpr int kRowsPerBlock = kRefineThreads / kParts;
 // reach the retained best) given, the best over all columns is the larger of
 // sim(i, twin0) and sim(i, twin1), the lower position on an exact tie; twin1 is
 // overwritten with it and b1 (if given) receives its value.  Grid: (row blocks, units),
-// kParts threads per row.  kMinBlocks = 5 (at most 51 registers) is the standalone
-// launch; 6 caps the registers at 40 so that a block fits on an SM beside a persistent
-// audit CTA.
+// kParts threads per row.  Bound by the gathers of 256-byte rows from L2 (about 7 TB/s at
+// 18x8x8192x128) and, with both candidates, by the TwoSum instructions.  kMinBlocks is the
+// number of 256 threads that fit on an SM: 5 (48 registers) for one candidate, 4 (64) where
+// rows have two, whose sums need 8 registers more; 6 (40) fits beside a CTA of at most 168
+// registers and 320 threads.  Blocks of 128 threads leave less of an SM waiting for its
+// slowest rows than blocks of 256: 82 against 86 us at 18x8x8192x128, 53 against 56 at
+// 16x8x8192x64, 221 against 232 with both candidates at 16x8x16384x128 (64 threads: 83, 72,
+// 217).  With even and odd elements summed in the halves of paired instructions, one
+// candidate went from 92 to 82 us and 62 to 53; two stay at 212 to 221.
 template <int D, int kMinBlocks>
-__global__ void __launch_bounds__(kRefineThreads, kMinBlocks)
+__global__ void __launch_bounds__(kRefineThreads, kMinBlocks * 256 / kRefineThreads)
     refine_kernel(const uint16_t* __restrict__ keys, int N, const float4* __restrict__ norms,
                   const int* __restrict__ twin0, int* __restrict__ twin1,
                   double* __restrict__ b0, double* __restrict__ b1)
@@ -137,8 +143,11 @@ cudaError_t launch_refine(const uint16_t* keys, int U, int N, int d, const float
         return launch_dependent(kernel, grid, kRefineThreads, 0, st, keys, N, norms, twin0, twin1,
                                 b0, b1);
     };
-    if (d == 128) return beside_audit ? go(refine_kernel<128, 6>) : go(refine_kernel<128, 5>);
-    return beside_audit ? go(refine_kernel<64, 6>) : go(refine_kernel<64, 5>);
+    if (d == 128)
+        return beside_audit ? go(refine_kernel<128, 6>)
+                            : twin1 ? go(refine_kernel<128, 4>) : go(refine_kernel<128, 5>);
+    return beside_audit ? go(refine_kernel<64, 6>)
+                        : twin1 ? go(refine_kernel<64, 4>) : go(refine_kernel<64, 5>);
 }
 
 }  // namespace twk
