@@ -11,6 +11,7 @@ Sec. 3.4 (Eq. 4, orphans, donors, the budget-exact swap).
 from __future__ import annotations
 
 import ctypes
+import functools
 import math
 import os
 import threading
@@ -68,6 +69,8 @@ def library_path() -> str:
 def load(build_if_missing: bool = True):
     """Load libtwinkv.so (building it with nvcc first when it is missing or stale)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -139,16 +142,20 @@ def _check(status: int, what: str):
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
     if stream is None:
         stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    return stream.cuda_stream
 
 
 def _need(t, name, dtype, shape, device):
+    # what a call with valid tensors passes, before the checks that name what is wrong
+    if (isinstance(t, torch.Tensor) and t.dtype is dtype and t.is_cuda and t.shape == shape
+            and t.device == device and t.is_contiguous()):
+        return t
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a torch tensor")
     if t.device != device or not t.is_cuda:
@@ -189,8 +196,13 @@ def twinkv_swaps_capacity(shape: Shape) -> int:
     return int(load().twinkv_swaps_capacity(shape))
 
 
+@functools.lru_cache(maxsize=1024)
+def _workspace_size(L, H, N, d, dtype, op) -> int:
+    return int(load().twinkv_workspace_size(Shape(L, H, N, d, dtype), op))
+
+
 def twinkv_workspace_size(shape: Shape, op: int) -> int:
-    return int(load().twinkv_workspace_size(shape, int(op)))
+    return _workspace_size(shape.L, shape.H, shape.N, shape.d, shape.dtype, int(op))
 
 
 def workspace(shape: Shape, op: int, device) -> torch.Tensor:
@@ -244,9 +256,15 @@ def twinkv_redundancy_symmetric(keys, window: int = 32, out_score=None, out_twin
     return out_score, out_twin
 
 
+@functools.lru_cache(maxsize=1)
+def _defaults():
+    p = twinkv_default_params()
+    return p.threshold, p.window, p.n_sink, p.n_recent
+
+
 def _params(params, threshold, window, n_sink, n_recent):
-    p = twinkv_default_params() if params is None else params
-    p = Params(p.threshold, p.window, p.n_sink, p.n_recent)
+    p = Params(*(_defaults() if params is None else
+                 (params.threshold, params.window, params.n_sink, params.n_recent)))
     if threshold is not None:
         p.threshold = float(threshold)
     if window is not None:
@@ -299,7 +317,7 @@ def twinkv_repair(keys, retained_mask, budget=None, threshold=None, params=None,
         o["twin_all"] = _out(out.get("twin_all"), "twin_all", torch.int32, (L, H, N), dev)
     ws = _ws(ws, s, OP_REPAIR, dev)
     st = getattr(load(), _fn)(
-        _ptr(keys), s, _ptr(retained_mask), _ptr(budget), ctypes.c_float(p.threshold),
+        _ptr(keys), s, _ptr(retained_mask), _ptr(budget), p.threshold,
         ctypes.byref(p), _ptr(o["mask"]), _ptr(o["swaps"]), _ptr(o["nswaps"]),
         _ptr(o.get("score_ret")), _ptr(o.get("twin_ret")), _ptr(o.get("score_all")),
         _ptr(o.get("twin_all")), _ptr(o["status"]), _ptr(ws), ws.numel(), _stream(stream))
@@ -332,7 +350,7 @@ def twinkv_repair_select_dedup(score_ret, twin_ret, retained_mask, budget=None, 
     ws = _ws(ws, s, OP_REPAIR_SELECT_DEDUP, dev)
     st = load().twinkv_repair_select_dedup(
         _ptr(score_ret), _ptr(twin_ret), s, _ptr(retained_mask), _ptr(budget),
-        ctypes.c_float(p.threshold), ctypes.byref(p), _ptr(o["mask"]), _ptr(o["swaps"]),
+        p.threshold, ctypes.byref(p), _ptr(o["mask"]), _ptr(o["swaps"]),
         _ptr(o["nswaps"]), _ptr(o["status"]), _ptr(ws), ws.numel(), _stream(stream))
     _check(st, "twinkv_repair_select_dedup")
     return o
@@ -361,7 +379,7 @@ def twinkv_repair_select(score_ret, retained_mask, budget=None, threshold=None, 
     }
     ws = _ws(ws, s, OP_REPAIR_SELECT, dev)
     st = load().twinkv_repair_select(
-        _ptr(score_ret), s, _ptr(retained_mask), _ptr(budget), ctypes.c_float(p.threshold),
+        _ptr(score_ret), s, _ptr(retained_mask), _ptr(budget), p.threshold,
         ctypes.byref(p), _ptr(o["mask"]), _ptr(o["swaps"]), _ptr(o["nswaps"]),
         _ptr(o["status"]), _ptr(ws), ws.numel(), _stream(stream))
     _check(st, "twinkv_repair_select")
@@ -394,7 +412,7 @@ def twinkv_repair_select_noalloc(score_ret, retained_mask, budget=None, threshol
         "status": _out(out.get("status"), "status", torch.int32, (L * H,), dev),
     }
     st = load().twinkv_repair_select_noalloc(
-        _ptr(score_ret), s, _ptr(retained_mask), _ptr(budget), ctypes.c_float(p.threshold),
+        _ptr(score_ret), s, _ptr(retained_mask), _ptr(budget), p.threshold,
         ctypes.byref(p), _ptr(o["mask"]), _ptr(o["swaps"]), _ptr(o["nswaps"]),
         _ptr(o["status"]), _stream(stream))
     _check(st, "twinkv_repair_select_noalloc")
@@ -431,7 +449,7 @@ def twinkv_policy(keys, budget, threshold=None, params=None, *, window=None, n_s
         o["count"] = _out(out.get("count"), "count", torch.int32, (L, H, N), dev)
     ws = _ws(ws, s, OP_POLICY, dev)
     st = load().twinkv_policy(
-        _ptr(keys), s, _ptr(budget), ctypes.c_float(p.threshold), ctypes.byref(p),
+        _ptr(keys), s, _ptr(budget), p.threshold, ctypes.byref(p),
         _ptr(o["mask"]), _ptr(o.get("count")), _ptr(o["status"]), _ptr(ws), ws.numel(),
         _stream(stream))
     _check(st, "twinkv_policy")
@@ -531,7 +549,7 @@ def twinkv_repair_host(keys, retained_mask, budget=None, threshold=None, params=
     if not arena.is_cuda or arena.dtype != torch.uint8:
         raise ValueError("arena must be a CUDA uint8 tensor")
     st = load().twinkv_repair_host(
-        _ptr(keys), s, _ptr(retained_mask), _ptr(budget), ctypes.c_float(p.threshold),
+        _ptr(keys), s, _ptr(retained_mask), _ptr(budget), p.threshold,
         ctypes.byref(p), _ptr(o["mask"]), _ptr(o["swaps"]), _ptr(o["nswaps"]),
         _ptr(o.get("score_ret")), _ptr(o.get("twin_ret")), _ptr(o.get("score_all")),
         _ptr(o.get("twin_all")), _ptr(o["status"]), int(chunk_units), _ptr(arena),
