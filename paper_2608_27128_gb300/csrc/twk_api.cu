@@ -699,7 +699,7 @@ namespace {
 // The audit's inputs in `workspace`: bf16 keys (fp32 keys are rounded), the retained
 // prefix counts, and the retained-first column layout with its metadata and the norm
 // records.  *k16 receives the bf16 keys.
-twinkv_status prep_stages(const void* keys, const twinkv_shape& s, const uint8_t* retained_mask,
+twinkv_status prep_stages(const DeviceInfo* dev, const void* keys, const twinkv_shape& s, const uint8_t* retained_mask,
                           bool need_all, void* workspace, const Layout& L, cudaStream_t st,
                           const uint16_t** k16)
 {
@@ -710,6 +710,14 @@ twinkv_status prep_stages(const void* keys, const twinkv_shape& s, const uint8_t
     unsigned* ukk = at<unsigned>(workspace, L.ukk);
     {
         ProfScope pr(TWINKV_KERNEL_PREP, st);
+        bool launched = false;
+        if (launch_prep_unit(keys, s.dtype == TWINKV_F32, rows, retained_mask,
+                             at<int>(workspace, L.cnt), at<int>(workspace, L.kb), U, s.N, s.d, NP,
+                             at<uint16_t>(workspace, L.kp), at<float>(workspace, L.colrinv),
+                             at<int>(workspace, L.colpos), at<float4>(workspace, L.norm2),
+                             need_all, dev->sms, st, &launched) != cudaSuccess)
+            return TWINKV_ERR_CUDA;
+        if (launched) return TWINKV_OK;
         if (launch_scan(retained_mask, U, s.N, at<int>(workspace, L.cnt),
                         at<int>(workspace, L.kb), ukk, st) != cudaSuccess)
             return TWINKV_ERR_CUDA;
@@ -779,7 +787,7 @@ twinkv_status audit_stages(const DeviceInfo* dev, const void* keys, const twinkv
                            void* workspace, const Layout& L, cudaStream_t st)
 {
     const uint16_t* k16 = nullptr;
-    const twinkv_status r = prep_stages(keys, s, retained_mask, out_score_all || out_twin_all,
+    const twinkv_status r = prep_stages(dev, keys, s, retained_mask, out_score_all || out_twin_all,
                                         workspace, L, st, &k16);
     if (r != TWINKV_OK) return r;
     return main_stages(dev, k16, s, p, bret, t0, out_score_all, out_twin_all, workspace, L, st);
@@ -1026,7 +1034,7 @@ twinkv_status twinkv_repair_host(const void* keys, twinkv_shape s, const uint8_t
         const Layout Lc = layout(sc, TWINKV_OP_REPAIR);
         char* wsb = base + A.ws + b * A.ws_bytes;
         const uint16_t* k16 = nullptr;
-        if ((r = prep_stages(kbuf, sc, d_mask + u0 * N, need_all, wsb, Lc, st, &k16)) != TWINKV_OK)
+        if ((r = prep_stages(dev, kbuf, sc, d_mask + u0 * N, need_all, wsb, Lc, st, &k16)) != TWINKV_OK)
             return fail(r);
         r = main_stages(dev, k16, sc, p, d_bret + u0 * N, d_tret + u0 * N,
                         need_all ? d_sall + u0 * N : nullptr, need_all ? d_tall + u0 * N : nullptr,

@@ -120,6 +120,12 @@ cudaError_t launch_norms_identity(const void* keys, bool f32, uint16_t* keys16, 
                                   int d, int64_t NP, float* colrinv, int* colpos,
                                   float4* norms, cudaStream_t st, float rscale = 1.0f,
                                   unsigned* unit_kk = nullptr);
+// launch_scan, launch_gather and launch_scale_columns in one kernel; *launched = false where
+// the sizes are not its own.
+cudaError_t launch_prep_unit(const void* keys, bool f32, uint16_t* keys16, const uint8_t* mask,
+                             int* cnt, int* kb, int U, int N, int d, int64_t NP, uint16_t* kp,
+                             float* colrinv, int* colpos, float4* norms, bool evicted, int sms,
+                             cudaStream_t st, bool* launched);
 // Also zeroes unit_kk for launch_gather.  `evicted`: the evicted segment is wanted too.
 cudaError_t launch_scan(const uint8_t* mask, int U, int N, int* cnt, int* kb, unsigned* unit_kk,
                         cudaStream_t st);

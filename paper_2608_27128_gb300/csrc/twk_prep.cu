@@ -29,6 +29,12 @@ template <int D>
 constexpr int kKeys = 128 / D;
 template <int D>
 constexpr int kKeysPerBlock = kKeysPerStep * kKeys<D>;   // NP is a multiple of this
+// prep_unit_kernel: CTAs per unit, threads, a CTA's slots (one per lane group), and the
+// largest N whose column stride they cover.
+constexpr int kUnitCtas = 8;
+constexpr int kUnitThreads = 1024;
+constexpr int kUnitSlots = kUnitThreads / kParts;
+constexpr int kUnitMaxN = kUnitCtas * kUnitSlots - kBN;
 
 // A lane's 16-byte chunks part, part + kParts, ... of a key's bf16 row, from bf16 keys or
 // from float32 ones rounded to nearest even (8 floats per chunk).
@@ -145,6 +151,63 @@ __global__ void __launch_bounds__(kPrepThreads)
 
 constexpr int kScanBytes = 16;   // mask bytes per thread and step
 
+// Bit j: position p0 + j of a unit's mask m is retained (a non-zero byte).  vec: N and m are
+// multiples of 16.
+__device__ __forceinline__ uint32_t keep_bits(const uint8_t* m, int p0, int N, bool vec)
+{
+    uint32_t keep = 0;
+    if (vec) {
+        if (p0 < N) {
+            const uint4 v = *reinterpret_cast<const uint4*>(m + p0);
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int j = 0; j < kScanBytes; ++j)
+                keep |= ((w[j / 4] >> (8 * (j % 4))) & 255u) != 0u ? 1u << j : 0u;
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < kScanBytes; ++j)
+            if (p0 + j < N && m[p0 + j] != 0) keep |= 1u << j;
+    }
+    return keep;
+}
+
+// c[p0 + j] = run + the bits of `keep` below j, for the positions below N.
+__device__ __forceinline__ void store_counts(int* c, int p0, int N, bool vec, uint32_t keep, int run)
+{
+    if (vec) {   // N, and so every row of cnt, is a multiple of 16 entries
+        if (p0 < N) {
+#pragma unroll
+            for (int j = 0; j < kScanBytes; j += 4) {
+                int4 o;
+                o.x = run;
+                o.y = o.x + ((keep >> j) & 1u);
+                o.z = o.y + ((keep >> (j + 1)) & 1u);
+                o.w = o.z + ((keep >> (j + 2)) & 1u);
+                run = o.w + ((keep >> (j + 3)) & 1u);
+                *reinterpret_cast<int4*>(c + p0 + j) = o;
+            }
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < kScanBytes; ++j) {
+            if (p0 + j < N) c[p0 + j] = run;
+            run += (keep >> j) & 1u;
+        }
+    }
+}
+
+// The inclusive sum of x over the warp's lanes up to this one.
+__device__ __forceinline__ int warp_prefix(int x, int lane)
+{
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+        if (lane >= o) x += y;
+    }
+    return x;
+}
+
 // Mode 1, step 1: cnt[u][p] = number of retained positions before p; kb[u] = |S0|;
 // unit_kk[u] = 0.  One block per unit; a mask byte counts as retained when non-zero.  A
 // thread takes 16 consecutive positions, so that a block covers 16384 per step of one
@@ -163,54 +226,15 @@ __global__ void scan_kernel(const uint8_t* __restrict__ mask, int N, int* __rest
     int carry = 0, step = 0;
     for (int base = 0; base < N; base += blockDim.x * kScanBytes, step ^= 1) {
         const int p0 = base + threadIdx.x * kScanBytes;
-        uint32_t keep = 0;   // bit j: position p0 + j is retained
-        if (vec) {
-            if (p0 < N) {
-                const uint4 v = *reinterpret_cast<const uint4*>(m + p0);
-                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                for (int j = 0; j < kScanBytes; ++j)
-                    keep |= ((w[j / 4] >> (8 * (j % 4))) & 255u) != 0u ? 1u << j : 0u;
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < kScanBytes; ++j)
-                if (p0 + j < N && m[p0 + j] != 0) keep |= 1u << j;
-        }
-        const int f = __popc(keep);
-        int x = f;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-            if (lane >= o) x += y;
-        }
+        const uint32_t keep = keep_bits(m, p0, N, vec);
+        const int f = __popc(keep), x = warp_prefix(f, lane);
         if (lane == 31) warp_tot[step][wid] = x;
         __syncthreads();
         const int t = lane < nw ? warp_tot[step][lane] : 0;
         const int all = __reduce_add_sync(0xFFFFFFFFu, t);
         const int mine = __reduce_add_sync(0xFFFFFFFFu, lane < wid ? t : 0);
-        int run = carry + mine + x - f;
+        store_counts(c, p0, N, vec, keep, carry + mine + x - f);
         carry += all;
-        if (vec) {   // N, and so every row of cnt, is a multiple of 16 entries
-            if (p0 < N) {
-#pragma unroll
-                for (int j = 0; j < kScanBytes; j += 4) {
-                    int4 o;
-                    o.x = run;
-                    o.y = o.x + ((keep >> j) & 1u);
-                    o.z = o.y + ((keep >> (j + 1)) & 1u);
-                    o.w = o.z + ((keep >> (j + 2)) & 1u);
-                    run = o.w + ((keep >> (j + 3)) & 1u);
-                    *reinterpret_cast<int4*>(c + p0 + j) = o;
-                }
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < kScanBytes; ++j) {
-                if (p0 + j < N) c[p0 + j] = run;
-                run += (keep >> j) & 1u;
-            }
-        }
         // the next step writes the other half of warp_tot; the one after it follows the
         // next step's barrier
     }
@@ -289,6 +313,14 @@ __global__ void __launch_bounds__(kPrepThreads)
     unit_max_kk(unit_kk, u, top);
 }
 
+// ceil(E / 2) for kk < 2^E: the largest ||k|| of a unit is below 2 to this.
+__device__ __forceinline__ int unit_exponent(float kk)
+{
+    int E;
+    (void)frexpf(kk, &E);
+    return (E + 1) >> 1;   // also for E <= 0
+}
+
 // colrinv[u][c] *= 2^-e_u, the power of two with 2^e_u >= the largest ||k|| of unit u
 // (from unit_kk), so that every scaled similarity x_ij * colrinv_j = sim(i,j) ||k_i||
 // 2^-e_u lies in [-1, 1].  Exact (a power of two); NaN padding stays NaN.  A unit of
@@ -304,10 +336,96 @@ __global__ void __launch_bounds__(kPrepThreads)
     const float kk = __uint_as_float(unit_kk[u]);
     const int64_t cols = kb ? (static_cast<int64_t>(kb[u]) + kBN - 1) / kBN * kBN : NP;
     if (c >= cols || !(kk > 0.f)) return;
-    int E;
-    (void)frexpf(kk, &E);               // kk < 2^E, so ||k|| < 2^ceil(E / 2)
-    const int e = (E + 1) >> 1;          // ceil(E / 2), also for E <= 0
-    colrinv[u * NP + c] = ldexpf(colrinv[u * NP + c], -e);
+    colrinv[u * NP + c] = ldexpf(colrinv[u * NP + c], -unit_exponent(kk));
+}
+
+// Mode 1 in one launch, for the smallest calls, where three launches and the waits between
+// them take longer than their work: a cluster of kUnitCtas CTAs does a unit's scan, gather
+// and scaling.  Every CTA scans the whole mask (16 bytes per thread) for the retained
+// positions before its slots [r NP / 8, (r + 1) NP / 8), so that only the largest k.k
+// crosses the cluster; each lane group keeps its slot's 1/||k|| until the scale is known.
+// Same values as the three kernels above.  Grid 8 U.
+template <int D, typename Key>
+__global__ void __cluster_dims__(kUnitCtas, 1, 1) __launch_bounds__(kUnitThreads)
+    prep_unit_kernel(const Key* __restrict__ keys, const uint8_t* __restrict__ mask, int N,
+                     int64_t NP, int* __restrict__ cnt, int* __restrict__ kb,
+                     uint16_t* __restrict__ kp, float* __restrict__ colrinv,
+                     int* __restrict__ colpos, float4* __restrict__ norms,
+                     uint16_t* __restrict__ keys16, bool evicted)
+{
+    wait_for_previous();
+    constexpr int Q = D / 8 / kParts, kWarps = kUnitThreads / 32;
+    static_assert(kWarps == 32, "one warp's total per lane");
+    __shared__ int warp_tot[kWarps];
+    __shared__ unsigned warp_top[kWarps];
+    __shared__ unsigned peer_top[kUnitCtas];
+    __shared__ int slot[kUnitSlots];         // retained positions before it; bit 31: retained
+    const int rank = static_cast<int>(cluster_rank());
+    const int64_t u = blockIdx.x / kUnitCtas;
+    const int per = static_cast<int>(NP) / kUnitCtas;   // at most kUnitSlots, a multiple of 32
+    const int lo = rank * per;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int part = threadIdx.x % kParts, j = threadIdx.x / kParts, p = lo + j;
+    uint4 v[Q];                              // in flight over the scan
+    load_key<D>(keys, u * N + (j < per && p < N ? p : 0), part, v);
+    const bool vec = N % kScanBytes == 0 && (reinterpret_cast<uintptr_t>(mask) & 15) == 0;
+    const int s0 = threadIdx.x * kScanBytes;
+    const uint32_t keep = keep_bits(mask + u * N, s0, N, vec);
+    const int f = __popc(keep), x = warp_prefix(f, lane);
+    if (lane == 31) warp_tot[wid] = x;
+    __syncthreads();
+    const int t = warp_tot[lane];
+    const int kept = __reduce_add_sync(0xFFFFFFFFu, t);
+    const int first = __reduce_add_sync(0xFFFFFFFFu, lane < wid ? t : 0) + x - f;
+    const int kpad = ((kept + kBN - 1) / kBN) * kBN;
+    if (s0 >= lo && s0 < lo + per) {         // 16 slots lie in one CTA's share
+        store_counts(cnt + u * N, s0, N, vec, keep, first);
+#pragma unroll
+        for (int k = 0; k < kScanBytes; ++k)
+            slot[s0 - lo + k] = (first + __popc(keep & ((1u << k) - 1u))) |
+                                static_cast<int>(((keep >> k) & 1u) << 31);
+    }
+    if (rank == 0 && threadIdx.x == 0) kb[u] = kept;
+    float r32;
+    const float4 nr = key_norms(v, r32);     // every lane takes part in its shuffles
+    const bool key = j < per && p < N;
+    const unsigned wt = __reduce_max_sync(0xFFFFFFFFu, key ? __float_as_uint(fmaxf(nr.x, 0.f)) : 0u);
+    if (lane == 0) warp_top[wid] = wt;
+    __syncwarp();
+    cluster_barrier();                       // slot and warp_top; the other CTAs have started
+    if (wid == 0) {
+        const unsigned bt = __reduce_max_sync(0xFFFFFFFFu, warp_top[lane]);
+        if (lane < kUnitCtas)
+            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr(peer_top + rank, lane)),
+                         "r"(bt)
+                         : "memory");
+    }
+    int col = 0;
+    bool read = false;
+    if (j < per) {
+        const int r = p - N, before = slot[j] & 0x7FFFFFFF;
+        col = p >= N       ? (r < kpad - kept ? kept + r : kpad + (N - kept) + (r - (kpad - kept)))
+              : slot[j] < 0 ? before
+                            : kpad + (p - before);
+        read = evicted || col < kpad;
+        if constexpr (sizeof(Key) == 4)
+            if (p < N) store_key<D>(keys16, u * N + p, part, v);
+        if (p >= N) {
+#pragma unroll
+            for (int q = 0; q < Q; ++q) v[q] = make_uint4(0u, 0u, 0u, 0u);
+        }
+        if (read) store_key<D>(kp, u * NP + col, part, v);
+        if (part == 0 && p < N) norms[u * N + p] = nr;
+    }
+    __syncwarp();
+    cluster_barrier();
+    if (part != 0 || !read) return;
+    unsigned kk = 0u;
+#pragma unroll
+    for (int r = 0; r < kUnitCtas; ++r) kk = max(kk, peer_top[r]);
+    const int e = kk != 0u ? unit_exponent(__uint_as_float(kk)) : 0;
+    colrinv[u * NP + col] = p < N ? ldexpf(r32, -e) : nan_f();
+    colpos[u * NP + col] = p < N ? p : -1;
 }
 
 }  // namespace
@@ -347,6 +465,44 @@ cudaError_t launch_scan(const uint8_t* mask, int U, int N, int* cnt, int* kb, un
     const int threads = std::min(1024, (N + 32 * kScanBytes - 1) / (32 * kScanBytes) * 32);
     scan_kernel<<<U, threads, 0, st>>>(mask, N, cnt, kb, unit_kk);
     return cudaGetLastError();
+}
+
+cudaError_t launch_prep_unit(const void* keys, bool f32, uint16_t* keys16, const uint8_t* mask,
+                             int* cnt, int* kb, int U, int N, int d, int64_t NP, uint16_t* kp,
+                             float* colrinv, int* colpos, float4* norms, bool evicted, int sms,
+                             cudaStream_t st, bool* launched)
+{
+    *launched = false;
+    // One slot per lane group, half of the SMs at most, and 64 KB of keys per CTA.  us per
+    // call, three kernels / one: 1 unit of 512 x 64 (fp32) 31.7 / 27.0, 8 of 1024 x 128
+    // 30.0 / 26.2, of 1792 29.5 / 26.8.  Beyond: two slots per group, 8 units of 3072 36.4 /
+    // 37.5; 16 units of 1792, whose clusters do not all fit at once, 32.2 / 35.8; 8 fp32 ones of
+    // 1792 x 128 with both audits 32.8 / 34.6.
+    const int64_t bytes = static_cast<int64_t>(N) * d * (f32 ? 4 : 2);
+    if (N > kUnitMaxN || static_cast<int64_t>(U) * kUnitCtas * 2 > sms ||
+        bytes > kUnitCtas * (64 << 10))
+        return cudaSuccess;
+    auto go = [&](auto kernel, auto* k) {
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(static_cast<unsigned>(U) * kUnitCtas);
+        cfg.blockDim = dim3(kUnitThreads);
+        cfg.stream = st;
+        int clusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) != cudaSuccess || clusters < 1) {
+            cudaGetLastError();   // no room for a cluster: the caller's other kernels need none
+            return cudaSuccess;
+        }
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, k, mask, N, NP, cnt, kb, kp, colrinv,
+                                                 colpos, norms, keys16, evicted);
+        *launched = e == cudaSuccess;
+        return e;
+    };
+    const float* kf = static_cast<const float*>(keys);
+    const uint16_t* kh = static_cast<const uint16_t*>(keys);
+    if (f32 && d == 128) return go(prep_unit_kernel<128, float>, kf);
+    if (f32) return go(prep_unit_kernel<64, float>, kf);
+    if (d == 128) return go(prep_unit_kernel<128, uint16_t>, kh);
+    return go(prep_unit_kernel<64, uint16_t>, kh);
 }
 
 cudaError_t launch_gather(const void* keys, bool f32, uint16_t* keys16, const uint8_t* mask,
