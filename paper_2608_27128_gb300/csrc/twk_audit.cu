@@ -115,6 +115,12 @@ struct AuditCfg {
     static constexpr int B_STAGE = kBN / 2 * 128;     // 16 KB: this CTA's half of a K chunk
     static constexpr int STAGES = 6;
     static constexpr int MSLOTS = 4;
+    // Count mode at d = 128: a column group takes every second tile whole, in two passes,
+    // instead of its half of every tile, so that one group's accumulator loads run beside the
+    // other's counting (policy 36x8x8192x128: 2977 -> 2940 us of audit).  At d = 64 it changes
+    // nothing (172.5 -> 173.4), and the argmax loses 3 to 4 %.
+    static constexpr bool WHOLE = kCount && D == 128;
+    static constexpr int TILE_WARPS = WHOLE ? kEpiWarps / kGroups : kEpiWarps;   // of a CTA
     static constexpr int META = kBN * 8;              // rinv[256] + pos[256]
     static constexpr int OFF_A = 0;
     static constexpr int OFF_B = OFF_A + 2 * A_BYTES;
@@ -597,7 +603,7 @@ __global__ void __cluster_dims__(2, 1, 1)
             mbar_init(&a_full[i], 1);
             mbar_init(&a_empty[i], 1);
             mbar_init(&t_full[i], 1);
-            mbar_init(&t_empty[i], 2 * kEpiWarps);   // both CTAs' epilogues
+            mbar_init(&t_empty[i], 2 * C::TILE_WARPS);   // both CTAs' epilogues
             mbar_init(&x_full[i], kGroups * kBM);
             mbar_init(&x_empty[i], 64);
         }
@@ -607,7 +613,7 @@ __global__ void __cluster_dims__(2, 1, 1)
         }
         for (int i = 0; i < C::MSLOTS; ++i) {
             mbar_init(&m_full[i], 1);
-            mbar_init(&m_empty[i], kEpiWarps);
+            mbar_init(&m_empty[i], C::TILE_WARPS);
         }
         mbar_init(drain, 1);
         if (kSym)
@@ -909,126 +915,138 @@ __global__ void __cluster_dims__(2, 1, 1)
                 thr = (a.count_tau /
                        (a.colrinv[static_cast<int64_t>(u) * a.NP + row] * (1.0f / kCountScale))) *
                       kCountScale;
-            for (int t = 0; t < nt; ++t) {
+            constexpr int kStep = C::WHOLE ? kGroups : 1;
+            const uint32_t n_item = n_t;   // the item's first tile
+            // whole tiles: group h takes those whose accumulator is h
+            const int t_first =
+                C::WHOLE ? static_cast<int>((n_t ^ static_cast<uint32_t>(h)) & 1u) : 0;
+            if (C::WHOLE) n_t += static_cast<uint32_t>(t_first);
+            for (int t = t_first; t < nt; t += kStep) {
                 const uint32_t ms = n_t % C::MSLOTS, acc = n_t & 1u;
                 if (!__all_sync(0xFFFFFFFFu, ready != 0u)) {
                     ok = all_wait(&m_full[ms], (n_t / C::MSLOTS) & 1u, wc, 7);
                     if (ok) ok = all_wait(&t_full[acc], (n_t >> 1) & 1u, wc, 8);
                     if (!ok) break;
                 }
-                ++n_t;
+                n_t += kStep;
                 tc_fence_after();
-                const float* rinv = reinterpret_cast<const float*>(sMeta + ms * C::META) + h * kGW;
-                const int* pos =
-                    reinterpret_cast<const int*>(sMeta + ms * C::META + kBN * 4) + h * kGW;
-                const int c_lo = (ut.t0 + t) * kBN + h * kGW;
-                const bool band = static_cast<uint32_t>(c_lo - s0a) < s0n ||
-                                  static_cast<uint32_t>(c_lo - s1a) < s1n;
-                const uint32_t taddr = tmem + lane_base + acc * kBN + static_cast<uint32_t>(h * kGW);
                 auto test_next = [&]() {
                     ready = mbar_test2(m_full0 + 8u * (n_t % C::MSLOTS), (n_t / C::MSLOTS) & 1u,
                                        t_full0 + 8u * (n_t & 1u), (n_t >> 1) & 1u);
                 };
-                uint32_t x[kCh][32];
-                load_group(taddr, x);
-                // The tile is in registers: hand the accumulator back to the MMA warp now,
-                // so it can compute the next-but-one tile while this one is reduced.
-                tc_fence_before();
-                if (lane == 0) mbar_arrive_cluster(acc ? release1 : release0);
-                if constexpr (kSym) {
-                    ready = 0;
-                    // row maxima (the eager fold: the column pass already costs more than
-                    // the vote saves) and each chunk's column maxima over this warp's 32
-                    // rows right after it (while its registers are live)
-                    uint32_t cr[4];
-                    if (band) {
-                        fold32_packed<true>(x[0], rinv, pos, rw, w2, mask, c_lo, b0);
-                        cr[0] = colpass32<true>(x[0], pos, rw, w2, si, row_ok);
-                        fold32_packed<true>(x[1], rinv + 32, pos + 32, rw, w2, mask, c_lo + 32, b0);
-                        cr[1] = colpass32<true>(x[1], pos + 32, rw, w2, si, row_ok);
-                        fold32_packed<true>(x[2], rinv + 64, pos + 64, rw, w2, mask, c_lo + 64, b0);
-                        cr[2] = colpass32<true>(x[2], pos + 64, rw, w2, si, row_ok);
-                        fold32_packed<true>(x[3], rinv + 96, pos + 96, rw, w2, mask, c_lo + 96, b0);
-                        cr[3] = colpass32<true>(x[3], pos + 96, rw, w2, si, row_ok);
-                    } else if (pad_item) {
-                        fold32_packed<false>(x[0], rinv, pos, rw, w2, mask, c_lo, b0);
-                        cr[0] = colpass32<true>(x[0], pos, rw, w2, si, row_ok);
-                        fold32_packed<false>(x[1], rinv + 32, pos + 32, rw, w2, mask, c_lo + 32, b0);
-                        cr[1] = colpass32<true>(x[1], pos + 32, rw, w2, si, row_ok);
-                        fold32_packed<false>(x[2], rinv + 64, pos + 64, rw, w2, mask, c_lo + 64, b0);
-                        cr[2] = colpass32<true>(x[2], pos + 64, rw, w2, si, row_ok);
-                        fold32_packed<false>(x[3], rinv + 96, pos + 96, rw, w2, mask, c_lo + 96, b0);
-                        cr[3] = colpass32<true>(x[3], pos + 96, rw, w2, si, row_ok);
+                int g = C::WHOLE ? 0 : h;   // the half of the tile
+                do {
+                    const float* rinv = reinterpret_cast<const float*>(sMeta + ms * C::META) + g * kGW;
+                    const int* pos =
+                        reinterpret_cast<const int*>(sMeta + ms * C::META + kBN * 4) + g * kGW;
+                    const int c_lo = (ut.t0 + t) * kBN + g * kGW;
+                    const bool band = static_cast<uint32_t>(c_lo - s0a) < s0n ||
+                                      static_cast<uint32_t>(c_lo - s1a) < s1n;
+                    const uint32_t taddr = tmem + lane_base + acc * kBN + static_cast<uint32_t>(g * kGW);
+                    uint32_t x[kCh][32];
+                    load_group(taddr, x);
+                    // The tile is in registers: hand the accumulator back to the MMA warp now,
+                    // so it can compute the next-but-one tile while this one is reduced.
+                    tc_fence_before();
+                    if (lane == 0 && (!C::WHOLE || g == kGroups - 1))
+                        mbar_arrive_cluster(acc ? release1 : release0);
+                    if constexpr (kSym) {
+                        ready = 0;
+                        // row maxima (the eager fold: the column pass already costs more than
+                        // the vote saves) and each chunk's column maxima over this warp's 32
+                        // rows right after it (while its registers are live)
+                        uint32_t cr[4];
+                        if (band) {
+                            fold32_packed<true>(x[0], rinv, pos, rw, w2, mask, c_lo, b0);
+                            cr[0] = colpass32<true>(x[0], pos, rw, w2, si, row_ok);
+                            fold32_packed<true>(x[1], rinv + 32, pos + 32, rw, w2, mask, c_lo + 32, b0);
+                            cr[1] = colpass32<true>(x[1], pos + 32, rw, w2, si, row_ok);
+                            fold32_packed<true>(x[2], rinv + 64, pos + 64, rw, w2, mask, c_lo + 64, b0);
+                            cr[2] = colpass32<true>(x[2], pos + 64, rw, w2, si, row_ok);
+                            fold32_packed<true>(x[3], rinv + 96, pos + 96, rw, w2, mask, c_lo + 96, b0);
+                            cr[3] = colpass32<true>(x[3], pos + 96, rw, w2, si, row_ok);
+                        } else if (pad_item) {
+                            fold32_packed<false>(x[0], rinv, pos, rw, w2, mask, c_lo, b0);
+                            cr[0] = colpass32<true>(x[0], pos, rw, w2, si, row_ok);
+                            fold32_packed<false>(x[1], rinv + 32, pos + 32, rw, w2, mask, c_lo + 32, b0);
+                            cr[1] = colpass32<true>(x[1], pos + 32, rw, w2, si, row_ok);
+                            fold32_packed<false>(x[2], rinv + 64, pos + 64, rw, w2, mask, c_lo + 64, b0);
+                            cr[2] = colpass32<true>(x[2], pos + 64, rw, w2, si, row_ok);
+                            fold32_packed<false>(x[3], rinv + 96, pos + 96, rw, w2, mask, c_lo + 96, b0);
+                            cr[3] = colpass32<true>(x[3], pos + 96, rw, w2, si, row_ok);
+                        } else {
+                            fold32_packed<false>(x[0], rinv, pos, rw, w2, mask, c_lo, b0);
+                            cr[0] = colpass32<false>(x[0], pos, rw, w2, si, row_ok);
+                            fold32_packed<false>(x[1], rinv + 32, pos + 32, rw, w2, mask, c_lo + 32, b0);
+                            cr[1] = colpass32<false>(x[1], pos + 32, rw, w2, si, row_ok);
+                            fold32_packed<false>(x[2], rinv + 64, pos + 64, rw, w2, mask, c_lo + 64, b0);
+                            cr[2] = colpass32<false>(x[2], pos + 64, rw, w2, si, row_ok);
+                            fold32_packed<false>(x[3], rinv + 96, pos + 96, rw, w2, mask, c_lo + 96, b0);
+                            cr[3] = colpass32<false>(x[3], pos + 96, rw, w2, si, row_ok);
+                        }
+                        // merge the four lane quarters of this group: the warps exchange their
+                        // 128 column maxima, then warp q takes columns 32q .. 32q + 31
+                        const int par = static_cast<int>(n_c & 1);
+                        uint32_t* cb = sCB + (par * kGroups + h) * 4 * kBM;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) cb[q * kBM + 32 * k + lane] = cr[k];
+                        mbar_arrive(&cbar[par * kGroups + h]);
+                        ok = all_wait(&cbar[par * kGroups + h], (n_c >> 1) & 1, wc, 11);
+                        ++n_c;
+                        if (!ok) break;
+                        const int c = q * 32 + lane;
+                        uint32_t best = cb[c];
+                        int bq = 0;
+#pragma unroll
+                        for (int qq = 1; qq < 4; ++qq) {
+                            const uint32_t vq = cb[qq * kBM + c];
+                            if ((vq & 0xFFFFFFE0u) > (best & 0xFFFFFFE0u)) {
+                                best = vq;
+                                bq = qq;
+                            }
+                        }
+                        const int gcol = c_lo + c;
+                        if (gcol < a.N && (best & 0xFFFFFFE0u) != 0u) {
+                            const uint32_t win = static_cast<uint32_t>(r0 + 32 * bq + 31) - (best & 31u);
+                            atomicMax(a.slots + static_cast<int64_t>(u) * a.N + gcol,
+                                      (static_cast<unsigned long long>(best & 0xFFFFFFE0u) << 32) |
+                                          (0xFFFFFFFFull - win));
+                        }
+                    } else if constexpr (kCount) {
+                        cnt += band ? count_group<true>(x, rinv, pos, rw, w2, thr)
+                                    : count_group<false>(x, rinv, pos, rw, w2, thr);
+                        test_next();
                     } else {
-                        fold32_packed<false>(x[0], rinv, pos, rw, w2, mask, c_lo, b0);
-                        cr[0] = colpass32<false>(x[0], pos, rw, w2, si, row_ok);
-                        fold32_packed<false>(x[1], rinv + 32, pos + 32, rw, w2, mask, c_lo + 32, b0);
-                        cr[1] = colpass32<false>(x[1], pos + 32, rw, w2, si, row_ok);
-                        fold32_packed<false>(x[2], rinv + 64, pos + 64, rw, w2, mask, c_lo + 64, b0);
-                        cr[2] = colpass32<false>(x[2], pos + 64, rw, w2, si, row_ok);
-                        fold32_packed<false>(x[3], rinv + 96, pos + 96, rw, w2, mask, c_lo + 96, b0);
-                        cr[3] = colpass32<false>(x[3], pos + 96, rw, w2, si, row_ok);
-                    }
-                    // merge the four lane quarters of this group: the warps exchange their
-                    // 128 column maxima, then warp q takes columns 32q .. 32q + 31
-                    const int par = static_cast<int>(n_c & 1);
-                    uint32_t* cb = sCB + (par * kGroups + h) * 4 * kBM;
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) cb[q * kBM + 32 * k + lane] = cr[k];
-                    mbar_arrive(&cbar[par * kGroups + h]);
-                    ok = all_wait(&cbar[par * kGroups + h], (n_c >> 1) & 1, wc, 11);
-                    ++n_c;
-                    if (!ok) break;
-                    const int c = q * 32 + lane;
-                    uint32_t best = cb[c];
-                    int bq = 0;
-#pragma unroll
-                    for (int qq = 1; qq < 4; ++qq) {
-                        const uint32_t vq = cb[qq * kBM + c];
-                        if ((vq & 0xFFFFFFE0u) > (best & 0xFFFFFFE0u)) {
-                            best = vq;
-                            bq = qq;
+                        if (t == ut.tr) {
+                            // The evicted segment matters only where it reaches the retained
+                            // one: start its running best just below this group's retained
+                            // best (exact similarities decide between the two later; the
+                            // FLT_MIN keeps an exact tie at 0 in play).
+                            if constexpr (!kPacked) resolve_best(slot, mask, best);
+                            b0 = best;
+                            best = Best{b0.v - (fabsf(b0.v) * 0x1p-13f + FLT_MIN), -1};
+                        }
+                        if constexpr (kPacked) {
+                            if (band) fold_packed<true>(x, rinv, pos, rw, w2, mask, c_lo, best);
+                            else fold_packed<false>(x, rinv, pos, rw, w2, mask, c_lo, best);
+                            test_next();
+                        } else {
+                            float v[kCh][32], m[kCh];
+                            if (band) scale_group<true>(x, rinv, pos, rw, w2, v, m);
+                            else scale_group<false>(x, rinv, pos, rw, w2, v, m);
+                            const uint32_t stamp = 2u * n_x + (t < ut.tr ? 0u : 1u);
+                            const float other = published(pub + (1 - h) * kBM * 8, stamp);
+                            test_next();
+                            keep_best(v, m, c_lo, slot, pub + h * kBM * 8, stamp, other, best);
                         }
                     }
-                    const int gcol = c_lo + c;
-                    if (gcol < a.N && (best & 0xFFFFFFE0u) != 0u) {
-                        const uint32_t win = static_cast<uint32_t>(r0 + 32 * bq + 31) - (best & 31u);
-                        atomicMax(a.slots + static_cast<int64_t>(u) * a.N + gcol,
-                                  (static_cast<unsigned long long>(best & 0xFFFFFFE0u) << 32) |
-                                      (0xFFFFFFFFull - win));
-                    }
-                } else if constexpr (kCount) {
-                    cnt += band ? count_group<true>(x, rinv, pos, rw, w2, thr)
-                                : count_group<false>(x, rinv, pos, rw, w2, thr);
-                    test_next();
-                } else {
-                    if (t == ut.tr) {
-                        // The evicted segment matters only where it reaches the retained
-                        // one: start its running best just below this group's retained
-                        // best (exact similarities decide between the two later; the
-                        // FLT_MIN keeps an exact tie at 0 in play).
-                        if constexpr (!kPacked) resolve_best(slot, mask, best);
-                        b0 = best;
-                        best = Best{b0.v - (fabsf(b0.v) * 0x1p-13f + FLT_MIN), -1};
-                    }
-                    if constexpr (kPacked) {
-                        if (band) fold_packed<true>(x, rinv, pos, rw, w2, mask, c_lo, best);
-                        else fold_packed<false>(x, rinv, pos, rw, w2, mask, c_lo, best);
-                        test_next();
-                    } else {
-                        float v[kCh][32], m[kCh];
-                        if (band) scale_group<true>(x, rinv, pos, rw, w2, v, m);
-                        else scale_group<false>(x, rinv, pos, rw, w2, v, m);
-                        const uint32_t stamp = 2u * n_x + (t < ut.tr ? 0u : 1u);
-                        const float other = published(pub + (1 - h) * kBM * 8, stamp);
-                        test_next();
-                        keep_best(v, m, c_lo, slot, pub + h * kBM * 8, stamp, other, best);
-                    }
-                }
+                } while (C::WHOLE && ++g < kGroups);
+                if (kSym && !ok) break;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&m_empty[ms]);
             }
             if (!ok) break;
+            if (C::WHOLE) n_t = n_item + static_cast<uint32_t>(nt);
             if constexpr (!kCount && !kSym) {
                 if constexpr (!kPacked) resolve_best(slot, mask, best);
                 if (nt > ut.tr) b1 = best;
