@@ -262,13 +262,13 @@ twinkv_status twinkv_repair_select_noalloc(const double* score_ret, twinkv_shape
  * units' keys go to the device in chunks of at most `chunk_units` units (0: the value
  * twinkv_host_default_chunk returns).  Nothing computes while the first chunk copies
  * in and each chunk's compute has to cover the next one's copy, so the chunks grow
- * from one unit by x2.5 (sizes of a whole wave of 128-row blocks or more rounded to
- * the nearest multiple of such a wave) up to `chunk_units`.
+ * from one unit by x2.5 (sizes of a whole wave of 128-row blocks, one per SM, or more
+ * rounded to the nearest multiple of such a wave) up to `chunk_units`.
  * Per chunk, ordered by events:
  *   - its keys and mask are copied in on a copy stream the library keeps per device;
  *   - its prefix counts, retained-first layout and audit run on `stream`;
- *   - the exact values of its winners run on a second library stream, in blocks that
- *     fit on the SMs beside the next chunk's audit;
+ *   - the exact values of its winners run on a second library stream, so that the next
+ *     chunk's kernels do not wait for them;
  *   - its scores and twins are copied back on a third.
  * Three chunk buffers let chunk c + 1's copy run while chunk c - 1 is still being
  * finished.  One selection over all units follows the last chunk, and S1,

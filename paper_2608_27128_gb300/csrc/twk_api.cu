@@ -735,7 +735,7 @@ twinkv_status prep_stages(const DeviceInfo* dev, const void* keys, const twinkv_
 
 // The audit (Eq. 4 and b_i(all)) and the exact value of each winner, on the inputs
 // prep_stages left in `workspace`.  With refine_st given, the exact values run there
-// after the audit (ordered by audit_done), in blocks that fit beside the next audit.
+// after the audit (ordered by audit_done), beside what the caller queues on `st` next.
 twinkv_status main_stages(const DeviceInfo* dev, const uint16_t* k16, const twinkv_shape& s,
                           const twinkv_params& p, double* bret, int* t0, double* out_score_all,
                           int32_t* out_twin_all, void* workspace, const Layout& L,
@@ -1027,7 +1027,7 @@ twinkv_status twinkv_repair_host(const void* keys, twinkv_shape s, const uint8_t
             return fail(TWINKV_ERR_CUDA);
         // Prefix counts, retained-first layout and audit of this chunk on `stream`, into
         // this buffer's workspace and the all-unit arrays; the exact values on the
-        // refine stream, beside the next chunk's audit.
+        // refine stream, which the next chunk's kernels do not wait for.
         twinkv_shape sc = s;
         sc.L = 1;
         sc.H = un;

@@ -17,8 +17,9 @@
 //               one thread issues tcgen05.mma.cta_group::2 (M=256, N=256, K=16,
 //               bf16 -> fp32) for both and commits to both CTAs' barriers.
 //   warps 2, 3  merge the column groups of every finished row and write the results.
-//   warps 4..   epilogue: four warps per column group (128 columns of each tile); a thread
-//               owns one row (TMEM lane) and keeps its running maximum.
+//   warps 4..   epilogue: four warps per column group (128 columns of each tile; in the count
+//               mode at d = 128 every second tile); a thread owns one row (TMEM lane) and
+//               keeps its running maximum.
 // Why pairs: with one CTA per 128 rows, each tile moves 64 KB of B into shared memory
 // and 96 KB of operands out of it (d = 128), beside the epilogue's broadcast loads; a
 // pair moves 32 KB in and 64 KB out per SM.  Whole calls, one CTA -> pair: Qwen3-4B
@@ -42,11 +43,19 @@
 // (|i - j| <= w) are set to NaN on the few tiles that intersect the window band of the
 // row block.
 //
-// What bounds the epilogue (cycle counters and copies with parts left out, at d = 128 and
-// 64): not the scaling, whose 32 broadcast loads and 64 paired multiply-adds per warp and
-// tile hide behind the MMAs, but the maxima and the look-up of the column, on an ALU that
-// issues one instruction every two cycles, and about 100 instructions per warp and tile
-// of waits and bookkeeping.  Two warps per scheduler hide little latency, so:
+// What bounds it, from copies with parts left out (TFLOP/s of redundancy 16x8x16384x128,
+// repair 16x8x8192x64, policy 36x8x8192x128 and 16x8x3001x64):
+//   every part                        1579   745  1662   848
+//   no reduction                      1968  1502  1937  1378
+//   no MMAs                           1934   816  2169   910
+//   no MMAs, no accumulator loads     2125   878  2406  1000
+//   no loads of the column scales     1632   782  1670   923
+//   no column codes (d = 64)             -   963     -     -
+// At d = 64 it is the reduction: per thread and tile 64 paired multiply-adds, 128 column
+// codes and 64 three-input maxima, the last two on an ALU that issues one instruction every
+// two cycles.  At d = 128 MMAs and reduction overlap to within a fifth of the MMAs alone, at a
+// rate that a seconds-long run holds under the power limit only just.  Two warps per
+// scheduler hide little latency, so:
 //   * the warpgroups trade registers (setmaxnreg): with 200 and more the four chunks of
 //     a warp are scaled and reduced side by side (at 168 the compiler kept them apart);
 //   * at d = 128 a row that improves only copies its chunk's values to its slot in shared
@@ -57,10 +66,10 @@
 //   * the next tile's barriers are tested while the current one is reduced (a wait on a
 //     completed barrier took 150 cycles), the next item's counts are loaded one item
 //     ahead, and two spare warps merge and write what the last item found.
-// Audit alone, before -> after: Qwen3-4B 16x8x16384x128 1279 -> 1559 TFLOP/s,
-// Llama-3.2-1B 16x8x8192x64 672 -> 740, policy 36x8x8192x128 1629 -> 1655, policy
-// 16x8x3001x64 728 -> 851.  Sixteen epilogue warps of 64 columns (104 registers): 1322,
-// 674, 1522, 811.  Copies without the look-up ran at 946 (d = 64).
+// Audit alone, one CTA per 128 rows and 320 threads -> as built: Qwen3-4B 16x8x16384x128
+// 1279 -> 1570 TFLOP/s, Llama-3.2-1B 16x8x8192x64 672 -> 746, policy 36x8x8192x128
+// 1629 -> 1680, policy 16x8x3001x64 728 -> 853.  Sixteen epilogue warps of 64 columns (104
+// registers): 1322, 674, 1522, 811.
 //
 // Count mode (Sec. 3.2 Eq. 2, the standalone scorer): instead of the maximum, each row i
 // counts the columns j outside the window with sim(i,j) > tau.  With x_ij the raw dot

@@ -75,8 +75,8 @@ constexpr int kRowsPerBlock = kRefineThreads / kParts;
 // kParts threads per row.  Bound by the gathers of 256-byte rows from L2 (about 7 TB/s at
 // 18x8x8192x128) and, with both candidates, by the TwoSum instructions.  kMinBlocks is the
 // number of 256 threads that fit on an SM: 5 (48 registers) for one candidate, 4 (64) where
-// rows have two, whose sums need 8 registers more; 6 (40) fits beside a CTA of at most 168
-// registers and 320 threads.  Blocks of 128 threads leave less of an SM waiting for its
+// rows have two, whose sums need 8 registers more; 6 (40) on the host path's own stream.
+// Blocks of 128 threads leave less of an SM waiting for its
 // slowest rows than blocks of 256: 82 against 86 us at 18x8x8192x128, 53 against 56 at
 // 16x8x8192x64, 221 against 232 with both candidates at 16x8x16384x128 (64 threads: 83, 72,
 // 217).  With even and odd elements summed in the halves of paired instructions, one
@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(kRefineThreads, kMinBlocks * 256 / kRefineThre
     const int64_t s1 = base + (j1 >= 0 ? j1 : r - base);
     // The standalone launch loads the norm records the cosine needs (the row's, and
     // the twin's this lane evaluates) beside the keys rather than after the dot
-    // product; the launch beside the audit has no registers to hold them.
+    // product; the host path's 40-register one has none to hold them.
     constexpr bool kEarly = kMinBlocks < 6;
     float4 nr{}, nt{};
     if constexpr (kEarly) {
