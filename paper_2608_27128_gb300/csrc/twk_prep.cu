@@ -325,18 +325,27 @@ __device__ __forceinline__ int unit_exponent(float kk)
 // (from unit_kk), so that every scaled similarity x_ij * colrinv_j = sim(i,j) ||k_i||
 // 2^-e_u lies in [-1, 1].  Exact (a power of two); NaN padding stays NaN.  A unit of
 // zero keys keeps its scale.  Given kb, only the retained columns, padded to a tile, are
-// scaled.  Grid (NP / kPrepThreads, U).
+// scaled.  Four columns per thread: the prep of 144 units of 8192 x 128 79.8 -> 76.6 us, of 128 of
+// 8192 x 64 54.6 -> 52.8, of 128 of 16384 x 128 184 -> 179.
+// Grid (NP / (4 kPrepThreads) rounded up, U).
 __global__ void __launch_bounds__(kPrepThreads)
     scale_columns_kernel(float* __restrict__ colrinv, int64_t NP,
                          const unsigned* __restrict__ unit_kk, const int* __restrict__ kb)
 {
     wait_for_previous();
     const int64_t u = blockIdx.y;
-    const int64_t c = static_cast<int64_t>(blockIdx.x) * kPrepThreads + threadIdx.x;
+    const int64_t c = (static_cast<int64_t>(blockIdx.x) * kPrepThreads + threadIdx.x) * 4;
     const float kk = __uint_as_float(unit_kk[u]);
     const int64_t cols = kb ? (static_cast<int64_t>(kb[u]) + kBN - 1) / kBN * kBN : NP;
-    if (c >= cols || !(kk > 0.f)) return;
-    colrinv[u * NP + c] = ldexpf(colrinv[u * NP + c], -unit_exponent(kk));
+    if (c >= cols || !(kk > 0.f)) return;   // cols and NP are multiples of a tile
+    const int e = unit_exponent(kk);
+    float4* p = reinterpret_cast<float4*>(colrinv + u * NP + c);
+    float4 v = *p;
+    v.x = ldexpf(v.x, -e);
+    v.y = ldexpf(v.y, -e);
+    v.z = ldexpf(v.z, -e);
+    v.w = ldexpf(v.w, -e);
+    *p = v;
 }
 
 // Mode 1 in one launch, for the smallest calls, where three launches and the waits between
@@ -453,7 +462,8 @@ cudaError_t launch_norms_identity(const void* keys, bool f32, uint16_t* keys16, 
 cudaError_t launch_scale_columns(float* colrinv, int U, int64_t NP, const unsigned* unit_kk,
                                  const int* kb, cudaStream_t st)
 {
-    const dim3 grid(static_cast<unsigned>((NP + kPrepThreads - 1) / kPrepThreads), U);
+    constexpr int per = 4 * kPrepThreads;
+    const dim3 grid(static_cast<unsigned>((NP + per - 1) / per), U);
     return launch_dependent(scale_columns_kernel, grid, kPrepThreads, 0, st, colrinv, NP, unit_kk,
                             kb);
 }
