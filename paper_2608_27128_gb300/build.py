@@ -22,7 +22,7 @@ BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libtwinkv.so")
 SOURCES = ["twk_api.cu", "twk_audit.cu", "twk_prep.cu", "twk_refine.cu", "twk_repair.cu",
            "twk_policy.cu"]
-HEADERS = ["twk_internal.h", "twk_ptx.cuh", "twk_df.cuh"]
+HEADERS = ["twk_internal.h", "twk_ptx.cuh", "twk_df.cuh", "twk_bound.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]
 

@@ -89,6 +89,7 @@
 #include <atomic>
 #include <cfloat>
 
+#include "twk_bound.cuh"
 #include "twk_internal.h"
 #include "twk_ptx.cuh"
 
@@ -145,7 +146,7 @@ struct AuditCfg {
         kCount || kSym || D == 64 ? 0 : kGroups * kBM * kSlot;
     // and the best value each group has published for each row, with its segment's stamp
     static constexpr int OFF_PUB = OFF_BEST + BEST_BYTES;
-    static constexpr int PUB_BYTES = BEST_BYTES ? kGroups * kBM * 8 : 0;
+    static constexpr int PUB_BYTES = BEST_BYTES ? kGroups * kBM * 4 : 0;
     static constexpr int OFF_BAR = OFF_PUB + PUB_BYTES;
     static constexpr int NBAR = 2 + 2 + 2 * STAGES + 2 * MSLOTS + 2 + 2 + 2 + 2 + 1 +
                                 (kSym ? 2 * kGroups : 0);
@@ -320,20 +321,22 @@ __device__ __forceinline__ void scale_group(const uint32_t (&x)[kCh][32], const 
     for (int k = 0; k < kCh; ++k) m[k] = tree32(v[k]);
 }
 
-// A value published, with a stamp, to the thread of the row's other column group: one aligned
-// 8-byte access each way, which shared memory serves whole.  (As one 64-bit register, or with
-// a check word, the compiler's schedule of the loop around it lost 15 %.)
-__device__ __forceinline__ void publish(uint32_t at, uint32_t stamp, float v)
+// A best value published to the thread of the row's other column group, which reads it with
+// nothing ordering the two: one 32-bit word (twk_bound.cuh) that is written and read whole by
+// relaxed accesses, whatever mixture of segments the two threads are at.  (As a (value, stamp)
+// pair in one vector access it could be seen half written, since a vector access is several
+// scalar ones in no given order, and an old segment's value would then drop a row's maximum.)
+__device__ __forceinline__ void publish(uint32_t at, uint32_t word)
 {
-    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(at), "f"(v), "f"(__uint_as_float(stamp)));
+    asm volatile("st.relaxed.cta.shared::cta.u32 [%0], %1;" ::"r"(at), "r"(word));
 }
 
-// The value at `at` if it carries this stamp, else -inf.
+// What the word at `at` bounds from below in segment `stamp` (-inf: nothing).
 __device__ __forceinline__ float published(uint32_t at, uint32_t stamp)
 {
-    float v, s;
-    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v), "=f"(s) : "r"(at));
-    return __float_as_uint(s) == stamp ? v : -INFINITY;
+    uint32_t word;
+    asm volatile("ld.relaxed.cta.shared::cta.u32 %0, [%1];" : "=r"(word) : "r"(at));
+    return __uint_as_float(bound_bits(word, stamp));
 }
 
 // Where a row of the warp improves on its best (strictly, so an earlier chunk keeps a
@@ -342,8 +345,9 @@ __device__ __forceinline__ float published(uint32_t at, uint32_t stamp)
 // `other` is the best that the row's other column group has published for this segment
 // (-inf if none): what stays below it cannot be the row's maximum and is not kept.  The
 // improved best is published at `mine` with the segment's stamp.  The two groups of a row
-// then improve 4.1 instead of 6.8 times over 32 tiles: dedup 18x8x8192x128 (10 tiles per row
-// block) 611 -> 591 us of audit, redundancy 2x8x5003x128 99 -> 96, Qwen3-4B 0.6 %.
+// then improve 4.1 instead of 6.8 times over 32 tiles.  Calls without the exchange -> with it:
+// dedup 18x8x8192x128 (10 tiles per row block) 831 -> 820 us, redundancy 2x8x5003x128 118 ->
+// 116, repair 1x8x131072x128 11625 -> 11300, Qwen3-4B 0.3 %.
 __device__ __forceinline__ void keep_best(const float (&v)[kCh][32], const float (&m)[kCh],
                                           int col0, uint32_t slot, uint32_t mine,
                                           uint32_t stamp, float other, Best& b)
@@ -367,7 +371,8 @@ __device__ __forceinline__ void keep_best(const float (&v)[kCh][32], const float
         b.col = here[k] ? col0 + 32 * k : b.col;
     }
     b.v = up ? top : b.v;
-    if (up) publish(mine, stamp, top);
+    // a value that is not positive (keys whose norms overflow) has no word that rounds down
+    if (up && top > 0.f) publish(mine, bound_word(__float_as_uint(top), stamp));
 }
 
 // The same without a slot: the low 5 mantissa bits of each value give way to (31 - column),
@@ -630,8 +635,8 @@ __global__ void __cluster_dims__(2, 1, 1)
         *abort_flag = 0;
         fence_mbarrier_init();
     }
-    for (int i = threadIdx.x; i < C::PUB_BYTES / 8; i += kThreads)
-        publish(smem_u32(smem + C::OFF_PUB) + 8 * i, ~0u, 0.f);   // a stamp of no segment
+    for (int i = threadIdx.x; i < C::PUB_BYTES / 4; i += kThreads)
+        publish(smem_u32(smem + C::OFF_PUB) + 4 * i, bound_word(kNoBound, 0u));
     if (warp == 0 && lane == 0) {
         prefetch_tensormap(&tmA);
         prefetch_tensormap(&tmB);
@@ -862,8 +867,9 @@ __global__ void __cluster_dims__(2, 1, 1)
         const uint32_t release1 = cluster_addr(&t_empty[1], 0);
         const uint32_t m_full0 = smem_u32(m_full), t_full0 = smem_u32(t_full);
         uint32_t n_t = 0;   // tiles seen: metadata slot n_t mod MSLOTS, accumulator n_t mod 2
-        // the row's published bests, one per group; stamps count this CTA's segments
-        const uint32_t pub = smem_u32(smem + C::OFF_PUB) + static_cast<uint32_t>(row_local * 8);
+        // the row's published bests, one per group; stamps count this CTA's segments, and a
+        // thread clears its word when it enters one (see twk_bound.cuh)
+        const uint32_t pub = smem_u32(smem + C::OFF_PUB) + static_cast<uint32_t>(row_local * 4);
         uint32_t n_x = 0;
         uint32_t n_c = 0;   // symmetric mode: tiles whose column maxima were merged
         bool ok = true;
@@ -917,6 +923,8 @@ __global__ void __cluster_dims__(2, 1, 1)
             Best b0{-INFINITY, -1}, b1{-INFINITY, -1};   // retained (or all) / evicted
             Best best = b0;                              // of the segment at hand
             const int rw = row - w;
+            if constexpr (C::PUB_BYTES != 0)
+                publish(pub + h * kBM * 4, bound_word(kNoBound, 2u * n_x));
 
             float cnt = 0.f;                               // count mode: r_i so far
             float thr = 0.f;                               // count mode: S tau ||k_i||
@@ -1034,6 +1042,8 @@ __global__ void __cluster_dims__(2, 1, 1)
                             if constexpr (!kPacked) resolve_best(slot, mask, best);
                             b0 = best;
                             best = Best{b0.v - (fabsf(b0.v) * 0x1p-13f + FLT_MIN), -1};
+                            if constexpr (C::PUB_BYTES != 0)
+                                publish(pub + h * kBM * 4, bound_word(kNoBound, 2u * n_x + 1u));
                         }
                         if constexpr (kPacked) {
                             if (band) fold_packed<true>(x, rinv, pos, rw, w2, mask, c_lo, best);
@@ -1044,9 +1054,9 @@ __global__ void __cluster_dims__(2, 1, 1)
                             if (band) scale_group<true>(x, rinv, pos, rw, w2, v, m);
                             else scale_group<false>(x, rinv, pos, rw, w2, v, m);
                             const uint32_t stamp = 2u * n_x + (t < ut.tr ? 0u : 1u);
-                            const float other = published(pub + (1 - h) * kBM * 8, stamp);
+                            const float other = published(pub + (1 - h) * kBM * 4, stamp);
                             test_next();
-                            keep_best(v, m, c_lo, slot, pub + h * kBM * 8, stamp, other, best);
+                            keep_best(v, m, c_lo, slot, pub + h * kBM * 4, stamp, other, best);
                         }
                     }
                 } while (C::WHOLE && ++g < kGroups);
