@@ -239,13 +239,16 @@ twinkv_status params_ok(const twinkv_params& p, float threshold)
     return TWINKV_OK;
 }
 
+// after_refine: the call's refine kernel is the one before it on `st`.
 twinkv_status launch_select(const twinkv_shape& s, const double* b, const uint8_t* mask,
                             const int32_t* budget, float threshold, const twinkv_params& p,
                             uint8_t* out_mask, int32_t* out_swaps, int32_t* out_nswaps,
                             int32_t* out_status, void* ws, const Layout& L, cudaStream_t st,
-                            const DeviceInfo* dev, const int32_t* twin = nullptr)
+                            const DeviceInfo* dev, const int32_t* twin = nullptr,
+                            bool after_refine = false)
 {
     RepairArgs r;
+    r.dependent = after_refine;
     r.U = s.L * s.H;
     r.N = s.N;
     r.b = b;
@@ -818,7 +821,8 @@ twinkv_status repair_impl(const void* keys, twinkv_shape s, const uint8_t* retai
                           out_twin_all, workspace, L, st)) != TWINKV_OK)
         return r;
     return launch_select(s, bret, retained_mask, budget, threshold, p, out_mask, out_swaps,
-                         out_nswaps, out_status, workspace, L, st, dev, dedup ? t0 : nullptr);
+                         out_nswaps, out_status, workspace, L, st, dev, dedup ? t0 : nullptr,
+                         true);
 }
 }  // namespace
 

@@ -74,6 +74,7 @@ struct RepairArgs {
     const int* twin;            // [U][N] argmax position of b_i(S0), or null
     int* rank_of;               // [U][N] scratch: donor rank of each position
     int cluster;                // literal variant: CTAs per unit (1, 2, 4, 8 or 16)
+    bool dependent;             // launched as the programmatic dependent of the kernel before it
 };
 
 // CTAs per unit of the literal repair's selection: a power of two up to 8 (see the
@@ -90,7 +91,9 @@ constexpr int kDedupMaxN = 1 << 19;
 // Every kernel that follows another one of the library on a stream is launched as its
 // programmatic dependent: its blocks are set up while the last ones before it still run, and
 // wait (wait_for_previous in twk_ptx.cuh) before they touch memory.  Each kernel waits at its
-// start, in every thread, so that a kernel's end implies the end of all before it.  A call is
+// start, in every thread, so that a kernel's end implies the end of all before it.  A caller's
+// kernel need not do that (itself launched so, it may end while what it depends on still
+// writes), so the first kernel of a call is a plain launch, ordered after everything.  A call is
 // five or six kernels of 4 to 10 us on a small cache, where the gaps between them count:
 // one layer 1x8x4096x128 59 -> 49 us per call, policy 16x8x3001x64 198 -> 192, redundancy
 // 2x8x5003x128 125 -> 119, host repair 9x8x8192x128 1003 -> 981.

@@ -1704,14 +1704,19 @@ cudaError_t config_select(const RepairArgs& a, cudaStream_t st, cudaLaunchConfig
     cfg.blockDim = dim3(kT);
     cfg.dynamicSmemBytes = bytes;
     cfg.stream = st;
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // as launch_dependent
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    at[1].id = cudaLaunchAttributeClusterDimension;
-    at[1].val.clusterDim.x = C;
-    at[1].val.clusterDim.y = 1;
-    at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = C > 1 ? 2 : 1;   // one CTA per unit: no cluster
+    if (a.dependent) {   // as launch_dependent
+        cudaLaunchAttribute& p = at[cfg.numAttrs++];
+        p.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        p.val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (C > 1) {         // one CTA per unit: no cluster
+        cudaLaunchAttribute& p = at[cfg.numAttrs++];
+        p.id = cudaLaunchAttributeClusterDimension;
+        p.val.clusterDim.x = C;
+        p.val.clusterDim.y = 1;
+        p.val.clusterDim.z = 1;
+    }
     return cudaSuccess;
 }
 
@@ -1781,7 +1786,9 @@ cudaError_t launch_repair(const RepairArgs& a, cudaStream_t st)
     const cudaError_t e = cudaFuncSetAttribute(
         dedup_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
     if (e != cudaSuccess) return e;
-    return launch_dependent(dedup_kernel, dim3(a.U), kT, bytes, st, a);
+    if (a.dependent) return launch_dependent(dedup_kernel, dim3(a.U), kT, bytes, st, a);
+    dedup_kernel<<<a.U, kT, bytes, st>>>(a);
+    return cudaGetLastError();
 }
 
 }  // namespace twk
