@@ -262,8 +262,8 @@ twinkv_status twinkv_repair_select_noalloc(const double* score_ret, twinkv_shape
  * units' keys go to the device in chunks of at most `chunk_units` units (0: the value
  * twinkv_host_default_chunk returns).  Nothing computes while the first chunk copies
  * in and each chunk's compute has to cover the next one's copy, so the chunks grow
- * from one unit by x2.5 (sizes of a whole wave of 128-row blocks, one per SM, or more
- * rounded to the nearest multiple of such a wave) up to `chunk_units`.
+ * from one unit by x2.5 (sizes of a whole wave of 256-row blocks, one per pair of SMs, or
+ * more rounded to the nearest multiple of such a wave) up to `chunk_units`.
  * Per chunk, ordered by events:
  *   - its keys and mask are copied in on a copy stream the library keeps per device;
  *   - its prefix counts, retained-first layout and audit run on `stream`;
@@ -286,9 +286,9 @@ twinkv_status twinkv_repair_select_noalloc(const double* score_ret, twinkv_shape
 size_t twinkv_host_arena_size(twinkv_shape s, int32_t chunk_units);
 /* The chunk size twinkv_repair_host and twinkv_host_arena_size use for chunk_units = 0
  * on the current device: about L*H / 8 units, rounded to the nearest multiple of
- * sms / gcd(sms, ceil(N / 128)), the number of units whose 128-row blocks fill every
- * SM an equal number of times (so no chunk's audit ends in a partial wave), clamped
- * to [1, L*H]; without a device, L*H / 8 unrounded.  Returns 0 for an invalid shape. */
+ * p / gcd(p, ceil(N / 256)), p = sms / 2, the number of units whose 256-row blocks fill
+ * every pair of SMs an equal number of times (so no chunk's audit ends in a partial
+ * wave), clamped to [1, L*H]; without a device, L*H / 8 unrounded.  Returns 0 for an invalid shape. */
 int32_t twinkv_host_default_chunk(twinkv_shape s);
 twinkv_status twinkv_repair_host(const void* keys, twinkv_shape s, const uint8_t* retained_mask,
                                  const int32_t* budget, float threshold,

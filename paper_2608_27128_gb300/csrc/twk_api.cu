@@ -290,21 +290,25 @@ twinkv_status run_refine(const uint16_t* k16, const twinkv_shape& s, const float
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 // ---- host-buffer pipeline (twinkv_repair_host) ------------------------------------
-// The number of units whose 128-row blocks fill `sms` SMs an equal number of times.
+// The number of units whose work items (kPM rows, one per CTA pair) fill the pairs of `sms`
+// SMs an equal number of times.
 int wave_units(const twinkv_shape& s, int sms)
 {
-    const int rb = (s.N + kBM - 1) / kBM;
-    return sms > 0 ? sms / std::gcd(sms, rb) : 0;
+    const int items = (s.N + kPM - 1) / kPM, pairs = sms / 2;
+    return pairs > 0 ? pairs / std::gcd(pairs, items) : 0;
 }
 
 // Units per chunk of the host path when the caller passes 0: about an eighth of the
-// units, so that later chunks' copies hide behind earlier chunks' compute, rounded to
-// the nearest multiple of the unit count whose row blocks are a whole number of waves
-// over the SMs (the persistent audit then ends no launch in a partial wave).
+// units, so that later chunks' copies hide behind earlier chunks' compute, but 4 MB of keys
+// at least (a chunk's launches and copies take some 20 us to queue: 288 units of 300 x 64
+// take 215 us in chunks of 38, 1.5 MB, and 163 in chunks of 152), rounded to
+// the nearest multiple of the unit count whose work items are a whole number of rounds over
+// the CTA pairs (the persistent audit then ends no launch in a partial round).
 int default_chunk_units(const twinkv_shape& s)
 {
     const int U = s.L * s.H;
-    int uc = (U + 7) / 8;
+    const int64_t unit = static_cast<int64_t>(s.N) * s.d * (s.dtype == TWINKV_F32 ? 4 : 2);
+    int uc = std::max((U + 7) / 8, static_cast<int>((4 << 20) / unit));
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) == cudaSuccess &&
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
