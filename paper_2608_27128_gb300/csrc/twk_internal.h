@@ -77,7 +77,7 @@ struct RepairArgs {
     bool dependent;             // launched as the programmatic dependent of the kernel before it
 };
 
-// CTAs per unit of the literal repair's selection: a power of two up to 8 (see the
+// CTAs per unit of the literal repair's selection: a power of two up to 16 (see the
 // definition for where the lines lie).
 int select_cluster_size(int U, int N, int sms);
 

@@ -11,11 +11,11 @@
 //   orphan k); a unit whose mask has a byte > 1 or whose popcount differs from its
 //   budget gets status, nswaps = -1 and S1 = S0.
 //
-// The literal rule (select_kernel<C>) runs each unit on a cluster of C CTAs (C = 1 to 8 by
-// select_cluster_size; 16 can be forced): by buckets in shared memory where the swap list
-// fits (see "bucket path" below), else by a radix select and sorts over the workspace
-// ("cluster selection").  Its scratch is caller workspace ([U][N] keys and positions,
-// twice) and 72 KB of dynamic shared memory per CTA.
+// The literal rule (select_kernel<C>) runs each unit on a cluster of C CTAs (C = 1 to 16 by
+// select_cluster_size): by buckets in shared memory (see "bucket path" below) up to 2^18
+// positions, a unit with an overfull bucket of several values and longer ones by a radix
+// select and sorts over the workspace ("cluster selection").  Its scratch is caller workspace
+// ([U][N] keys and positions, twice) and 72 KB of dynamic shared memory per CTA.
 //
 // Dedup variant (dedup_kernel, given the twin of every position; one 512-thread block
 // per unit): evicting a donor keeps its twin, so a twin pair never loses both members.
@@ -489,18 +489,39 @@ __device__ __forceinline__ void cluster_sync()
     else cg::this_cluster().sync();
 }
 
-// The same shared-memory object in CTA `rank` of the cluster.
-template <int C, typename T>
-__device__ __forceinline__ T* peer(T* p, int rank)
+// The value of the same shared-memory object in CTA `rank` of the cluster, by a 32-bit
+// shared::cluster address (generic pointers made the kernel spill).
+__device__ __forceinline__ int load_at(uint32_t at, int)
 {
-    if constexpr (C == 1) return p;
-    else return cg::this_cluster().map_shared_rank(p, rank);
+    int v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
+    return v;
 }
+__device__ __forceinline__ uint64_t load_at(uint32_t at, uint64_t)
+{
+    uint64_t v;
+    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(at) : "memory");
+    return v;
+}
+template <int C, typename T>
+__device__ __forceinline__ T peer(const T* p, int rank)
+{
+    if constexpr (C == 1) return *p;
+    else return load_at(cluster_addr(p, static_cast<uint32_t>(rank)), T());
+}
+
+constexpr int kMaxHeavy = 32;   // buckets ranked by position in a unit's selection
 
 struct ClusterShared {
     int cnt[8];          // this CTA's orphans, donors, retained count, invalid-byte flag;
                          // bucket path: smallest and largest orphan, then donor, as_int order
     int all[8];          // bucket path: the same over the cluster
+    // the bucket path's overfull buckets (see rank_heavy): how many; which, how many items,
+    // the first one's rank, the least and largest key and the count in this slice, the rank
+    // of the slice's next item
+    int n_heavy;
+    int hk[kMaxHeavy], hc[kMaxHeavy], hrank[kMaxHeavy], hcnt[kMaxHeavy], hnext[kMaxHeavy];
+    uint64_t hmin[kMaxHeavy], hmax[kMaxHeavy];
     int lcnt[2];         // compaction: this CTA's items below the cut and at it
     int hist[2][256];    // this CTA's digit histogram, alternating between passes
     int tot[8];          // cluster-wide values derived by thread 0
@@ -511,15 +532,20 @@ __device__ __forceinline__ bool before(uint64_t ka, int pa, uint64_t kb, int pb)
     return ka < kb || (ka == kb && pa < pb);
 }
 
-// Number of entries of the sorted (key, position) array of P = 2^k entries that order
-// before (k, p).
-__device__ __forceinline__ int count_before(const uint64_t* sk, const int* si, int P, uint64_t k,
-                                            int p)
+// Number of entries of the sorted (key, position) array of P = 2^k entries in CTA `rank`'s
+// shared memory that order before (k, p).
+__device__ __forceinline__ int count_before(const uint64_t* sk, const int* si, int rank, int P,
+                                            uint64_t k, int p)
 {
+    const uint32_t ak = cluster_addr(sk, static_cast<uint32_t>(rank));
+    const uint32_t ai = cluster_addr(si, static_cast<uint32_t>(rank));
+    auto first = [&](int at) {
+        return before(load_at(ak + 8u * at, uint64_t()), load_at(ai + 4u * at, 0), k, p);
+    };
     int pos = 0;
     for (int half = P >> 1; half > 0; half >>= 1)
-        if (before(sk[pos + half - 1], si[pos + half - 1], k, p)) pos += half;
-    if (before(sk[pos], si[pos], k, p)) ++pos;
+        if (first(pos + half - 1)) pos += half;
+    if (first(pos)) ++pos;
     return pos;
 }
 
@@ -570,6 +596,9 @@ __device__ __forceinline__ void load_run(const uint64_t* sk, const int* si, int 
     }
 }
 
+// x, as a value that the compiler knows nothing about.
+__device__ __forceinline__ void forget(int& x) { asm volatile("" : "+r"(x)); }
+
 constexpr int kEA = 8;   // consecutive positions per thread in the classification pass
 
 // Slice length: ceil(N / C) rounded up to a multiple of kEA.
@@ -593,17 +622,37 @@ __host__ __device__ inline int slice_len(int N, int C)
 // An item's rank is its bucket's first rank plus the number of items of its bucket ordered
 // before it, counted one by one.  The intervals are taken on b rounded toward zero to fp32,
 // which keeps the order, so the ranks are those of the (key, position) order whatever the
-// values.  Where the shares would not fit in shared memory or a bucket is too full to count
-// through (many equal values), the general path below does the whole unit instead.
+// values.  A unit that does not fit so goes on in rank_many: lists beyond the shared memory
+// window by window, overfull buckets of one value (exact duplicate keys, coarse scores) by
+// position (rank_heavy).  Only an overfull bucket of several values is left to the general
+// path.
 // Why: the selection is bound by latency, the round trips of its passes and barriers.  The
 // general path's radix select takes up to eight passes over lists in memory with several
 // block barriers each, and its bitonic sort was 58 of 182 thousand cycles per unit at 16384
-// positions.  General -> buckets, with the cluster size each was given: 288 units of 16384
-// positions 120 -> 64 us, 8 of 8192 67 -> 23, 8 of 4096 57 -> 16, 8 of 131072 128 -> 65,
-// 128 of 8192 64 -> 27.
+// positions.  General -> buckets, half of the positions kept, 20 % of b near 1: 288 units of
+// 16384 positions 119 -> 59 us, 128 of 8192 62 -> 23, 8 of 4096 55 -> 14, 8 of 8192 67 -> 19,
+// 8 of 131072 289 -> 89; 50 % near 1 (lists beyond one window) 288 of 16384 394 -> 109, 8 of
+// 131072 629 -> 203; 30 % equal to 1 288 of 16384 182 -> 125, 288 of 4096 58 -> 39, 8 of
+// 131072 363 -> 174.  What is left to the general path has paid for the attempt: with 60 % of
+// b within 1e-6 of 0.5, 288 of 16384 197 -> 231, 288 of 4096 62 -> 76 (8 of 8192 88 -> 64, by
+// fewer CTAs).
 constexpr int kBk = 1024;      // buckets per side
 constexpr int kCap = 3072;     // items per side a CTA holds (36 KB): two CTAs per SM fit
-constexpr int kMaxBucket = 256;
+// The number of items of a bucket above which counting one by one costs too much.  Buckets
+// are as full as the unit is long: at 131072 positions with normally distributed b up to 330
+// items (8 units 89 us counted through, 267 by the general path).
+__host__ __device__ inline int max_bucket(int N) { return min(1024, max(256, N / 256)); }
+
+// Beyond this a unit's buckets are too full whatever its values: the general path only.
+constexpr int kBucketMaxN = 1 << 18;
+
+// Where a unit has an overfull bucket, its buckets of one value and more than this many items
+// are ranked by position as well.
+constexpr int kFew = 48;
+
+// How far the bucket path got: all done; counts and ranges are in cs.all (and S1 = S0); or
+// also the buckets' first ranks are in s.warp_cnt and the ends of what is in play in cs.tot.
+enum Attempt { kNone, kDone, kCounted, kRanked };
 
 // A float's bits as an int with the float's order.
 __device__ __forceinline__ int as_int(float f)
@@ -706,11 +755,371 @@ __device__ void dedup_swap(Shared& s, uint64_t* sk, int* si, const Buckets& bd,
                            const RepairArgs& a, int u, const int* end, int n_o, uint64_t ktau,
                            const int (&rank)[2][kCap / kT]);
 
-// Runs the unit by buckets; every thread of the cluster calls it.  False (and, apart from
+// The thread's kP positions of the step at c0: c0 + tid, + kT, ...
+template <int kP>
+__device__ __forceinline__ void load_step(const uint8_t* S0, const double* b, int c0, int hi,
+                                          uint32_t (&mv)[kP], double (&bv)[kP])
+{
+#pragma unroll
+    for (int j = 0; j < kP; ++j) {
+        const int i = c0 + j * kT + static_cast<int>(threadIdx.x);
+        mv[j] = i < hi ? S0[i] : 255u;
+        bv[j] = i < hi ? b[i] : 0.0;
+    }
+}
+
+// For a unit with an overfull bucket (more than max_bucket items in play): the buckets of one
+// value and more than kFew items are ranked by position, which takes no counting and no place
+// in shared memory.  They leave the buckets' places (base, cur): base is marked with the top
+// bit and cur holds the bucket's number.  A first pass finds which candidates hold one value
+// and counts this slice's items; a second one goes through the slice in position order (warp
+// votes, then a prefix over the rows of a step, as in a radix pass) and writes their swaps.
+// cs.tot is then the fullest of the other buckets and the ends of the places in play.  False,
+// with nothing written, where an overfull bucket holds several values or there are too many.
+template <int C>
+__device__ bool rank_heavy(Shared& s, ClusterShared& cs, int* rows, const RepairArgs& a, int u,
+                           int r, int m)
+{
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int64_t off = static_cast<int64_t>(u) * a.N;
+    const uint8_t* S0 = a.mask + off;
+    const double* b = a.b + off;
+    const int slice = slice_len(a.N, C);
+    const int lo = min(a.N, r * slice), hi = min(a.N, lo + slice);
+    const uint64_t ktau = ordered(a.tau);
+    int* base = &s.warp_cnt[0][0];
+    int* cur = base + 2 * kBk;
+    constexpr int kPer = 2 * kBk / kT;
+    const int b0 = tid * kPer, side = b0 / kBk, limit = max_bucket(a.N);
+
+    // 1. the candidates
+    int first[kPer + 1];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) first[k] = base[b0 + k];
+    first[kPer] = (b0 + kPer) % kBk ? base[b0 + kPer] : cs.all[side];
+    int least = kFew, id, unused, n_all;
+    for (;;) {
+        int n = 0;
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) n += first[k] < m && first[k + 1] - first[k] > least;
+        scan2n(s, n, 0, id, unused, n_all, unused);   // (every thread has read base and tot)
+        if (n_all <= kMaxHeavy) break;
+        if (least == limit) return false;             // alike in every CTA
+        least = limit;
+    }
+    if (tid == 0) cs.n_heavy = n_all;
+    if (tid < kMaxHeavy) {
+        cs.hmin[tid] = ~0ull;
+        cs.hmax[tid] = 0ull;
+        cs.hcnt[tid] = 0;
+    }
+#pragma unroll
+    for (int k = 0, h = id; k < kPer; ++k) {
+        const int c = first[k + 1] - first[k];
+        if (first[k] >= m || c <= least) continue;
+        cs.hc[h] = c;
+        cs.hk[h] = b0 + k;
+        cs.hrank[h] = first[k];
+        base[b0 + k] |= static_cast<int>(0x80000000u);
+        cur[b0 + k] = h++;
+    }
+    __syncthreads();
+
+    const Buckets bo = make_buckets(from_int(cs.all[4]), from_int(cs.all[5]));
+    const Buckets bd = make_buckets(from_int(cs.all[7]), from_int(cs.all[6]));
+    constexpr int kStep = 4, kRows = kStep * kW;   // rows of 512 positions at a time
+    static_assert(kRows == 64, "two rows per lane");
+    // the overfull bucket of position i, or -1; its side and severity key
+    auto heavy_at = [&](int i, uint32_t mi, double bi, int& x, uint64_t& key) {
+        const uint64_t ki = ordered(bi);
+        x = i < hi ? side_of(mi, bi, ki, i, a, ktau) : 2;
+        if (x == 2) return -1;
+        key = x ? ~ki : ki;
+        const int k = x * kBk + bucket_of(narrow(static_cast<uint64_t>(__double_as_longlong(bi))),
+                                          x ? bd : bo);
+        return base[k] < 0 ? cur[k] : -1;
+    };
+
+    // 2. one value each?  And how many this slice holds
+#pragma unroll 1
+    for (int c0 = lo; c0 < hi; c0 += kT * kStep) {
+        uint32_t mv[kStep];
+        double bv[kStep];
+        load_step<kStep>(S0, b, c0, hi, mv, bv);
+        int mixed = 0;
+#pragma unroll
+        for (int j = 0; j < kStep; ++j) {
+            int x;
+            uint64_t key = 0;
+            const int h = heavy_at(c0 + j * kT + tid, mv[j], bv[j], x, key);
+            const uint32_t peers = __match_any_sync(0xFFFFFFFFu, h);
+            if (h < 0) continue;
+            volatile uint64_t* mn = &cs.hmin[h];
+            volatile uint64_t* mx = &cs.hmax[h];
+            if (lane == __ffs(peers) - 1) atomicAdd(&cs.hcnt[h], __popc(peers));
+            if (key < *mn) atomicMin(reinterpret_cast<unsigned long long*>(&cs.hmin[h]), key);
+            if (key > *mx) atomicMax(reinterpret_cast<unsigned long long*>(&cs.hmax[h]), key);
+            mixed |= *mn != *mx && cs.hc[h] > limit;
+        }
+        if (__syncthreads_or(mixed)) break;   // the verdict below sees it in every CTA
+    }
+    cluster_sync<C>();
+    int mixed = 0;
+    if (tid < n_all) {
+        uint64_t mn = ~0ull, mx = 0ull;
+        int before_me = cs.hrank[tid];
+        for (int q = 0; q < C; ++q) {
+            mn = min(mn, peer<C>(cs.hmin + tid, q));
+            mx = max(mx, peer<C>(cs.hmax + tid, q));
+            if (q < r) before_me += peer<C>(cs.hcnt + tid, q);
+        }
+        mixed = mn != mx && cs.hc[tid] > limit;
+        if (mn != mx) cs.hc[tid] = 0;                 // counted through after all
+        cs.hnext[tid] = before_me;
+    }
+    if (__syncthreads_or(mixed)) return false;        // alike in every CTA
+
+    // the ones of one value leave the places
+    int items = 0, top = 0, last = 0, before_me, all;
+#pragma unroll
+    for (int k = 0, h = id; k < kPer; ++k) {
+        const int c = first[k + 1] - first[k];
+        if (first[k] >= m) continue;
+        if (c > least && cs.hc[h++] > 0) items += c;
+        else top = max(top, c);
+    }
+    scan2n(s, items, 0, before_me, unused, all, unused);
+    if (tid == kT / 2) s.flag = before_me;            // what the orphans' side holds
+    if (tid < 3) cs.tot[tid] = 0;
+    __syncthreads();
+    if (side) before_me -= s.flag;
+#pragma unroll
+    for (int k = 0, h = id; k < kPer; ++k) {
+        const int c = first[k + 1] - first[k], place = first[k] - before_me;
+        const bool candidate = first[k] < m && c > least;
+        if (candidate && cs.hc[h] > 0) {
+            base[b0 + k] = place | static_cast<int>(0x80000000u);
+            before_me += c;
+        } else {
+            base[b0 + k] = cur[b0 + k] = place;
+            if (first[k] < m) last = max(last, place + c);
+        }
+        h += candidate;
+    }
+    atomicMax(&cs.tot[0], top);
+    atomicMax(&cs.tot[1 + side], last);
+    __syncthreads();
+
+    // 3. their ranks in position order
+    int* swaps = a.out_swaps + static_cast<int64_t>(u) * 2 * (a.N / 2);
+    uint8_t* S1 = a.out_mask + off;
+#pragma unroll 1
+    for (int c0 = lo; c0 < hi; c0 += kT * kStep) {
+        for (int i = tid; i < n_all * kRows; i += kT) rows[i] = 0;
+        __syncthreads();
+        int code[kStep];   // bucket, rank within the warp's row, side; or -1
+        uint32_t mv[kStep];
+        double bv[kStep];
+        load_step<kStep>(S0, b, c0, hi, mv, bv);
+#pragma unroll
+        for (int j = 0; j < kStep; ++j) {
+            int x;
+            uint64_t key;
+            const int h = heavy_at(c0 + j * kT + tid, mv[j], bv[j], x, key);
+            const uint32_t peers = __match_any_sync(0xFFFFFFFFu, h);
+            const int rk = __popc(peers & ((1u << lane) - 1u));
+            if (h >= 0 && rk == 0) rows[h * kRows + j * kW + wid] = __popc(peers);
+            code[j] = h < 0 ? -1 : h << 6 | rk << 1 | x;
+        }
+        __syncthreads();
+        for (int h = wid; h < n_all; h += kW) {
+            const int at = h * kRows + 2 * lane;
+            const int r0 = rows[at], r1 = rows[at + 1], next = cs.hnext[h];
+            int incl = r0 + r1;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            rows[at] = next + incl - r0 - r1;
+            rows[at + 1] = next + incl - r1;
+            if (lane == 31) cs.hnext[h] = next + incl;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kStep; ++j) {
+            if (code[j] < 0) continue;
+            const int h = code[j] >> 6, x = code[j] & 1, i = c0 + j * kT + tid;
+            const int rank = rows[h * kRows + j * kW + wid] + ((code[j] >> 1) & 31);
+            if (rank < m) {
+                swaps[2 * rank + (x ? 0 : 1)] = i;
+                S1[i] = x ? 0 : 1;
+            }
+        }
+        __syncthreads();
+    }
+    cluster_sync<C>();   // the rows are free for the peers' items
+    return true;
+}
+
+// The end of the bucket path: the items in play go to their buckets' owners, and every owner
+// writes the swaps of its own.  kMany: window by window of C * share places, beside overfull
+// buckets that have none.
+template <int C, bool kDedup, bool kMany>
+__device__ __forceinline__ void place_and_rank(Shared& s, ClusterShared& cs, uint64_t* sk, int* si,
+                                               const RepairArgs& a, int u, int r, int m, int share,
+                                               const int (&end)[2], const Buckets& bo,
+                                               const Buckets& bd, const uint8_t* S0,
+                                               const double* b, uint8_t* S1, int lo, int hi,
+                                               uint64_t ktau)
+{
+    constexpr int kP = C == 1 && !kMany ? 8 : 4;   // positions per thread and step
+    const int tid = threadIdx.x;
+    int* base = &s.warp_cnt[0][0];
+    int* cur = base + 2 * kBk;
+    constexpr int kPlace = kMany ? 0x7FFFFFFF : -1;   // overfull buckets have the top bit
+    constexpr bool kWrap = C > 1 || kMany;            // a CTA's places need not start at 0
+    auto slot = [](int g) { return kWrap ? g % kCap : g; };
+    auto bucket = [&](int x, uint64_t bits) { return bucket_of(narrow(bits), x ? bd : bo); };
+    // the place of a bucket in the window, or beyond its end (an overfull one always)
+    auto in_window = [&](int x, int place, int w0) {
+        if constexpr (!kMany) return place < (kDedup && x ? cs.all[1] : m);
+        return static_cast<unsigned>(place) - static_cast<unsigned>(w0) <
+               static_cast<unsigned>(max(0, min(end[x] - w0, C * share)));
+    };
+
+    for (int w0 = 0;; w0 += C * share) {
+        // the window's items to their buckets' owners
+        for (int c0 = lo; c0 < hi; c0 += kT * kP) {
+            uint32_t mv[kP];
+            double bv[kP];
+            load_step<kP>(S0, b, c0, hi, mv, bv);
+#pragma unroll
+            for (int j = 0; j < kP; ++j) {
+                const int i = c0 + j * kT + tid;
+                const uint64_t ki = ordered(bv[j]);
+                const int x = i < hi ? side_of(mv[j], bv[j], ki, i, a, ktau) : 2;
+                if (x == 2) continue;
+                const int k = x * kBk + bucket(x, static_cast<uint64_t>(__double_as_longlong(bv[j])));
+                if (!in_window(x, base[k], w0)) continue;
+                if constexpr (C == 1) {
+                    const int at = x * kCap + slot(atomicAdd(&cur[k], 1));
+                    sk[at] = x ? ~ki : ki;
+                    si[at] = i;
+                } else {
+                    const int t = (base[k] - w0) / share;
+                    const int at = x * kCap + slot(peer_add(cur + k, t, 1));
+                    peer_store(sk + at, t, x ? ~ki : ki);
+                    peer_store(si + at, t, i);
+                }
+            }
+        }
+        // this CTA's own items: the places from its first bucket's to its last one's end
+        int g0[2] = {0, 0}, g1[2] = {end[0], end[1]};
+        if constexpr (C > 1 || kMany) {
+#pragma unroll 1
+            for (int k = threadIdx.x; k < 2 * kBk; k += kT) {
+                const int x = k / kBk, bk = base[k];
+                const int ek = (k + 1) % kBk ? base[k + 1] & kPlace : kMany ? end[x] : cs.all[x];
+                if (in_window(x, bk, w0) && ek > bk && (C == 1 || (bk - w0) / share == r)) {
+                    atomicMin(&cs.tot[4 + x], bk);
+                    atomicMax(x ? &s.sel_before : &s.sel_digit, ek);
+                }
+            }
+        }
+        cluster_sync<C>();
+        if constexpr (C > 1 || kMany) {
+            g0[0] = cs.tot[4];
+            g0[1] = cs.tot[5];
+            g1[0] = s.sel_digit;
+            g1[1] = s.sel_before;
+        }
+        // the rank of the item at place g of side x
+        auto rank_of = [&](int x, int g) {
+            const uint64_t key = sk[x * kCap + slot(g)];
+            const int pos = si[x * kCap + slot(g)];
+            const int k = bucket(x, bits_of_key(key, x));
+            const int from_g = base[x * kBk + k];
+            const int to_g =
+                k + 1 < kBk ? base[x * kBk + k + 1] & kPlace : kMany ? end[x] : cs.all[x];
+            int rank = from_g;
+            if constexpr (kMany)   // the overfull buckets before it have ranks but no places
+                for (int h = 0; h < cs.n_heavy; ++h)
+                    rank += cs.hk[h] / kBk == x && cs.hk[h] < x * kBk + k ? cs.hc[h] : 0;
+            int at = x * kCap + slot(from_g);
+#pragma unroll 4
+            for (int n = to_g - from_g; n > 0; --n) {
+                rank += before(sk[at], si[at], key, pos) ? 1 : 0;
+                ++at;
+                if (kWrap && at == (x + 1) * kCap) at = x * kCap;
+            }
+            return rank;
+        };
+        if constexpr (kDedup) {
+            int rank[2][kCap / kT];
+#pragma unroll
+            for (int x = 0; x < 2; ++x)
+#pragma unroll
+                for (int j = 0; j < kCap / kT; ++j) {
+                    const int g = tid + j * kT;
+                    rank[x][j] = g < end[x] ? rank_of(x, g) : -1;
+                }
+            dedup_swap(s, sk, si, bd, a, u, end, cs.all[0], ktau, rank);
+            return;
+        }
+        int* swaps = a.out_swaps + static_cast<int64_t>(u) * 2 * (a.N / 2);
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+            for (int g = g0[x] + tid; g < g1[x]; g += kT) {
+                const int rank = rank_of(x, g), pos = si[x * kCap + slot(g)];
+                if (rank < m) {
+                    swaps[2 * rank + (x ? 0 : 1)] = pos;
+                    S1[pos] = x ? 0 : 1;
+                }
+            }
+        if (!kMany || w0 + C * share >= max(end[0], end[1])) break;
+        cluster_sync<C>();   // the window's items and its ends have been read
+        if (tid < 2) cs.tot[4 + tid] = 1 << 30;
+        if (tid == 0) s.sel_digit = s.sel_before = 0;
+        __syncthreads();
+    }
+    if (r == 0 && tid == 0) {
+        a.out_nswaps[u] = m;
+        if (a.out_status) a.out_status[u] = 0;
+    }
+}
+
+// The rest of the bucket path for a unit with overfull buckets or with lists too long for one
+// window.  A function by itself, so that the usual path keeps its registers.
+template <int C>
+__device__ __noinline__ bool rank_many(Shared& s, ClusterShared& cs, const RepairArgs& a, int u,
+                                       int r)
+{
+    extern __shared__ __align__(16) uint32_t dyn[];
+    uint64_t* sk = reinterpret_cast<uint64_t*>(dyn);
+    int* si = reinterpret_cast<int*>(sk + 2 * kCap);
+    const int m = min(cs.all[0], cs.all[1]);
+    if (cs.tot[0] > max_bucket(a.N) && !rank_heavy<C>(s, cs, reinterpret_cast<int*>(sk), a, u, r, m))
+        return false;
+    // as few windows as hold all places, and these dealt out evenly
+    const int end[2] = {cs.tot[1], cs.tot[2]}, places = max(end[0], end[1]);
+    const int most = C * (kCap - cs.tot[0]), wins = max(1, (places + most - 1) / most);
+    const int share = max(1, (places + C * wins - 1) / (C * wins));
+    const Buckets bo = make_buckets(from_int(cs.all[4]), from_int(cs.all[5]));
+    const Buckets bd = make_buckets(from_int(cs.all[7]), from_int(cs.all[6]));
+    const int64_t off = static_cast<int64_t>(u) * a.N;
+    const int slice = slice_len(a.N, C);
+    const int lo = min(a.N, r * slice), hi = min(a.N, lo + slice);
+    place_and_rank<C, false, true>(s, cs, sk, si, a, u, r, m, share, end, bo, bd, a.mask + off,
+                                   a.b + off, a.out_mask + off, lo, hi, ordered(a.tau));
+    return true;
+}
+
+// Runs the unit by buckets; every thread of the cluster calls it.  Not kDone (and, apart from
 // S1 = S0, nothing written) where the unit is left to the general path.  kDedup (C = 1): every
 // donor is in play, not only the m most severe, and dedup_swap ends the unit.
 template <int C, bool kDedup = false>
-__device__ bool select_by_buckets(Shared& s, ClusterShared& cs, uint64_t* sk, int* si,
+__device__ Attempt select_by_buckets(Shared& s, ClusterShared& cs, uint64_t* sk, int* si,
                                   const RepairArgs& a, int u, int r)
 {
     const int64_t off = static_cast<int64_t>(u) * a.N;
@@ -726,23 +1135,13 @@ __device__ bool select_by_buckets(Shared& s, ClusterShared& cs, uint64_t* sk, in
     int* cur = base + 2 * kBk;       // [2][kBk] counts, then the next free place
     static_assert(sizeof(s.warp_cnt) == 4 * kBk * sizeof(int), "bucket arrays fill warp_cnt");
 
-    // the thread's kP positions of one step: c0 + tid, + kT, ...
-    auto load = [&](int c0, uint32_t (&mv)[kP], double (&bv)[kP]) {
-#pragma unroll
-        for (int j = 0; j < kP; ++j) {
-            const int i = c0 + j * kT + tid;
-            mv[j] = i < hi ? S0[i] : 255u;
-            bv[j] = i < hi ? b[i] : 0.0;
-        }
-    };
-
     // 1. counts and ranges
     int bad = 0, cnt = 0, n[2] = {0, 0};
     int mn[2] = {0x7FFFFFFF, 0x7FFFFFFF}, mx[2] = {-0x7FFFFFFF - 1, -0x7FFFFFFF - 1};
     for (int c0 = lo; c0 < hi; c0 += kT * kP) {
         uint32_t mv[kP];
         double bv[kP];
-        load(c0, mv, bv);
+        load_step<kP>(S0, b, c0, hi, mv, bv);
 #pragma unroll
         for (int j = 0; j < kP; ++j) {
             const int i = c0 + j * kT + tid;
@@ -787,8 +1186,7 @@ __device__ bool select_by_buckets(Shared& s, ClusterShared& cs, uint64_t* sk, in
         const bool mini = tid == 4 || tid == 6, maxi = tid == 5 || tid == 7;
         int v = mini ? 0x7FFFFFFF : maxi ? -0x7FFFFFFF - 1 : 0;
         for (int q = 0; q < C; ++q) {
-            const int* rc = peer<C>(cs.cnt, q);   // cnt[4], then ends[4]
-            const int x = rc[tid];
+            const int x = peer<C>(cs.cnt + tid, q);   // cnt[4], then ends[4]
             v = mini ? min(v, x) : maxi ? max(v, x) : tid == 3 ? v | x : v + x;
         }
         cs.all[tid] = v;
@@ -806,11 +1204,11 @@ __device__ bool select_by_buckets(Shared& s, ClusterShared& cs, uint64_t* sk, in
             a.out_nswaps[u] = status ? -1 : 0;
             if (a.out_status) a.out_status[u] = status;
         }
-        return true;
+        return kDone;
     }
-    // ranks in play per side; lists that cannot fit are left at once
+    // ranks in play per side; the dedup variant needs all of them at once
     const int lim_o = m, lim_d = kDedup ? tot[1] : m;
-    if (max(lim_o, lim_d) > C * kCap) return false;
+    if (kDedup && max(lim_o, lim_d) > kCap) return kCounted;
     // side x's bucket: orphans from the smallest b up, donors from the largest down
     const Buckets bo = make_buckets(from_int(ends[0]), from_int(ends[1]));
     const Buckets bd = make_buckets(from_int(ends[3]), from_int(ends[2]));
@@ -822,7 +1220,7 @@ __device__ bool select_by_buckets(Shared& s, ClusterShared& cs, uint64_t* sk, in
     for (int c0 = lo; c0 < hi; c0 += kT * kP) {
         uint32_t mv[kP];
         double bv[kP];
-        load(c0, mv, bv);
+        load_step<kP>(S0, b, c0, hi, mv, bv);
 #pragma unroll
         for (int j = 0; j < kP; ++j) {
             const int i = c0 + j * kT + tid;
@@ -835,7 +1233,7 @@ __device__ bool select_by_buckets(Shared& s, ClusterShared& cs, uint64_t* sk, in
     }
     // maxima, then minima (beyond every place, yet far from overflow for a CTA without items)
     if (tid < 8) cs.tot[tid] = (tid & 4) ? 1 << 30 : 0;
-    if (tid == 0) s.sel_digit = s.sel_before = 0;
+    if (tid == 0) s.sel_digit = s.sel_before = cs.n_heavy = 0;
     cluster_sync<C>();
     constexpr int kPer = 2 * kBk / kT;   // buckets per thread; side 0: the lower half of the block
     static_assert(kPer * kT == 2 * kBk && kW % 2 == 0, "whole warps per side");
@@ -845,7 +1243,7 @@ __device__ bool select_by_buckets(Shared& s, ClusterShared& cs, uint64_t* sk, in
     for (int k = 0; k < kPer; ++k) {
         c[k] = 0;
 #pragma unroll 1
-        for (int q = 0; q < C; ++q) c[k] += peer<C>(cur, q)[b0 + k];
+        for (int q = 0; q < C; ++q) c[k] += peer<C>(cur + b0 + k, q);
         sum += c[k];
     }
     int incl = sum;
@@ -875,94 +1273,11 @@ __device__ bool select_by_buckets(Shared& s, ClusterShared& cs, uint64_t* sk, in
     full = cs.tot[0];
     const int end[2] = {cs.tot[1], cs.tot[2]};   // items in play per side
     const int share = (max(end[0], end[1]) + C - 1) / C;
-    if (full > kMaxBucket || share + full > kCap) return false;   // alike in every CTA
-
-    // 3. the items in play to their buckets' owners
-    for (int c0 = lo; c0 < hi; c0 += kT * kP) {
-        uint32_t mv[kP];
-        double bv[kP];
-        load(c0, mv, bv);
-#pragma unroll
-        for (int j = 0; j < kP; ++j) {
-            const int i = c0 + j * kT + tid;
-            const uint64_t ki = ordered(bv[j]);
-            const int x = i < hi ? side_of(mv[j], bv[j], ki, i, a, ktau) : 2;
-            if (x == 2) continue;
-            const int k = x * kBk + bucket(x, static_cast<uint64_t>(__double_as_longlong(bv[j])));
-            if (base[k] >= (x ? lim_d : lim_o)) continue;
-            const int t = C == 1 ? 0 : base[k] / share;
-            if constexpr (C == 1) {
-                const int at = x * kCap + atomicAdd(&cur[k], 1);
-                sk[at] = x ? ~ki : ki;
-                si[at] = i;
-            } else {
-                const int at = x * kCap + peer_add(cur + k, t, 1) % kCap;
-                peer_store(sk + at, t, x ? ~ki : ki);
-                peer_store(si + at, t, i);
-            }
-        }
-    }
-    // this CTA's own items: the places from its first bucket's to its last one's end
-    int g0[2] = {0, 0}, g1[2] = {end[0], end[1]};
-    if constexpr (C > 1) {
-#pragma unroll 1
-        for (int k = threadIdx.x; k < 2 * kBk; k += kT) {
-            const int x = k / kBk, bk = base[k];
-            const int ek = (k + 1) % kBk ? base[k + 1] : x ? tot[1] : tot[0];
-            if (ek > bk && bk < m && bk / share == r) {
-                atomicMin(&cs.tot[4 + x], bk);
-                atomicMax(x ? &s.sel_before : &s.sel_digit, ek);
-            }
-        }
-    }
-    cluster_sync<C>();
-    if constexpr (C > 1) {
-        g0[0] = cs.tot[4];
-        g0[1] = cs.tot[5];
-        g1[0] = s.sel_digit;
-        g1[1] = s.sel_before;
-    }
-    // the rank of the item at place g of side x
-    auto rank_of = [&](int x, int g) {
-        const uint64_t key = sk[x * kCap + g % kCap];
-        const int pos = si[x * kCap + g % kCap];
-        const int k = bucket(x, bits_of_key(key, x));
-        const int from_g = base[x * kBk + k];
-        const int to_g = k + 1 < kBk ? base[x * kBk + k + 1] : tot[x];
-        int rank = from_g;
-        for (int h = from_g; h < to_g; ++h) {
-            const int at = x * kCap + h % kCap;
-            rank += before(sk[at], si[at], key, pos) ? 1 : 0;
-        }
-        return rank;
-    };
-    if constexpr (kDedup) {
-        int rank[2][kCap / kT];
-#pragma unroll
-        for (int x = 0; x < 2; ++x)
-#pragma unroll
-            for (int j = 0; j < kCap / kT; ++j) {
-                const int g = tid + j * kT;
-                rank[x][j] = g < end[x] ? rank_of(x, g) : -1;
-            }
-        dedup_swap(s, sk, si, bd, a, u, end, tot[0], ktau, rank);
-    } else {
-        int* swaps = a.out_swaps + static_cast<int64_t>(u) * 2 * (a.N / 2);
-#pragma unroll
-        for (int x = 0; x < 2; ++x)
-            for (int g = g0[x] + tid; g < g1[x]; g += kT) {
-                const int rank = rank_of(x, g), pos = si[x * kCap + g % kCap];
-                if (rank < m) {
-                    swaps[2 * rank + (x ? 0 : 1)] = pos;
-                    S1[pos] = x ? 0 : 1;
-                }
-            }
-        if (r == 0 && tid == 0) {
-            a.out_nswaps[u] = m;
-            if (a.out_status) a.out_status[u] = 0;
-        }
-    }
-    return true;
+    if (full > max_bucket(a.N) || share + full > kCap) return kRanked;   // alike in every CTA
+    // 3. (one window)
+    place_and_rank<C, kDedup, false>(s, cs, sk, si, a, u, r, m, share, end, bo, bd, S0, b, S1, lo,
+                                     hi, ktau);
+    return kDone;
 }
 
 // The end of the dedup variant's bucket path: the walk over the donors in severity order as
@@ -1085,13 +1400,22 @@ __global__ void __launch_bounds__(kT, 2) select_kernel(const RepairArgs a)
     int* si_o = reinterpret_cast<int*>(sk_d + kChunk);   // [kChunk] positions
     int* si_d = si_o + kChunk;
 
-    const int tid = threadIdx.x, lane = tid & 31;
+    int tid = threadIdx.x;
     int r = 0;
     if constexpr (C > 1) r = static_cast<int>(cg::this_cluster().block_rank());
-    const int u = static_cast<int>(blockIdx.x / C);
+    int u = static_cast<int>(blockIdx.x / C);
     wait_for_previous();
-    if (select_by_buckets<C>(s, cs, sk_o, reinterpret_cast<int*>(sk_o + 2 * kCap), a, u, r))
-        return;
+    if (a.N <= kBucketMaxN) {
+        int* si = reinterpret_cast<int*>(sk_o + 2 * kCap);
+        if (select_by_buckets<C>(s, cs, sk_o, si, a, u, r) == kDone) return;
+        forget(u);   // nothing computed from them stays in registers over what follows
+        forget(r);
+        if (rank_many<C>(s, cs, a, u, r)) return;
+        forget(u);
+        forget(r);
+        forget(tid);
+    }
+    const int lane = tid & 31;
     cluster_sync<C>();   // what the attempt left in shared memory is free
 
     const int N = a.N;
@@ -1206,15 +1530,14 @@ __global__ void __launch_bounds__(kT, 2) select_kernel(const RepairArgs a)
     if (tid == 0) {
         int n_o = 0, n_d = 0, tc = 0, tb = 0, bo = 0, bd = 0;
         for (int q = 0; q < C; ++q) {
-            const int* rc = peer<C>(cs.cnt, q);
             if (q == r) {
                 bo = n_o;
                 bd = n_d;
             }
-            n_o += rc[0];
-            n_d += rc[1];
-            tc += rc[2];
-            tb |= rc[3];
+            n_o += peer<C>(cs.cnt, q);
+            n_d += peer<C>(cs.cnt + 1, q);
+            tc += peer<C>(cs.cnt + 2, q);
+            tb |= peer<C>(cs.cnt + 3, q);
         }
         int status = 0;
         if (tb) status = 1;                                  // TWINKV_ERR_INVALID_ARG
@@ -1286,7 +1609,7 @@ __global__ void __launch_bounds__(kT, 2) select_kernel(const RepairArgs a)
             int own = 0;
             if (tid < 256) {
                 int t = 0;
-                for (int q = 0; q < C; ++q) t += peer<C>(h, q)[tid];
+                for (int q = 0; q < C; ++q) t += peer<C>(h + tid, q);
                 s.base[tid] = t;
                 own = h[tid];
             }
@@ -1322,24 +1645,25 @@ __global__ void __launch_bounds__(kT, 2) select_kernel(const RepairArgs a)
         if (tid == 0) {
             int sel_before = 0, eq_before = 0;
             for (int q = 0; q < r; ++q) {
-                const int* lc = peer<C>(cs.lcnt, q);
-                sel_before += lc[0] + max(0, min(lc[1], need - eq_before));
-                eq_before += lc[1];
+                const int at_cut_q = peer<C>(cs.lcnt + 1, q);
+                sel_before += peer<C>(cs.lcnt, q) + max(0, min(at_cut_q, need - eq_before));
+                eq_before += at_cut_q;
             }
             cs.tot[6] = sel_before;
             cs.tot[7] = eq_before;
         }
         __syncthreads();
+        constexpr int kEB = kEA / 2;   // (kEA would spill beside rank_many's call)
         int base = cs.tot[6], seen_eq = cs.tot[7];
-        for (int c0 = 0; c0 < mine; c0 += kT * kEA) {
-            // a thread takes kEA consecutive items; fl: below the cut (or at it when
+        for (int c0 = 0; c0 < mine; c0 += kT * kEB) {
+            // a thread takes kEB consecutive items; fl: below the cut (or at it when
             // `whole`), fe: at the cut
-            const int k0 = c0 + tid * kEA;
-            uint64_t kk[kEA];
-            int pp[kEA];
+            const int k0 = c0 + tid * kEB;
+            uint64_t kk[kEB];
+            int pp[kEB];
             uint32_t fl = 0, fe = 0;
 #pragma unroll
-            for (int j = 0; j < kEA; ++j) {
+            for (int j = 0; j < kEB; ++j) {
                 kk[j] = 0;
                 pp[j] = 0;
                 if (k0 + j < mine) {
@@ -1354,7 +1678,7 @@ __global__ void __launch_bounds__(kT, 2) select_kernel(const RepairArgs a)
             scan2n(s, __popc(fl), __popc(fe), pl, pe, tl, te);
             const int k_eq = max(0, min(te, need - seen_eq));   // taken at the cut here
 #pragma unroll
-            for (int j = 0; j < kEA; ++j) {
+            for (int j = 0; j < kEB; ++j) {
                 const int l = (fl >> j) & 1, e = (fe >> j) & 1;
                 if (l || (e && pe < k_eq)) {
                     const int dst = base + pl + min(pe, k_eq);
@@ -1466,8 +1790,7 @@ __global__ void __launch_bounds__(kT, 2) select_kernel(const RepairArgs a)
                 int rank = ts;
                 for (int qq = 0; qq < C; ++qq)
                     if (qq != r)
-                        rank += count_before(peer<C>(const_cast<uint64_t*>(k2), qq),
-                                             peer<C>(const_cast<int*>(i2), qq), P, key, pos);
+                        rank += count_before(k2, i2, qq, P, key, pos);
                 swaps[2 * rank + (sdx ? 0 : 1)] = pos;
                 S1[pos] = sdx ? 0 : 1;
             }
@@ -1495,6 +1818,44 @@ __global__ void __launch_bounds__(kT, 2) select_kernel(const RepairArgs a)
     }
 }
 
+// The dedup variant's counts where no attempt by buckets has left them: cs.all[0..3] (orphans,
+// donors, retained positions, whether a mask byte is invalid), and S1 = S0.
+__device__ void count_unit(ClusterShared& cs, const RepairArgs& a, int64_t off, uint64_t ktau)
+{
+    const uint8_t* S0 = a.mask + off;
+    const double* b = a.b + off;
+    uint8_t* S1 = a.out_mask + off;
+    int bad = 0, cnt = 0, no = 0, nd = 0;
+    for (int c0 = 0; c0 < a.N; c0 += kT * kE) {
+#pragma unroll
+        for (int j = 0; j < kE; ++j) {
+            const int i = c0 + threadIdx.x * kE + j;
+            if (i >= a.N) continue;
+            const uint32_t v = S0[i];
+            const double bi = b[i];
+            S1[i] = static_cast<uint8_t>(v);
+            bad |= v > 1u;
+            cnt += v != 0u;
+            const int x = side_of(v, bi, ordered(bi), i, a, ktau);
+            no += x == 0;
+            nd += x == 1;
+        }
+    }
+    if (threadIdx.x < 4) cs.all[threadIdx.x] = 0;
+    __syncthreads();
+    bad = __reduce_or_sync(0xFFFFFFFFu, bad);
+    cnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
+    no = __reduce_add_sync(0xFFFFFFFFu, no);
+    nd = __reduce_add_sync(0xFFFFFFFFu, nd);
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(&cs.all[0], no);
+        atomicAdd(&cs.all[1], nd);
+        atomicAdd(&cs.all[2], cnt);
+        atomicOr(&cs.all[3], bad);
+    }
+    __syncthreads();
+}
+
 __global__ void __launch_bounds__(kT, 2) dedup_kernel(const RepairArgs a)   // 2 blocks/SM
 {
     __shared__ Shared s;
@@ -1502,10 +1863,14 @@ __global__ void __launch_bounds__(kT, 2) dedup_kernel(const RepairArgs a)   // 2
     extern __shared__ __align__(16) uint32_t dyn[];
     wait_for_previous();
     const int u = blockIdx.x;
-    if (uint64_t* keys = reinterpret_cast<uint64_t*>(dyn); select_by_buckets<1, true>(
-            s, cs, keys, reinterpret_cast<int*>(keys + 2 * kCap), a, u, 0))
-        return;
-    __syncthreads();   // what the attempt left in shared memory is free
+    Attempt by_buckets = kNone;
+    if (a.N <= kBucketMaxN) {
+        uint64_t* keys = reinterpret_cast<uint64_t*>(dyn);
+        by_buckets = select_by_buckets<1, true>(s, cs, keys, reinterpret_cast<int*>(keys + 2 * kCap),
+                                                a, u, 0);
+        if (by_buckets == kDone) return;
+    }
+    __syncthreads();   // what the attempt left in shared memory can be written
     const int N = a.N;
     const int64_t off = static_cast<int64_t>(u) * N;
     const uint8_t* S0 = a.mask + off;
@@ -1513,47 +1878,14 @@ __global__ void __launch_bounds__(kT, 2) dedup_kernel(const RepairArgs a)   // 2
     uint8_t* S1 = a.out_mask + off;
     int* swaps = a.out_swaps + static_cast<int64_t>(u) * 2 * (N / 2);
 
-    // 1. validation, counts, and S1 = S0 (also the answer for a failed unit or m = 0)
-    int bad = 0, cnt = 0, no = 0, nd = 0;
-    // b < tau and b >= tau decided on the order-preserving keys (integer operations;
-    // a NaN b is neither an orphan nor a donor, as in fp64 comparisons)
+    // 1. counts and S1 = S0 (also the answer for a failed unit or m = 0), unless the attempt has
+    // done them
     const uint64_t ktau = ordered(a.tau);
-    for (int c0 = 0; c0 < N; c0 += kT * kE) {
-#pragma unroll
-        for (int j = 0; j < kE; ++j) {
-            const int i = c0 + threadIdx.x * kE + j;
-            if (i < N) {
-                const uint8_t v = S0[i];
-                const double bi = b[i];
-                const uint64_t ki = ordered(bi);
-                const bool num = !is_nan_bits(bi);
-                S1[i] = v;
-                bad |= v > 1;
-                cnt += v != 0;
-                const bool prot = i < a.n_sink || i >= N - a.n_recent;
-                no += (v == 0 && num && ki < ktau);
-                nd += (v != 0 && !prot && num && ki >= ktau);
-            }
-        }
-    }
-    if (threadIdx.x < 4) s.red[threadIdx.x] = 0;
-    __syncthreads();
-    bad = __reduce_or_sync(0xFFFFFFFFu, bad);
-    cnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
-    no = __reduce_add_sync(0xFFFFFFFFu, no);
-    nd = __reduce_add_sync(0xFFFFFFFFu, nd);
-    if ((threadIdx.x & 31) == 0) {
-        atomicOr(&s.red[0], bad);
-        atomicAdd(&s.red[1], cnt);
-        atomicAdd(&s.red[2], no);
-        atomicAdd(&s.red[3], nd);
-    }
-    __syncthreads();
+    if (by_buckets == kNone) count_unit(cs, a, off, ktau);
     int status = 0;
-    if (s.red[0]) status = 1;                                   // TWINKV_ERR_INVALID_ARG
-    else if (a.budget && a.budget[u] != s.red[1]) status = 3;   // TWINKV_ERR_BUDGET
-    const int n_o = s.red[2], n_d = s.red[3];
-    const int m = status ? 0 : min(n_o, n_d);
+    if (cs.all[3]) status = 1;                                   // TWINKV_ERR_INVALID_ARG
+    else if (a.budget && a.budget[u] != cs.all[2]) status = 3;   // TWINKV_ERR_BUDGET
+    const int m = status ? 0 : min(cs.all[0], cs.all[1]);
 
     if (status != 0 || m == 0) {
         if (threadIdx.x == 0) {
@@ -1563,7 +1895,13 @@ __global__ void __launch_bounds__(kT, 2) dedup_kernel(const RepairArgs a)   // 2
         return;
     }
 
-    // 2-3. classify and compact: orphans at [0, n_o), donors at [n_o, n_o + n_d)
+    // 2-3. classify and compact: orphans at [0, n_o), donors at [n_o, n_o + n_d).  Where the
+    // attempt has filled the buckets, of the orphans only those of the buckets that hold the m
+    // most severe ones, as no other can be admitted.
+    const bool ranked = by_buckets == kRanked;
+    const int n_o = ranked ? cs.tot[1] : cs.all[0], n_d = cs.all[1];
+    const Buckets bo = make_buckets(from_int(cs.all[4]), from_int(cs.all[5]));
+    const int* first_rank = &s.warp_cnt[0][0];
     uint64_t* k0 = a.keys0 + off;
     int* i0 = a.idx0 + off;
     uint64_t* k1 = a.keys1 + off;
@@ -1585,6 +1923,9 @@ __global__ void __launch_bounds__(kT, 2) dedup_kernel(const RepairArgs a)   // 2
                 const bool num = !is_nan_bits(bv[j]);
                 fo[j] = (v == 0 && num && kj < ktau);
                 fd[j] = (v != 0 && !prot && num && kj >= ktau);
+                if (fo[j] && ranked)
+                    fo[j] = first_rank[bucket_of(
+                                narrow(static_cast<uint64_t>(__double_as_longlong(bv[j]))), bo)] < m;
             }
             co += fo[j];
             cd += fd[j];
@@ -1749,12 +2090,20 @@ int select_cluster_size(int U, int N, int sms)
 {
     // More CTAs per unit while each has an SM to itself and 4096 positions or more: below
     // that the cluster's barriers cost more than the shorter passes save, and a second CTA
-    // on an SM halves both (us per selection with C = 1 / 2 / 4 / 8: 8 units of 4096
-    // positions 17 / 19 / 18 / 21, 8 of 32768 193 / 55 / 36 / 31, 72 of 8192 25 / 22 / 27 /
-    // 79, 288 of 16384 61 / 80 / 112 / 286).  Slices above 24576 positions are split
-    // whatever the number of units, since their swap lists seldom fit one CTA's buckets
-    // (8 units of 131072 by the general path 1127 / 617 / 350, by buckets at C = 8 82).
+    // on an SM halves both (us per selection with C = 1 / 2 / 4 / 8, half kept and 20 % of b
+    // near 1: 8 units of 4096 positions 14 / 15 / 15 / 19, 8 of 32768 117 / 55 / 35 / 29, 72 of
+    // 8192 23 / 19 / 25 / 70, 288 of 16384 59 / 80 / 111 / 284; 30 % of b equal to 1: 28 / 25 / 23
+    // / 27, 215 / 117 / 72 / 51, 48 / 37 / 37 / 108, 125 / 152 / 195 / 404).  Slices above 24576
+    // positions are split whatever the number of units, since their swap lists seldom fit one
+    // CTA's buckets at once (16 units of 65536 312 / 174 / 69 / 64; 8 of 131072 919 / 461 / 217 /
+    // 89, and 103 at 16).
+    // Beyond the buckets' reach (kBucketMaxN): as many CTAs as two per SM allow, up to 16 (one
+    // unit of 2^20 by the general path 3.80 ms at C = 4, 3.46 at 8, 3.31 at 16).
     int C = 1;
+    if (N > kBucketMaxN) {
+        while (C < 16 && static_cast<int64_t>(U) * (2 * C) <= 2LL * sms) C <<= 1;
+        return C;
+    }
     while (C < 8 && ((static_cast<int64_t>(U) * (2 * C) <= sms && N / (2 * C) >= 4096) ||
                      N / C > 24576))
         C <<= 1;
