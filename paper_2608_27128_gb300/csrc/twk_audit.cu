@@ -548,6 +548,13 @@ __device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity, uint6
         if (globaltimer_ns() - t0 > limit) return;
 }
 
+// Lets `ns` nanoseconds pass.
+__device__ __forceinline__ void hold_ns(uint64_t ns)
+{
+    const uint64_t t0 = globaltimer_ns();
+    while (globaltimer_ns() - t0 < ns) __nanosleep(1000000u);
+}
+
 // Position in a ring of kN slots: the slot in use and the parity of its current phase.
 template <int kN>
 struct Ring {
@@ -720,8 +727,11 @@ __global__ void __cluster_dims__(2, 1, 1)
                 }
                 if (!ok) {
                     // Let every copy this warp started land before the block exits.  A and B
-                    // copies of both CTAs complete on the even CTA's barriers; the odd CTA
-                    // leaves its own to that wait (the cluster barrier at the end follows it).
+                    // copies of both CTAs complete on the even CTA's barriers, which waits for
+                    // the slots that it has armed itself.  The odd CTA can be a ring ahead of
+                    // that and cannot wait on those barriers: it stays for as long as a drain
+                    // lasts at least (a copy takes microseconds).
+                    if (!leader) hold_ns(kDrainFloorNs);
                     for (int s = 0; leader && s < 2; ++s) {
                         const int p = ra.last_parity(s);
                         if (p >= 0) drain_wait(&a_full[s], p, a.timeout_ns);
