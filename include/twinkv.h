@@ -169,8 +169,8 @@ twinkv_status twinkv_redundancy(const void* keys, twinkv_shape s, int32_t window
 /*
  * twinkv_redundancy computed from half the similarity tiles (Sec. 3.5: the audit costs
  * O(n^2 d) per head; Eq. 1 is symmetric, sim(i,j) = sim(j,i)).  Row block rb (rows
- * [128 rb, 128 rb + 128)) computes only the 256-column tiles from the one holding
- * column 128 rb on; each tile's similarities serve both its rows (maxima over its
+ * [256 rb, 256 rb + 256)) computes only the 256-column tiles from its own columns,
+ * tile rb, on; each tile's similarities serve both its rows (maxima over its
  * columns) and its columns (maxima over its rows, the candidates of the rows those
  * columns stand for).  The two directions meet per row in a packed (value,
  * position) word combined with atomic maxima: the larger value, the lower position
@@ -309,8 +309,9 @@ twinkv_status twinkv_repair_host(const void* keys, twinkv_shape s, const uint8_t
  * m most severe orphans are admitted, the k-th evicted donor paired with the k-th
  * orphan.  Arguments, outputs and the workspace (TWINKV_OP_REPAIR) as for
  * twinkv_repair; N must not exceed 524288 (TWINKV_ERR_UNSUPPORTED otherwise: the walk
- * keeps two bits per donor in shared memory).  The walk is sequential per unit, so a
- * unit with many donors takes longer than in twinkv_repair.
+ * keeps two bits per donor in shared memory).  A unit whose donors fit in shared memory
+ * (3072, fewer with many equal scores) is walked in parallel rounds; a longer walk is
+ * sequential, so such a unit takes longer than in twinkv_repair.
  */
 twinkv_status twinkv_repair_dedup(const void* keys, twinkv_shape s, const uint8_t* retained_mask,
                                   const int32_t* budget, float threshold,

@@ -280,11 +280,11 @@ twinkv_status launch_select(const twinkv_shape& s, const double* b, const uint8_
 
 twinkv_status run_refine(const uint16_t* k16, const twinkv_shape& s, const float4* norm2,
                          const int* t0, int* t1, double* b0, double* b1, cudaStream_t st,
-                         bool beside_audit = false)
+                         bool between_audits = false)
 {
     ProfScope p(TWINKV_KERNEL_REFINE, st);
     return cuda_status(
-        launch_refine(k16, s.L * s.H, s.N, s.d, norm2, t0, t1, b0, b1, st, beside_audit));
+        launch_refine(k16, s.L * s.H, s.N, s.d, norm2, t0, t1, b0, b1, st, between_audits));
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
@@ -706,8 +706,8 @@ namespace {
 // The audit's inputs in `workspace`: bf16 keys (fp32 keys are rounded), the retained
 // prefix counts, and the retained-first column layout with its metadata and the norm
 // records.  *k16 receives the bf16 keys.
-twinkv_status prep_stages(const DeviceInfo* dev, const void* keys, const twinkv_shape& s, const uint8_t* retained_mask,
-                          bool need_all, void* workspace, const Layout& L, cudaStream_t st,
+twinkv_status prep_stages(const DeviceInfo* dev, const void* keys, const twinkv_shape& s,
+                          const uint8_t* retained_mask, bool need_all, void* workspace, const Layout& L, cudaStream_t st,
                           const uint16_t** k16)
 {
     uint16_t* const rows = keys_bf16(keys, s, workspace, L);
@@ -1008,7 +1008,7 @@ twinkv_status twinkv_repair_host(const void* keys, twinkv_shape s, const uint8_t
         return fail(TWINKV_ERR_CUDA);
     // Nothing computes while the first chunk copies in, and each chunk's compute has to
     // cover the next chunk's copy: the chunks grow from one unit by x2.5 (the audit of a
-    // unit takes about three times the copy of its keys) up to uc.  A size of one wave
+    // unit of 16384 x 128 takes 2.2 times the copy of its keys) up to uc.  A size of one wave
     // of units (wave_units) or more is rounded to the nearest whole number of waves.
     const int step = wave_units(s, dev->sms);
     auto next_size = [&](int prev) {

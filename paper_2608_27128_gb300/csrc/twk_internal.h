@@ -151,7 +151,7 @@ cudaError_t launch_scale_columns(float* colrinv, int U, int64_t NP, const unsign
 cudaError_t launch_refine(const uint16_t* keys, int U, int N, int d, const float4* norms,
                           const int* twin0, int* twin1, double* b0, double* b1,
                           cudaStream_t st,
-                          bool beside_audit = false);
+                          bool between_audits = false);
 
 // audit kernel (tensor maps built by the caller)
 size_t audit_smem_bytes(int d);

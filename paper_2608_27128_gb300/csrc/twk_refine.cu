@@ -1,9 +1,9 @@
 // twk_refine.cu -- exact value of the winning similarity (TwinKV, arXiv 2608.27128,
 // Sec. 3.2 Eq. 1).
 //
-// The audit kernel picks each row's twin from fp32 tensor-core dot products whose low
-// mantissa bits carry the column index, so its own score is only good to ~2^-16.  This
-// pass recomputes, for the chosen twin j of every row i,
+// The audit kernel picks each row's twin from fp32 tensor-core dot products, at d = 64 and in
+// the symmetric mode with the column index in their low mantissa bits, and outputs no score.
+// This pass computes, for the chosen twin j of every row i,
 //     sim(i, j) = (k_i . k_j) / sqrt((k_i . k_i) (k_j . k_j))
 // with every dot product formed as a double-float sum: each bf16 x bf16 product is
 // exact in fp32, and the running sum is an unevaluated pair (hi, lo) updated with
@@ -12,8 +12,8 @@
 // cosine is then (k_i . k_j) * (1/||k_i|| * 1/||k_j||) in double-float arithmetic
 // (relative error below 1e-12; fp64 square roots and quotients are slow on this GPU),
 // except within 2^-20 of +-1, where the exact fp64 form is used.  All dot products
-// (norms included) use the same routine and term order (the paired version used when a
-// row has two candidates computes each dot exactly as the single one), and the product
+// (norms included) use the same routine and term order (where a row has two candidates,
+// two of its sums run side by side), and the product
 // of the two inverse norms is formed symmetrically, so the result is symmetric in
 // (i, j) bit for bit and exactly 1 for a duplicate.
 #include "twk_df.cuh"
@@ -75,9 +75,12 @@ constexpr int kRowsPerBlock = kRefineThreads / kParts;
 // kParts threads per row.  Bound by the gathers of 256-byte rows from L2 (about 7 TB/s at
 // 18x8x8192x128) and, with both candidates, by the TwoSum instructions.  kMinBlocks is the
 // number of 256 threads that fit on an SM: 5 (48 registers) for one candidate, 4 (64) where
-// rows have two, whose sums need 8 registers more; 6 (40) on the host path's own stream.
-// Blocks of 128 threads leave less of an SM waiting for its
-// slowest rows than blocks of 256: 82 against 86 us at 18x8x8192x128, 53 against 56 at
+// rows have two, whose sums need 8 registers more; 6 (40) on the host path's own stream, whose
+// blocks start in the gaps between the audits of two chunks (an audit takes a whole register
+// file), most of them at once: alike with 5 and 4 there (repair from host memory, 6 / 5 or 4:
+// 9x8x8192x128 970 / 969 us, with both audits 1255 / 1247, 16x8x8192x64 1070 / 1068).
+// Blocks of 128 threads leave less of an SM waiting for its slowest rows than blocks of 256:
+// 82 against 86 us at 18x8x8192x128, 53 against 56 at
 // 16x8x8192x64, 221 against 232 with both candidates at 16x8x16384x128 (64 threads: 83, 72,
 // 217).  With even and odd elements summed in the halves of paired instructions, one
 // candidate went from 92 to 82 us and 62 to 53; two stay at 212 to 221.
@@ -100,9 +103,9 @@ __global__ void __launch_bounds__(kRefineThreads, kMinBlocks * 256 / kRefineThre
     // stood in for by the row itself and its value discarded.
     const int64_t s0 = base + (j0 >= 0 ? j0 : r - base);
     const int64_t s1 = base + (j1 >= 0 ? j1 : r - base);
-    // The standalone launch loads the norm records the cosine needs (the row's, and
-    // the twin's this lane evaluates) beside the keys rather than after the dot
-    // product; the host path's 40-register one has none to hold them.
+    // The norm records that the cosine needs (the row's, and the twin's this lane evaluates)
+    // are loaded beside the keys rather than after the dot product, except in the host path's
+    // 40-register form, which has none to hold them.
     constexpr bool kEarly = kMinBlocks < 6;
     float4 nr{}, nt{};
     if constexpr (kEarly) {
@@ -110,7 +113,7 @@ __global__ void __launch_bounds__(kRefineThreads, kMinBlocks * 256 / kRefineThre
         nt = norms[part == 1 ? s1 : s0];
     }
     DF d0, d1{0.f, 0.f};
-    if (__any_sync(0xFFFFFFFFu, j1 >= 0))   // both dots at once, one per f32x2 half
+    if (__any_sync(0xFFFFFFFFu, j1 >= 0))   // two accumulators side by side
         group_dot2_df<D>(ki, keys + s0 * D, keys + s1 * D, j1 >= 0, part, d0, d1);
     else
         d0 = group_dot_df<D>(ki, keys + s0 * D, part);
@@ -136,7 +139,7 @@ __global__ void __launch_bounds__(kRefineThreads, kMinBlocks * 256 / kRefineThre
 
 cudaError_t launch_refine(const uint16_t* keys, int U, int N, int d, const float4* norms,
                           const int* twin0, int* twin1, double* b0, double* b1,
-                          cudaStream_t st, bool beside_audit)
+                          cudaStream_t st, bool between_audits)
 {
     const dim3 grid((N + kRowsPerBlock - 1) / kRowsPerBlock, U);
     auto go = [&](auto kernel) {
@@ -144,9 +147,9 @@ cudaError_t launch_refine(const uint16_t* keys, int U, int N, int d, const float
                                 b0, b1);
     };
     if (d == 128)
-        return beside_audit ? go(refine_kernel<128, 6>)
+        return between_audits ? go(refine_kernel<128, 6>)
                             : twin1 ? go(refine_kernel<128, 4>) : go(refine_kernel<128, 5>);
-    return beside_audit ? go(refine_kernel<64, 6>)
+    return between_audits ? go(refine_kernel<64, 6>)
                         : twin1 ? go(refine_kernel<64, 4>) : go(refine_kernel<64, 5>);
 }
 
