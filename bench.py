@@ -470,7 +470,7 @@ def _report(args, w, ratio, world, U, N, d, ms, prof, e2e_ms, h2d, d2h, chunk, c
     print(json.dumps(line), flush=True)
 
 
-AUDIT_SOURCES = ("twk_audit.cu", "twk_ptx.cuh", "twk_internal.h")
+AUDIT_SOURCES = ("twk_audit.cu", "twk_bound.cuh", "twk_ptx.cuh", "twk_internal.h")
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "audit_kernel_traffic.txt")
 
 
